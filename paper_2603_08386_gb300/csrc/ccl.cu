@@ -13,6 +13,8 @@
 // each group becomes its union box, the survivors are compacted in root
 // order, and the round repeats until no pair is close. The result is sorted
 // by (y0, x0, y1, x1, n_px) by rank counting.
+#include <algorithm>
+
 #include "ddhf_internal.cuh"
 
 namespace ddhf {
@@ -370,66 +372,130 @@ ddhf_status launch_label(Ctx *c, const uint8_t *mask, int32_t *labels, uint64_t 
   return DDHF_OK;
 }
 
-// Dominant frequency of each box: block b scans the rows of box b; warp by
-// warp, a row's active pixels are the run of the (ascending) active list
-// between the keys y W + x0 and y W + x1, found by binary search. First pass:
-// each rotor pixel offers (SNR bits, -active index) to a maximum (the
-// strongest pixel) and is counted; then, when asked for, the lower median of
-// the rotor pixels' dominant bins by a two-digit radix selection (bins below
-// 2^14, 7 bits per pass, one more scan of the box per digit). A box without
-// rotor pixels gets bin -1, SNR 0 and median 0 Hz.
-__global__ void __launch_bounds__(256) k_box_f0(const uint32_t *__restrict__ active,
-                                                const uint64_t *__restrict__ counters,
-                                                const uint8_t *__restrict__ mask,
-                                                const float *__restrict__ snr,
-                                                const int32_t *__restrict__ f0,
-                                                const ddhf_box *__restrict__ boxes,
-                                                const int32_t *__restrict__ n_boxes, int32_t cap,
-                                                int W, int H, int32_t *f0_out, float *snr_out,
-                                                float *med_hz, int64_t g_a0, int64_t g_da,
-                                                int64_t g_denom, uint32_t *flags) {
-  __shared__ unsigned long long red[8];
-  __shared__ uint32_t cnt[8];
-  __shared__ uint32_t hist[128];
-  __shared__ uint32_t sel[2];
-  const int b = blockIdx.x;
-  const int nb = min(*n_boxes, cap);
-  if (b >= nb) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t n_act = (int64_t)counters[2];
-  const ddhf_box bx = boxes[b];
-  const int x0 = max(bx.x0, 0), x1 = min(bx.x1, W - 1);
-  const int y0 = max(bx.y0, 0), y1 = min(bx.y1, H - 1);
-  // fn(i) for every rotor pixel i (active index) inside the box
-  auto visit = [&](auto fn) {
-    for (int y = y0 + warp; y <= y1 && x0 <= x1; y += 8) {
-      const uint32_t lo = (uint32_t)((int64_t)y * W + x0), hi = (uint32_t)((int64_t)y * W + x1);
-      int64_t l = 0, r = n_act;  // first index with active[i] >= lo
-      while (l < r) {
-        const int64_t m = (l + r) >> 1;
-        if (active[m] < lo) l = m + 1;
-        else r = m;
-      }
-      for (int64_t i = l + lane;; i += 32) {
-        const bool in = i < n_act && active[i] <= hi;
-        if (in && mask[active[i]]) fn(i);
-        if (!__any_sync(0xffffffffu, in)) break;
-      }
+// Dominant frequency of each box, over every block of the grid whatever the
+// boxes' sizes (a crowded mask merges into one box that covers the sensor, and
+// one block per box took 9.65 ms on a 1280x720 box of 921,348 rotor pixels:
+// detection and frequencies of that window 15.06 ms, split as here 5.28 ms,
+// of a 347x261 window 0.80 -> 0.57 ms). A box is cut into units of kF0Unit pixels of
+// its rows (the work is one pass over the box's rotor pixels, bound by the
+// latency of its dependent loads, so a unit is small enough that every warp of
+// the grid gets one or two row segments); each unit offers its strongest pixel
+// (SNR bits, -active index) to the box's maximum and adds its rotor pixels'
+// dominant bins to the box's histogram, one counter per bin, and the box's
+// last unit reads the lower median off the histogram. The order of these
+// integer atomics does not matter.
+//
+// Per box in scratch (the label workspace, free after the boxes are out): the
+// maximum (2 words), rotor count, units done and N histogram counters.
+constexpr int kF0Unit = 4096;  // pixels of a box per unit
+constexpr int kF0Seg = 256;    // pixels of a row per warp step
+constexpr int kF0Head = 4;     // words of a box's record before its histogram
+constexpr int kF0SharedBins = 4096;  // up to this many bins a unit counts in shared memory
+
+struct BoxF0Args {
+  const uint32_t *active;
+  const uint64_t *counters;
+  const uint8_t *mask;
+  const float *snr;
+  const int32_t *f0;
+  const ddhf_box *boxes;
+  const int32_t *n_boxes;
+  int32_t cap, W, H, N;
+  int32_t room;          // boxes whose records fit the scratch
+  uint32_t *first_unit;  // [min(cap, room) + 1] first unit of each box
+  int32_t rec_words;     // words of a record: kF0Head + N, rounded up to even
+  uint32_t *rec;         // [room] records
+  int32_t *f0_out;
+  float *snr_out, *med_hz;
+  int64_t g_a0, g_da, g_denom;
+  uint32_t *flags;
+};
+
+struct BoxRows {
+  int x0, x1, y0, y1, nseg, items;  // clipped bounds, row segments, segments in all
+};
+__device__ __forceinline__ BoxRows box_rows(const BoxF0Args &A, const ddhf_box &b) {
+  BoxRows r;
+  r.x0 = max(b.x0, 0);
+  r.x1 = min(b.x1, A.W - 1);
+  r.y0 = max(b.y0, 0);
+  r.y1 = min(b.y1, A.H - 1);
+  r.nseg = r.x1 >= r.x0 ? (r.x1 - r.x0) / kF0Seg + 1 : 0;
+  r.items = r.y1 >= r.y0 ? (r.y1 - r.y0 + 1) * r.nseg : 0;
+  return r;
+}
+__device__ __forceinline__ uint32_t box_units(const BoxRows &r) {
+  const int64_t px = r.items > 0 ? (int64_t)(r.x1 - r.x0 + 1) * (r.y1 - r.y0 + 1) : 0;
+  return (uint32_t)max((int64_t)1, (px + kF0Unit - 1) / kF0Unit);
+}
+
+// First index i of the ascending active[0..n) with active[i] >= key, by the
+// whole warp: each step narrows the range to one of 32 parts.
+__device__ __forceinline__ int64_t warp_lower_bound(const uint32_t *active, int64_t n,
+                                                    uint32_t key) {
+  const int lane = threadIdx.x & 31;
+  int64_t l = 0, r = n;  // active[l - 1] < key <= active[r]
+  while (r - l > 32) {
+    const int64_t step = (r - l) / 32;
+    const int64_t m = l + (lane + 1) * step - 1;
+    const uint32_t lower = __popc(__ballot_sync(0xffffffffu, active[m] < key));
+    // the values ascend, so the lanes below `lower` are the ones under the key
+    if (lower < 32) r = l + (lower + 1) * step - 1;
+    l += lower * step;
+  }
+  const bool under = l + lane < r && active[l + lane] < key;
+  return l + __popc(__ballot_sync(0xffffffffu, under));
+}
+
+// Row segments first, first + step, ... of a box: fn(i) for every rotor pixel
+// i (active index) in them, warp by warp.
+template <typename F>
+__device__ __forceinline__ void box_visit(const BoxF0Args &A, const BoxRows &r, int64_t n_act,
+                                          int first, int step, int end, F fn) {
+  const int lane = threadIdx.x & 31;
+  for (int it = first; it < end; it += step) {
+    const int y = r.y0 + it / r.nseg, xs = r.x0 + (it % r.nseg) * kF0Seg;
+    const uint32_t lo = (uint32_t)((int64_t)y * A.W + xs);
+    const uint32_t hi = (uint32_t)((int64_t)y * A.W + min(r.x1, xs + kF0Seg - 1));
+    const int64_t l = warp_lower_bound(A.active, n_act, lo);
+    // at most kF0Seg active pixels lie in the segment
+    uint32_t key[kF0Seg / 32];
+#pragma unroll
+    for (int u = 0; u < kF0Seg / 32; ++u) {
+      const int64_t i = l + lane + 32 * u;
+      key[u] = i < n_act ? A.active[i] : 0xffffffffu;
     }
-  };
-  unsigned long long best = 0ull;
-  uint32_t n = 0;
-  visit([&](int64_t i) {
-    const unsigned long long v =
-        ((unsigned long long)__float_as_uint(snr[i]) << 32) | (0xffffffffu - (uint32_t)i);
-    best = v > best ? v : best;
-    ++n;
-  });
+#pragma unroll
+    for (int u = 0; u < kF0Seg / 32; ++u)
+      if (key[u] <= hi && A.mask[key[u]]) fn(l + lane + 32 * u);
+  }
+}
+
+__device__ __forceinline__ void box_f0_best(const BoxF0Args &A, int b, unsigned long long best) {
+  if (best == 0ull) {
+    A.f0_out[b] = -1;
+    if (A.snr_out) A.snr_out[b] = 0.f;
+  } else {
+    const uint32_t i = 0xffffffffu - (uint32_t)best;
+    A.f0_out[b] = A.f0[i];
+    if (A.snr_out) A.snr_out[b] = A.snr[i];
+  }
+}
+
+__device__ __forceinline__ float box_f0_hz(const BoxF0Args &A, uint32_t bin) {
+  return (float)((double)(A.g_a0 + (int64_t)bin * A.g_da) * 1e6 / (double)A.g_denom);
+}
+
+// Strongest pixel and rotor count of the block's warps.
+__device__ __forceinline__ void box_f0_reduce(unsigned long long &best, uint32_t &n,
+                                              unsigned long long *red, uint32_t *cnt) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long u = __shfl_xor_sync(0xffffffffu, best, o);
     best = u > best ? u : best;
     n += __shfl_xor_sync(0xffffffffu, n, o);
   }
+  __syncthreads();
   if (lane == 0) {
     red[warp] = best;
     cnt[warp] = n;
@@ -441,66 +507,224 @@ __global__ void __launch_bounds__(256) k_box_f0(const uint32_t *__restrict__ act
     best = red[w] > best ? red[w] : best;
     n += cnt[w];
   }
-  if (threadIdx.x == 0) {
-    if (best == 0ull) {
-      f0_out[b] = -1;
-      if (snr_out) snr_out[b] = 0.f;
-    } else {
-      const uint32_t i = 0xffffffffu - (uint32_t)best;
-      f0_out[b] = f0[i];
-      if (snr_out) snr_out[b] = snr[i];
+}
+
+// First units of the boxes and cleared records (block 0 the former); boxes
+// beyond the scratch's room (many boxes on a small sensor with a large grid)
+// are done here, one block each: strongest pixel, then the lower median by a
+// two-digit radix selection (bins below 2^14, 7 bits per pass).
+__global__ void __launch_bounds__(256) k_box_f0_plan(BoxF0Args A) {
+  __shared__ unsigned long long red[8];
+  __shared__ uint32_t cnt[8];
+  __shared__ uint32_t hist[128];
+  __shared__ uint32_t sel[2];
+  const int nb = min(*A.n_boxes, A.cap), nr = min(nb, A.room);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t words = (int64_t)max(nr, 0) * A.rec_words;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < words;
+       i += (int64_t)gridDim.x * blockDim.x)
+    A.rec[i] = 0;
+  if (blockIdx.x == 0) {
+    uint32_t base = 0;
+    for (int b0 = 0; b0 < nr; b0 += 256) {
+      const int b = b0 + threadIdx.x;
+      uint32_t inc = b < nr ? box_units(box_rows(A, A.boxes[b])) : 0u;
+      const uint32_t own = inc;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
+      }
+      if (lane == 31) cnt[warp] = inc;
+      __syncthreads();
+      uint32_t pre = base;
+      for (int w = 0; w < 8; ++w) {
+        if (w < warp) pre += cnt[w];
+        base += cnt[w];
+      }
+      if (b < nr) A.first_unit[b] = pre + inc - own;
+      __syncthreads();
     }
+    if (threadIdx.x == 0) A.first_unit[max(nr, 0)] = base;
   }
-  if (!med_hz) return;
-  if (n == 0) {
-    if (threadIdx.x == 0) med_hz[b] = 0.f;
-    return;
-  }
-  // lower median: the element of rank (n - 1) / 2 of the dominant bins
-  uint32_t rank = (n - 1) / 2, prefix = 0;
-  for (int pass = 0; pass < 2; ++pass) {
-    const int shift = pass == 0 ? 7 : 0;
-    for (int k = threadIdx.x; k < 128; k += blockDim.x) hist[k] = 0;
-    __syncthreads();
-    visit([&](int64_t i) {
-      const uint32_t v = (uint32_t)f0[i];
-      if (!ddhf_check(v < (1u << 14), flags)) return;
-      if (pass == 1 && (v >> 7) != prefix) return;
-      atomicAdd(&hist[(v >> shift) & 127u], 1u);
+  const int64_t n_act = (int64_t)A.counters[2];
+  for (int b = A.room + (int)blockIdx.x; b < nb; b += (int)gridDim.x) {
+    const BoxRows r = box_rows(A, A.boxes[b]);
+    unsigned long long best = 0ull;
+    uint32_t n = 0;
+    box_visit(A, r, n_act, warp, 8, r.items, [&](int64_t i) {
+      const unsigned long long v =
+          ((unsigned long long)__float_as_uint(A.snr[i]) << 32) | (0xffffffffu - (uint32_t)i);
+      best = v > best ? v : best;
+      ++n;
     });
-    __syncthreads();
+    box_f0_reduce(best, n, red, cnt);
+    if (threadIdx.x == 0) box_f0_best(A, b, best);
+    if (!A.med_hz) continue;
+    uint32_t rank = n > 0 ? (n - 1) / 2 : 0, prefix = 0;
+    for (int pass = 0; pass < 2 && n > 0; ++pass) {
+      const int shift = pass == 0 ? 7 : 0;
+      for (int k = threadIdx.x; k < 128; k += blockDim.x) hist[k] = 0;
+      __syncthreads();
+      box_visit(A, r, n_act, warp, 8, r.items, [&](int64_t i) {
+        const uint32_t v = (uint32_t)A.f0[i];
+        if (!ddhf_check(v < (1u << 14), A.flags)) return;
+        if (pass == 1 && (v >> 7) != prefix) return;
+        atomicAdd(&hist[(v >> shift) & 127u], 1u);
+      });
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        uint32_t run = 0;
+        int dsel = 127;
+        for (int k = 0; k < 128; ++k) {
+          if (rank < run + hist[k]) {
+            dsel = k;
+            break;
+          }
+          run += hist[k];
+        }
+        sel[0] = (uint32_t)dsel;
+        sel[1] = rank - run;
+      }
+      __syncthreads();
+      prefix = pass == 0 ? sel[0] : (prefix << 7) | sel[0];
+      rank = sel[1];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) A.med_hz[b] = n > 0 ? box_f0_hz(A, prefix) : 0.f;
+  }
+}
+
+// The units of the boxes that have a record, and each box's results by its
+// last unit. SHARED: a unit counts its bins in shared memory first.
+template <bool SHARED>
+__global__ void __launch_bounds__(256) k_box_f0_units(BoxF0Args A) {
+  extern __shared__ uint32_t sh_hist[];
+  __shared__ unsigned long long red[8];
+  __shared__ uint32_t cnt[8];
+  __shared__ uint32_t s_last;
+  const int nr = min(min(*A.n_boxes, A.cap), A.room);
+  if (nr <= 0) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t n_act = (int64_t)A.counters[2];
+  const uint32_t n_units = A.first_unit[nr];
+  const bool want_med = A.med_hz != nullptr;
+  for (uint32_t u = blockIdx.x; u < n_units; u += gridDim.x) {
+    int lo = 0, hi = nr - 1;  // the box of unit u
+    while (lo < hi) {
+      const int m = (lo + hi + 1) >> 1;
+      if (A.first_unit[m] <= u) lo = m;
+      else hi = m - 1;
+    }
+    const int b = lo;
+    const uint32_t part = u - A.first_unit[b], parts = A.first_unit[b + 1] - A.first_unit[b];
+    const BoxRows r = box_rows(A, A.boxes[b]);
+    uint32_t *rec = A.rec + (int64_t)b * A.rec_words, *hist = rec + kF0Head;
+    if (SHARED && want_med) {
+      for (int k = threadIdx.x; k < A.N; k += blockDim.x) sh_hist[k] = 0;
+      __syncthreads();
+    }
+    const int i0 = (int)((int64_t)r.items * part / parts);
+    const int i1 = (int)((int64_t)r.items * (part + 1) / parts);
+    unsigned long long best = 0ull;
+    uint32_t n = 0;
+    box_visit(A, r, n_act, i0 + warp, 8, i1, [&](int64_t i) {
+      const unsigned long long v =
+          ((unsigned long long)__float_as_uint(A.snr[i]) << 32) | (0xffffffffu - (uint32_t)i);
+      best = v > best ? v : best;
+      ++n;
+      if (!want_med) return;
+      const uint32_t f = min((uint32_t)A.f0[i], (uint32_t)A.N - 1);  // always below N
+      atomicAdd(SHARED ? &sh_hist[f] : &hist[f], 1u);
+    });
+    box_f0_reduce(best, n, red, cnt);  // its barriers also end the shared counting
+    if (SHARED && want_med)
+      for (int k = threadIdx.x; k < A.N; k += blockDim.x)
+        if (sh_hist[k]) atomicAdd(&hist[k], sh_hist[k]);
     if (threadIdx.x == 0) {
-      uint32_t run = 0;
-      int dsel = 127;
-      for (int k = 0; k < 128; ++k) {
-        if (rank < run + hist[k]) {
-          dsel = k;
+      if (best) atomicMax(reinterpret_cast<unsigned long long *>(rec), best);
+      if (n) atomicAdd(&rec[2], n);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&rec[3], 1u) == parts - 1;
+    __syncthreads();
+    if (!s_last) continue;
+    __threadfence();
+    if (threadIdx.x == 0)
+      box_f0_best(A, b, __ldcg(reinterpret_cast<const unsigned long long *>(rec)));
+    if (!want_med) continue;
+    const uint32_t total = __ldcg(&rec[2]);
+    // lower median: the bin that holds rank (total - 1) / 2
+    const uint32_t rank = total > 0 ? (total - 1) / 2 : 0;
+    const int per = (A.N + 255) / 256, k0 = (int)threadIdx.x * per, k1 = min(A.N, k0 + per);
+    uint32_t own = 0;
+    for (int k = k0; k < k1; ++k) own += __ldcg(&hist[k]);
+    uint32_t inc = own;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) cnt[warp] = inc;
+    __syncthreads();
+    uint32_t pre = inc - own;
+    for (int w = 0; w < warp; ++w) pre += cnt[w];
+    if (total == 0) {
+      if (threadIdx.x == 0) A.med_hz[b] = 0.f;
+    } else if (rank >= pre && rank < pre + own) {
+      uint32_t run = pre;
+      for (int k = k0; k < k1; ++k) {
+        const uint32_t h = __ldcg(&hist[k]);
+        if (rank < run + h) {
+          A.med_hz[b] = box_f0_hz(A, (uint32_t)k);
           break;
         }
-        run += hist[k];
+        run += h;
       }
-      sel[0] = (uint32_t)dsel;
-      sel[1] = rank - run;
     }
     __syncthreads();
-    if (pass == 0) prefix = sel[0];
-    else prefix = (prefix << 7) | sel[0];
-    rank = sel[1];
-    __syncthreads();
   }
-  if (threadIdx.x == 0)
-    med_hz[b] = (float)((double)(g_a0 + (int64_t)prefix * g_da) * 1e6 / (double)g_denom);
 }
 
 ddhf_status launch_box_f0(Ctx *c, int slot, const ddhf_box *boxes, const int32_t *n_boxes,
                           int32_t cap, int32_t *f0_out, float *snr_out, float *med_hz,
                           cudaStream_t s) {
   const Slot &sl = c->slots[slot];
+  if (cap <= 0) return DDHF_OK;
+  BoxF0Args A{};
+  A.active = sl.active;
+  A.counters = sl.counters;
+  A.mask = sl.mask;
+  A.snr = sl.snr;
+  A.f0 = sl.f0;
+  A.boxes = boxes;
+  A.n_boxes = n_boxes;
+  A.cap = cap;
+  A.W = c->W;
+  A.H = c->H;
+  A.N = c->grid.n_bins;
+  // records (8-byte aligned, of an even number of words) in the box workspace
+  // of 15 npx words, after a word of first_unit each and one more
+  A.rec_words = (kF0Head + A.N + 1) & ~1;
+  const int64_t words = 15 * c->npx;
+  A.room = (int32_t)std::min<int64_t>(cap, std::max<int64_t>(0, (words - 4) / (A.rec_words + 1)));
+  A.first_unit = reinterpret_cast<uint32_t *>(c->box_tmp);
+  A.rec = A.first_unit + ((A.room + 1 + 1) & ~1);
+  A.f0_out = f0_out;
+  A.snr_out = snr_out;
+  A.med_hz = med_hz;
   // bin j at (a0 + j da) / denom cycles per microsecond
-  if (cap > 0)
-    k_box_f0<<<cap, 256, 0, s>>>(sl.active, sl.counters, sl.mask, sl.snr, sl.f0, boxes, n_boxes,
-                                 cap, c->W, c->H, f0_out, snr_out, med_hz, c->grid.a0, c->grid.da,
-                                 c->grid.denom, c->flags);
+  A.g_a0 = c->grid.a0;
+  A.g_da = c->grid.da;
+  A.g_denom = c->grid.denom;
+  A.flags = c->flags;
+  k_box_f0_plan<<<c->num_sms, 256, 0, s>>>(A);
+  if (A.room > 0) {
+    const unsigned units = (unsigned)c->num_sms * 4;
+    if (A.N <= kF0SharedBins)
+      k_box_f0_units<true><<<units, 256, A.N * sizeof(uint32_t), s>>>(A);
+    else
+      k_box_f0_units<false><<<units, 256, 0, s>>>(A);
+  }
   DDHF_CUDA_TRY(c, cudaGetLastError());
   return DDHF_OK;
 }
