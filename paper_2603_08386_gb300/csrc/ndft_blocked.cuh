@@ -1,28 +1,54 @@
-// Per-pixel non-uniform DFT power (Sec. 3.3 Eq. 6, P_k = |F_k|^2), the
-// comb-scoring kernel (Eq. 7-11) and the fused persistent kernel.
+// Per-pixel non-uniform DFT power (Sec. 3.3 Eq. 6, P_k = |F_k|^2) on the tensor
+// cores: the persistent kernel of DDHF_FORM_BLOCKED, writing spectra or (fused)
+// scoring them where they are (Eq. 7-11, comb.cuh).
 //
-// Phases are exact: the phase of event tau at bin j is the integer residue
-// r = (a_j * tau) mod D in units of 1/D cycles (64-bit products, Barrett
-// reduction), and only that residue is converted to floating point.
+// Bins j = 32 b + r. With the centre frequency of row b, a_c(b) = a0 + (32 b +
+// 15.5) da, and s = r - 15.5 = +-(k + 1/2), k = 0..15,
+//   F[32 b + r] = sum_e A_b(e) u_s(e),  A_b = p e^{-2 pi i a_c(b) tau / D},
+//                                       u_s = e^{-2 pi i s da tau / D} = c_k -+ i d_k,
+// and the sums over the events e of the four real products of (Re A, Im A) with
+// (c_k, d_k) give both bins +-s:
+//   F[+s] = (X1 - X2) + i (X3 + X4),  F[-s] = (X1 + X2) + i (X3 - X4),
+//   X1 = sum Ar c, X2 = sum Ai d, X3 = sum Ai c, X4 = sum Ar d:
+// two real multiply-adds per event and bin (a complex product needs three or
+// four), as one real matrix product per pixel, [Ar; Ai] (2 rows per b) x events
+// x [c d] (32 columns).
 //
-// Forms (see DDHF_FORM_* in ddhf.h):
-//   plain kernels   one warp per active pixel, lane l owns bins l + 32m; the
-//                   events are broadcast by warp shuffles; the residue is
-//                   advanced from bin to bin by an exact modular step.
-//   BLOCKED         bins j = 32b + r. With A[b][k] = p_k e^{-2 pi i a_{32b}
-//                   tau_k / D} and B[k][r] = u_k^r, u_k = e^{-2 pi i da tau_k
-//                   / D}, F[32b + r] = sum_k A[b][k] B[k][r]: a complex matrix
-//                   product per pixel whose factors are generated from two
-//                   exact seeds per event (A rows by the step u_k^32, B by
-//                   u_k). The product is accumulated with three real
-//                   multiplications per term (T1 = sum Ar Br, T2 = sum Ai Bi,
-//                   T3 = sum (Ar+Ai)(Br+Bi); Re F = T1 - T2, Im F = T3 - T1
-//                   - T2). Lanes hold a TB x 4 tile of (b, r) accumulators,
-//                   updated by paired FMAs; events are generated 16 at a time
-//                   into shared memory, two lanes per event. Light pixels take one warp,
-//                   heavy pixels a whole block (events split over warps,
-//                   partial sums reduced in a fixed order), heavy first.
+// The product runs on the tensor cores in FP32 accuracy: each factor x is split
+// into two FP16 words, x = hi + lo + O(2^-22) (|x| <= 1, so the error is absolute
+// and below the factor's own FP32 generation error), and one m16n8k16
+// instruction takes 8 events as 16 K entries (hi and lo of A side by side), once
+// against hi of B and once against lo: all four partial products, accumulated
+// in FP32. A pixel's product is too small and its operands too private for
+// tcgen05 (48 x 32 x a few tens of events, every pixel with operands of its own,
+// so each 64-row tcgen05 step would read as many shared-memory bytes as it has
+// multiply-adds to do): mma.sync takes its operands from registers and leaves
+// every accumulator of a bin pair in the lane that squares it.
+//
+// Factors are generated for 32 events at a time, one lane per event, into shared
+// memory: a column and a row phasor from exact phases, the others by rotation
+// away from them on both sides (at most 8 steps for the columns, 4 MT for the
+// rows, each step an exact phasor too). Phases are 64-bit fixed-point fractions
+// of a turn: the frequency's fraction a / D mod 1, rounded to 2^-64, times tau,
+// so the phase error is below 2^-33 of a turn. Measured error of the spectra
+// against FP64 (2-norm over all pixels): 2.4e-7 at 2000 bins on 640x480 pixels,
+// 4.0e-7 at 10,000 bins on 320x180 (the FP32 three-multiplication product
+// before it, with its longer rotation chains: 8.1e-7 and 1.3e-6).
+//
+// Measured (one 1280x720 window of 19.9M events, 750 bins, default tuning):
+// 2.58 -> 1.55 ms (FMA pipe -> issue 65 %, tensor pipe 32 %, 1,227 warp
+// instructions per pixel); 640x480 at 2000 bins 1.79 -> 0.99 ms.
+//
+// Bins whose frequency is a multiple of D (in practice bin 0 of a grid that
+// starts at 0 Hz) have the phase 0 for every event: their power is the squared
+// integer sum of the polarities, counted exactly (Eq. 7 takes the logarithm of
+// it, and a sum of zero must be exactly zero).
+//
+// Light pixels take one warp, heavy pixels a whole block (events split over
+// warps, partial sums reduced in a fixed order), heavy first.
 #pragma once
+
+#include <algorithm>
 
 #include "comb.cuh"
 #include "ddhf_internal.cuh"
@@ -30,203 +56,255 @@
 namespace ddhf {
 namespace blocked {
 
-constexpr int kGenChunk = 16;
+constexpr int kGenChunk = 32;  // events staged per warp, one lane each
+constexpr int kGroup = 8;      // events per tensor-core step
+constexpr int kMaxPasses = 64; // 512 rows of 32 bins, at least 8 per pass
 
-// (a of bin 32 b) mod D = (a0 + 32 b da) mod D, for b < 2^11 (the operand of
-// the reduction stays below 2^43).
-__device__ __forceinline__ uint64_t arow_residue(const GridConst &g, int b) {
-  return mod_barrett(g.a0_mod + (uint64_t)b * g.da32_mod, g.denom, g.barrett);
+// Phases as fractions of a turn in units of 2^-64.
+struct NdftConst {
+  uint64_t f_u;                // da / D (one bin)
+  uint64_t f_k8;               // 8.5 da / D (column k = 8)
+  uint64_t f_v;                // 32 da / D (one row)
+  uint64_t f_row[kMaxPasses];  // a_c(b0 + 4 MT) / D: the middle row of each pass
+  int32_t dc_first, dc_step;   // bins with a_j = 0 mod D: dc_first + i dc_step (-1: none)
+};
+
+inline uint64_t turn_fraction(unsigned __int128 num, uint64_t den) {
+  const uint64_t r = (uint64_t)(num % den);
+  return (uint64_t)((((unsigned __int128)r << 64) + den / 2) / den);
+}
+
+inline NdftConst make_ndft_const(const GridConst &g, int mt) {
+  NdftConst n{};
+  const unsigned __int128 a0 = g.a0, da = g.da;
+  n.f_u = turn_fraction(da, g.denom);
+  n.f_k8 = turn_fraction(17 * da, 2 * g.denom);
+  n.f_v = turn_fraction(32 * da, g.denom);
+  for (int i = 0; i < kMaxPasses; ++i)
+    n.f_row[i] = turn_fraction(2 * a0 + (64 * (unsigned)(8 * mt * i + 4 * mt) + 31) * da,
+                               2 * g.denom);
+  n.dc_first = -1;
+  uint64_t x = g.da, y = g.denom;
+  while (y) {
+    const uint64_t r = x % y;
+    x = y;
+    y = r;
+  }
+  n.dc_step = (int32_t)std::min<uint64_t>(g.denom / x, (uint64_t)1 << 30);
+  for (int j = 0; j < g.N && j < n.dc_step; ++j)
+    if ((g.a0 + (uint64_t)j * g.da) % g.denom == 0) {
+      n.dc_first = j;
+      break;
+    }
+  return n;
 }
 
 __device__ __forceinline__ void raise_flag(uint32_t *flags, uint32_t f) { atomicOr(flags, f); }
 
-// ---------------------------------------------------------------- blocked
+// e^{-2 pi i phi}, phi = f tau as a fraction of a turn (f in units of 2^-64).
+// The turn's top 32 bits are split into the nearest quarter turn and a signed
+// remainder of at most 1/8 turn, which converts to FP32 with an absolute error
+// below 2^-28 of a turn.
+__device__ __forceinline__ float2 phasor_of_turn(uint64_t f, uint32_t tau) {
+  const uint32_t turn = __umulhi((uint32_t)f, tau) + (uint32_t)(f >> 32) * tau;
+  const uint32_t q = (turn + 0x20000000u) >> 30;
+  const int32_t rem = (int32_t)(turn - (q << 30));
+  float sy, cy;
+  sincospi_reduced(__fmul_rn((float)rem, 0x1p-31f), sy, cy);
+  const float a = (q & 1u) ? sy : cy, b = (q & 1u) ? cy : sy;
+  return make_float2(__uint_as_float(__float_as_uint(a) ^ (((q + 1u) & 2u) << 30)),
+                     __uint_as_float(__float_as_uint(b) ^ (((q & 2u) ^ 2u) << 30)));
+}
 
-// Bank-conflict-free row stride (float4 units) of one lane group's A rows.
-template <int TB>
-struct ALayout {
-  static constexpr int kGroup = (TB % 4 == 0) ? TB + 1 : TB;  // stride between lane groups
-  static constexpr int kEvent = 4 * kGroup + 1;               // stride between events
+// x = hi + lo as two FP16 values, hi in the low half: hi is x cut to 11
+// significant bits, lo the rest rounded to FP16.
+__device__ __forceinline__ uint32_t split_half2(float x) {
+  const float hi = __uint_as_float(__float_as_uint(x) & 0xffffe000u);
+  const float lo = __fsub_rn(x, hi);
+  uint32_t w;
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(lo), "f"(hi));
+  return w;
+}
+
+// Shared-memory layout of one warp's staged factors, per event: B (32 columns)
+// as eight 16-byte units of four words, A as one such array per two m-tiles and
+// an array of eight 8-byte units for an odd one (MT m-tiles of 8 rows; the words
+// of lane group g belong to rows MT g .. MT g + MT - 1, Re and Im). Events are
+// nine units apart and the units permuted, so that neither the generating
+// lanes (one event each) nor the multiplying ones (lane (g, t): unit g of
+// events t and t + 4) meet a bank twice (8-byte units: one extra wavefront).
+template <int MT>
+struct Stage {
+  static constexpr int kPairs = MT / 2;                 // 16-byte A arrays
+  static constexpr int kB = 0;                          // bytes
+  static constexpr int kA = 144 * kGenChunk;
+  static constexpr int kArray = 144 * kGenChunk;        // per 16-byte array
+  static constexpr int kA64 = kA + kPairs * kArray;
+  static constexpr int kBytes = kA64 + (MT & 1) * 72 * kGenChunk;
 };
-constexpr int kBEvent = 25;  // float4 per event of B: [8 rg][3 comps] + 1 pad
+__device__ __forceinline__ int unit16(int g) { return (g >> 1) + 4 * (g & 1); }
+__device__ __forceinline__ int unit8(int g) {
+  return ((g >> 2) << 1) + ((g & 1) << 2) + ((g >> 1) & 1);
+}
 
-template <int TB>
-struct WarpLayout {
-  // float4 offsets within a warp's staging area
-  static constexpr int kB = 0;
-  static constexpr int kA = kGenChunk * kBEvent;
-  static constexpr int kStageF4 = kA + kGenChunk * ALayout<TB>::kEvent;
-};
-
-// Generate the A and B factors of the events of one chunk; w is the event
-// word of event e = lane % 16, active when e < the chunk's event count. Two
-// lanes per event run the same code: lane e (half 0) writes B columns
-// r = 0..15 and A rows 0..2TB-1, lane e + 16 (half 1) B columns 16..31 and A
-// rows 2TB..4TB-1. The step phasors u = e^{-2 pi i da tau / D} (columns) and
-// v = u^32 (rows) and each lane's first A row come from exact seeds
-// (residues); half 1's first column u^16 is u squared four times (one exact
-// seed fewer; its error stays near that of the 16 chain steps it replaces).
-// Each lane steps in two interleaved chains.
-// arow_mod[h]: (a of the first A row of half h) mod D.
-template <int TB>
-__device__ __forceinline__ void gen_chunk(uint32_t w, bool active, const GridConst &g,
-                                          const uint64_t (&arow_mod)[2], float4 *stage) {
-  const int lane = threadIdx.x & 31;
-  const int e = lane & 15, half = lane >> 4;
-  const uint64_t tau = w & 0x7fffffffu;
-  // the two lanes of an event make one step phasor each (half 0: u, half 1:
-  // v = u^32) and swap them; each makes its own first A row, and half 1 its
-  // first B column u^16 (half 0 starts at u^0 = 1)
-  const uint64_t ra = mod_barrett((half ? g.da32_mod : g.da_mod) * tau, g.denom, g.barrett);
-  const uint64_t rs = mod_barrett(arow_mod[half] * tau, g.denom, g.barrett);
-  const float2 pa = phasor_of_residue(ra, g.two_over_denom);
-  const float2 pb = make_float2(__shfl_xor_sync(0xffffffffu, pa.x, 16),
-                                __shfl_xor_sync(0xffffffffu, pa.y, 16));
-  if (!active) return;
-  const float2 u = half ? pb : pa;
-  const float2 v = half ? pa : pb;
-  float2 s = phasor_of_residue(rs, g.two_over_denom);
-  const float2 q2 = cmul(u, u), q4 = cmul(q2, q2), q8 = cmul(q4, q4), q16 = cmul(q8, q8);
-  float2 z = half ? q16 : make_float2(1.f, 0.f);
-  if (w & kSignBit) {
-    s.x = -s.x;
-    s.y = -s.y;
-  }
-  // columns: two interleaved chains (even and odd r) stepped by u^2
-  const float2 u2 = cmul(u, u);
-  float2 za = z, zb = cmul(z, u);
-  float4 *dstb = stage + WarpLayout<TB>::kB + e * kBEvent + half * 4 * 3;
+// The factors of event word w (lane = event of the chunk) into the warp's
+// staging area. Every lane writes, so that no slot holds anything but finite
+// factors (a lane past the last event generates those of word 0).
+template <int MT>
+__device__ __forceinline__ void gen_chunk(uint32_t w, const NdftConst &nd, uint64_t f_row,
+                                          unsigned char *stage) {
+  const int e = threadIdx.x & 31;
+  const uint32_t tau = w & 0x7fffffffu, sg = w & kSignBit;
+  const float2 u = phasor_of_turn(nd.f_u, tau);
+  const float2 uc = make_float2(u.x, -u.y);
+  // columns: k = 8 exact, 9..15 and 7..0 by rotation
+  {
+    float2 up = phasor_of_turn(nd.f_k8, tau), dn = up;
+    uint4 *b = reinterpret_cast<uint4 *>(stage + Stage<MT>::kB + e * 144);
 #pragma unroll
-  for (int rg = 0; rg < 4; ++rg) {
-    const float2 zc = cmul(za, u2), zd = cmul(zb, u2);
-    const float br[4] = {za.x, zb.x, zc.x, zd.x};
-    const float bi[4] = {za.y, zb.y, zc.y, zd.y};
-    if (rg < 3) {
-      za = cmul(zc, u2);
-      zb = cmul(zd, u2);
+    for (int h = 0; h < 2; ++h) {
+      uint32_t c[4], d[4], c2[4], d2[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (h + i > 0) up = cmul(up, u);
+        c[i] = split_half2(up.x);  // k = 8 + 4 h + i
+        d[i] = split_half2(up.y);
+        dn = cmul(dn, uc);
+        c2[3 - i] = split_half2(dn.x);  // k = 7 - 4 h - i
+        d2[3 - i] = split_half2(dn.y);
+      }
+      b[2 + h] = make_uint4(c[0], c[1], c[2], c[3]);
+      b[6 + h] = make_uint4(d[0], d[1], d[2], d[3]);
+      b[1 - h] = make_uint4(c2[0], c2[1], c2[2], c2[3]);
+      b[5 - h] = make_uint4(d2[0], d2[1], d2[2], d2[3]);
     }
-    dstb[rg * 3 + 0] = make_float4(br[0], bi[0], br[1], bi[1]);
-    dstb[rg * 3 + 1] = make_float4(br[2], bi[2], br[3], bi[3]);
-    dstb[rg * 3 + 2] = make_float4(__fadd_rn(br[0], bi[0]), __fadd_rn(br[1], bi[1]),
-                                   __fadd_rn(br[2], bi[2]), __fadd_rn(br[3], bi[3]));
   }
-  // rows: two interleaved chains (even and odd row) stepped by v^2
-  const float2 v2 = cmul(v, v);
-  float2 sa = s, sb = cmul(s, v);
-  float4 *dsta = stage + WarpLayout<TB>::kA + e * ALayout<TB>::kEvent +
-                 half * 2 * ALayout<TB>::kGroup;
+  // rows: 4 MT exact (the polarity's sign on it), the others by rotation
+  {
+    const float2 v = phasor_of_turn(nd.f_v, tau);
+    const float2 vc = make_float2(v.x, -v.y);
+    float2 up = phasor_of_turn(f_row, tau);
+    up.x = __uint_as_float(__float_as_uint(up.x) ^ sg);
+    up.y = __uint_as_float(__float_as_uint(up.y) ^ sg);
+    float2 dn = up;
 #pragma unroll
-  for (int k = 0; k < 2 * TB; k += 2) {
-    const float ssa = __fadd_rn(sa.x, sa.y), ssb = __fadd_rn(sb.x, sb.y);
-    dsta[(k / TB) * ALayout<TB>::kGroup + k % TB] = make_float4(sa.x, sa.y, ssa, ssa);
-    dsta[((k + 1) / TB) * ALayout<TB>::kGroup + (k + 1) % TB] = make_float4(sb.x, sb.y, ssb, ssb);
-    if (k + 2 < 2 * TB) {
-      sa = cmul(sa, v2);
-      sb = cmul(sb, v2);
+    for (int h = 0; h < 4; ++h) {
+      uint32_t r[2 * MT], r2[2 * MT];
+#pragma unroll
+      for (int i = 0; i < MT; ++i) {
+        if (h + i > 0) up = cmul(up, v);
+        r[2 * i] = split_half2(up.x);  // row MT (4 + h) + i
+        r[2 * i + 1] = split_half2(up.y);
+        dn = cmul(dn, vc);
+        r2[2 * (MT - 1 - i)] = split_half2(dn.x);  // row MT (3 - h) + MT - 1 - i
+        r2[2 * (MT - 1 - i) + 1] = split_half2(dn.y);
+      }
+      const int gu = 4 + h, gd = 3 - h;
+#pragma unroll
+      for (int p = 0; p < Stage<MT>::kPairs; ++p) {
+        uint4 *a = reinterpret_cast<uint4 *>(stage + Stage<MT>::kA + p * Stage<MT>::kArray +
+                                             e * 144);
+        a[unit16(gu)] = make_uint4(r[4 * p], r[4 * p + 1], r[4 * p + 2], r[4 * p + 3]);
+        a[unit16(gd)] = make_uint4(r2[4 * p], r2[4 * p + 1], r2[4 * p + 2], r2[4 * p + 3]);
+      }
+      if (MT & 1) {
+        uint2 *a = reinterpret_cast<uint2 *>(stage + Stage<MT>::kA64 + e * 72);
+        a[unit8(gu)] = make_uint2(r[2 * MT - 2], r[2 * MT - 1]);
+        a[unit8(gd)] = make_uint2(r2[2 * MT - 2], r2[2 * MT - 1]);
+      }
     }
   }
 }
 
-// Accumulators of a lane's TB x 4 tile, in float2 pairs so that one paired
-// FMA (FFMA2, each element rounded on its own) updates two of them:
-// t12[i][q] = (T1, T2) of bin (i, q), t3[i][h] = (T3 of bin (i, 2h), of (i, 2h+1)).
-// Shared-memory operands come in matching pairs: A rows as (Ar, Ai, Ar+Ai,
-// Ar+Ai), B columns as (Br0, Bi0, Br1, Bi1), (Br2, Bi2, Br3, Bi3),
-// (Br0+Bi0, .., Br3+Bi3).
-template <int TB>
+// A lane's accumulators: x[i][q] = (X1, X4, X3, X2) of row MT g + i and column
+// pair k = 4 t + q (lane (g, t) = (lane / 4, lane % 4)): the C fragment of an
+// m16n8k16 step whose rows g and g + 8 are Re and Im of A and whose columns 2 t
+// and 2 t + 1 are c and d.
+template <int MT>
 struct Acc {
-  float2 t12[TB][4], t3[TB][2];
+  float x[MT][4][4];
   __device__ __forceinline__ void zero() {
 #pragma unroll
-    for (int i = 0; i < TB; ++i) {
+    for (int i = 0; i < MT; ++i)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) t12[i][q] = make_float2(0.f, 0.f);
-      t3[i][0] = t3[i][1] = make_float2(0.f, 0.f);
-    }
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) x[i][q][c] = 0.f;
   }
-  // component c (0: T1, 1: T2, 2: T3) of bin (i, q)
-  __device__ __forceinline__ float &at(int c, int i, int q) {
-    if (c == 0) return t12[i][q].x;
-    if (c == 1) return t12[i][q].y;
-    return (q & 1) ? t3[i][q >> 1].y : t3[i][q >> 1].x;
-  }
-  __device__ __forceinline__ float get(int c, int i, int q) const {
-    if (c == 0) return t12[i][q].x;
-    if (c == 1) return t12[i][q].y;
-    return (q & 1) ? t3[i][q >> 1].y : t3[i][q >> 1].x;
+  // Powers of the bins at +s (k = 4 t + q) and -s of row i.
+  __device__ __forceinline__ void powers(int i, int q, float &pp, float &pm) const {
+    const float *a = x[i][q];
+    const float rp = __fsub_rn(a[0], a[3]), ip = __fadd_rn(a[2], a[1]);
+    const float rm = __fadd_rn(a[0], a[3]), im = __fsub_rn(a[2], a[1]);
+    pp = __fmaf_rn(rp, rp, __fmul_rn(ip, ip));
+    pm = __fmaf_rn(rm, rm, __fmul_rn(im, im));
   }
 };
 
-// Events [e_lo, e_hi) of the staged chunk into the lane's tile.
-template <int TB>
-__device__ __forceinline__ void gemm_range(int e_lo, int e_hi, const float4 *stage, Acc<TB> &acc) {
-  const int lane = threadIdx.x & 31;
-  const int bg = lane >> 3, rg = lane & 7;
-  const float4 *sb = stage + WarpLayout<TB>::kB + rg * 3;
-  const float4 *sa = stage + WarpLayout<TB>::kA + bg * ALayout<TB>::kGroup;
-  for (int e = e_lo; e < e_hi; ++e) {
-    const float4 b01 = sb[e * kBEvent + 0];
-    const float4 b23 = sb[e * kBEvent + 1];
-    const float4 bs = sb[e * kBEvent + 2];
-    const float2 bri[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
-                           make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
-    const float2 bss[2] = {make_float2(bs.x, bs.y), make_float2(bs.z, bs.w)};
+// d = A B + c, an m16n8k16 step.
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                         uint32_t b1, const float (&c)[4]) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%10,%11,%12,%13};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c[0]), "f"(c[1]),
+        "f"(c[2]), "f"(c[3]));
+}
+
+// Staged events q .. q + m - 1 (m <= 8, q + m <= 32) into the accumulators. A
+// pixel's events enter in groups of 8 counted from its first one, whatever the
+// chunk they were staged in, so its sums do not depend on how the work is split.
+template <int MT>
+__device__ __forceinline__ void mma_group(int q, int m, const unsigned char *stage, Acc<MT> &acc) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int e0 = min(q + t, kGenChunk - 1), e1 = min(q + t + 4, kGenChunk - 1);
+  const unsigned char *sb = stage + Stage<MT>::kB + 16 * unit16(g);
+  uint4 b0 = *reinterpret_cast<const uint4 *>(sb + e0 * 144);
+  uint4 b1 = *reinterpret_cast<const uint4 *>(sb + e1 * 144);
+  uint32_t a[MT][4];
 #pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const float4 a = sa[e * ALayout<TB>::kEvent + i];
-      const float2 axy = make_float2(a.x, a.y), ass = make_float2(a.z, a.w);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc.t12[i][q] = __ffma2_rn(axy, bri[q], acc.t12[i][q]);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) acc.t3[i][h] = __ffma2_rn(ass, bss[h], acc.t3[i][h]);
-    }
+  for (int p = 0; p < Stage<MT>::kPairs; ++p) {
+    const unsigned char *sa = stage + Stage<MT>::kA + p * Stage<MT>::kArray + 16 * unit16(g);
+    const uint4 x = *reinterpret_cast<const uint4 *>(sa + e0 * 144);
+    const uint4 y = *reinterpret_cast<const uint4 *>(sa + e1 * 144);
+    a[2 * p][0] = x.x, a[2 * p][1] = x.y, a[2 * p][2] = y.x, a[2 * p][3] = y.y;
+    a[2 * p + 1][0] = x.z, a[2 * p + 1][1] = x.w, a[2 * p + 1][2] = y.z, a[2 * p + 1][3] = y.w;
   }
-}
-
-template <int TB>
-__device__ __forceinline__ void gemm_chunk(int ne, const float4 *stage, Acc<TB> &acc) {
-  gemm_range<TB>(0, ne, stage, acc);
-}
-
-// Accumulate events [e_begin, e_end) of a pixel in steps of `estep` chunks
-// (warp w of a block takes chunks w, w + nw, ...).
-template <int TB>
-__device__ __forceinline__ void accumulate(const uint32_t *__restrict__ evp, int cnt, int chunk0,
-                                           int chunk_step, const GridConst &g,
-                                           const uint64_t (&arow_mod)[2],
-                                           float4 *stage, Acc<TB> &acc) {
-  const int e = threadIdx.x & 15;
-  const int step = chunk_step * kGenChunk;
-  int c0 = chunk0 * kGenChunk;
-  uint32_t w = c0 + e < cnt ? evp[c0 + e] : 0u;
-  for (; c0 < cnt; c0 += step) {
-    const int ne = min(kGenChunk, cnt - c0);
-    gen_chunk<TB>(w, e < ne, g, arow_mod, stage);
-    __syncwarp();
-    const int c1 = c0 + step;  // the next chunk's event word, loaded ahead
-    w = c1 + e < cnt ? evp[c1 + e] : 0u;
-    gemm_chunk<TB>(ne, stage, acc);
-    __syncwarp();
+  if (MT & 1) {
+    const unsigned char *sa = stage + Stage<MT>::kA64 + 8 * unit8(g);
+    const uint2 x = *reinterpret_cast<const uint2 *>(sa + e0 * 72);
+    const uint2 y = *reinterpret_cast<const uint2 *>(sa + e1 * 72);
+    a[MT - 1][0] = x.x, a[MT - 1][1] = x.y, a[MT - 1][2] = y.x, a[MT - 1][3] = y.y;
   }
-}
-
-// Power of the lane's tile into Pw (row-major bins, float4 per lane row).
-template <int TB>
-__device__ __forceinline__ void finalize_tile(const Acc<TB> &acc, float *Pw, int row_base) {
-  const int lane = threadIdx.x & 31;
-  const int bg = lane >> 3, rg = lane & 7;
+  if (m < kGroup) {  // past the pixel's last event
+    if (t >= m) b0 = make_uint4(0u, 0u, 0u, 0u);
+    if (t + 4 >= m) b1 = make_uint4(0u, 0u, 0u, 0u);
+  }
+  // The tensor core cuts its sums off instead of rounding them, so a long chain
+  // of steps through one accumulator drifts towards zero (1.5e-5 of the spectra
+  // at 2000 bins, 25 times the FP32 product's error). Each group is summed on
+  // its own (against lo of B, then hi) and added to the accumulators in FP32.
+  const uint32_t w0[4] = {b0.x, b0.y, b0.z, b0.w}, w1[4] = {b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-  for (int i = 0; i < TB; ++i) {
-    float pv[4];
+  for (int c = 0; c < 4; ++c) {
+    const uint32_t l0 = __byte_perm(w0[c], 0u, 0x3232u), l1 = __byte_perm(w1[c], 0u, 0x3232u);
+    const uint32_t h0 = __byte_perm(w0[c], 0u, 0x1010u), h1 = __byte_perm(w1[c], 0u, 0x1010u);
+    float d[MT][4];
+    const float zero[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float t1 = acc.get(0, i, q), t2 = acc.get(1, i, q), t3 = acc.get(2, i, q);
-      const float fr = __fsub_rn(t1, t2);
-      const float fi = __fsub_rn(__fsub_rn(t3, t1), t2);
-      pv[q] = __fmaf_rn(fr, fr, __fmul_rn(fi, fi));
+    for (int i = 0; i < MT; ++i) mma16816(d[i], a[i], l0, l1, zero);
+#pragma unroll
+    for (int i = 0; i < MT; ++i) mma16816(d[i], a[i], h0, h1, d[i]);
+#pragma unroll
+    for (int i = 0; i < MT; ++i) {
+      float *x = acc.x[i][c];
+#pragma unroll
+      for (int k = 0; k < 4; k += 2) {
+        const float2 r = __fadd2_rn(make_float2(x[k], x[k + 1]), make_float2(d[i][k], d[i][k + 1]));
+        x[k] = r.x;
+        x[k + 1] = r.y;
+      }
     }
-    const int row = row_base + bg * TB + i;
-    *reinterpret_cast<float4 *>(Pw + row * 32 + rg * 4) = make_float4(pv[0], pv[1], pv[2], pv[3]);
   }
 }
 
@@ -239,7 +317,7 @@ struct BlockedArgs {
   const uint32_t *n_heavy;   // count of heavy items
   uint32_t heavy_cap;        // capacity of the heavy list
   uint32_t *cursors;         // [0] heavy cursor, [1] light cursor
-  GridConst g;
+  int N, nbr;                // bins, rows of 32 bins
   CombConst cc;
   float *P;                  // spectra (write mode), rows in active order of slot 0
   int64_t ld;                // row stride of P in floats (>= N)
@@ -252,104 +330,122 @@ struct BlockedArgs {
   int pw_offset;             // byte offset of the spectrum buffer inside a warp's area
   uint32_t *flags;
   int64_t ev_cap;            // events each slot's event array holds (CSR bound)
+  NdftConst nd;
 };
 
-// Bins [j_begin, j_end) of spectrum row `prow` from Pw (bin j_begin at Pw[0])
-// to P, by 16-byte stores when rows are 16-byte aligned (j_begin is a
-// multiple of 32).
-__device__ __forceinline__ void store_row(const BlockedArgs &A, int64_t prow, int j_begin,
-                                          int j_end, const float *Pw) {
-  const int lane = threadIdx.x & 31;
-  float *dst = A.P + prow * A.ld + j_begin;
-  int j0 = j_begin;
-  if (A.vec_store) {
-    const int n4 = (j_end - j_begin) >> 2;
-    for (int i = lane; i < n4; i += 32)
-      reinterpret_cast<float4 *>(dst)[i] = reinterpret_cast<const float4 *>(Pw)[i];
-    j0 = j_begin + 4 * n4;
-  }
-  for (int j = j0 + lane; j < j_end; j += 32) dst[j - j_begin] = Pw[j - j_begin];
+// Bins of [j_begin, j_end) whose phase is 0 for every event: the squared sum
+// of the pixel's polarities, after the tile that holds them was written.
+__device__ __forceinline__ void exact_bins(const BlockedArgs &A, int sum_p, int j_begin, int j_end,
+                                           float *row) {
+  if (A.nd.dc_first < 0 || A.nd.dc_first >= j_end) return;
+  __syncwarp();
+  const float p2 = __fmul_rn((float)sum_p, (float)sum_p);
+  for (int j = A.nd.dc_first; j < j_end; j += A.nd.dc_step)
+    if (j >= j_begin && (threadIdx.x & 31) == 0) row[j] = p2;
 }
 
-// One pixel's spectrum into Pw (fused: all passes, N padded) or streamed to P.
-template <int TB, bool FUSED>
-__device__ __forceinline__ void pixel_spectrum_warp(const BlockedArgs &A, const uint32_t *evp,
-                                                    int cnt, int64_t prow, float4 *stage,
-                                                    float *Pw) {
-  const int lane = threadIdx.x & 31;
-  const GridConst &g = A.g;
-  const int rows_per_pass = 4 * TB;
-  for (int b0 = 0; b0 < g.nbr; b0 += rows_per_pass) {
-    const uint64_t arow_mod[2] = {arow_residue(g, b0), arow_residue(g, b0 + 2 * TB)};
-    Acc<TB> acc;
-    acc.zero();
-    accumulate<TB>(evp, cnt, 0, 1, g, arow_mod, stage, acc);
-    if (FUSED) {
-      finalize_tile<TB>(acc, Pw, b0);
-    } else {
-      finalize_tile<TB>(acc, Pw, 0);
-      __syncwarp();
-      const int j_begin = 32 * b0, j_end = min(g.N, 32 * (b0 + rows_per_pass));
-      store_row(A, prow, j_begin, j_end, Pw);
-    }
-    __syncwarp();
+// Power of the lane's tile into Pw (row-major bins from row_base on).
+template <int MT>
+__device__ __forceinline__ void finalize_tile(const Acc<MT> &acc, float *Pw, int row_base) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+    float pp[4], pm[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc.powers(i, q, pp[q], pm[q]);
+    float *row = Pw + (row_base + MT * g + i) * 32;
+    *reinterpret_cast<float4 *>(row + 16 + 4 * t) = make_float4(pp[0], pp[1], pp[2], pp[3]);
+    *reinterpret_cast<float4 *>(row + 12 - 4 * t) = make_float4(pm[3], pm[2], pm[1], pm[0]);
   }
 }
 
-// Power of the lane's tile straight to spectrum row `prow` (bin rows from b0):
-// lane (bg, rg) holds bins 32 (b0 + bg TB + i) + 4 rg + q, so each store of
-// the warp covers four whole 128-byte rows; bins at or beyond N are not written.
-template <int TB>
-__device__ __forceinline__ void store_tile(const BlockedArgs &A, const Acc<TB> &acc, int64_t prow,
-                                           int b0) {
-  const int lane = threadIdx.x & 31;
-  const int bg = lane >> 3, rg = lane & 7;
-  const int N = A.g.N;
+// Power of the lane's tile straight to spectrum row `prow` (bin rows from b0),
+// by 16-byte stores when rows are 16-byte aligned; bins at or beyond N are not
+// written.
+template <int MT>
+__device__ __forceinline__ void store_tile(const BlockedArgs &A, const Acc<MT> &acc, int64_t prow,
+                                           int b0, int sum_p) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   float *dst = A.P + prow * A.ld;
 #pragma unroll
-  for (int i = 0; i < TB; ++i) {
-    float pv[4];
+  for (int i = 0; i < MT; ++i) {
+    float pv[2][4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float t1 = acc.get(0, i, q), t2 = acc.get(1, i, q), t3 = acc.get(2, i, q);
-      const float fr = __fsub_rn(t1, t2);
-      const float fi = __fsub_rn(__fsub_rn(t3, t1), t2);
-      pv[q] = __fmaf_rn(fr, fr, __fmul_rn(fi, fi));
-    }
-    const int j = 32 * (b0 + bg * TB + i) + 4 * rg;
-    if (A.vec_store && j + 3 < N) {
-      *reinterpret_cast<float4 *>(dst + j) = make_float4(pv[0], pv[1], pv[2], pv[3]);
-    } else {
+    for (int q = 0; q < 4; ++q) acc.powers(i, q, pv[1][q], pv[0][3 - q]);
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (j + q < N) dst[j + q] = pv[q];
+    for (int h = 0; h < 2; ++h) {
+      const int j = 32 * (b0 + MT * g + i) + (h ? 16 + 4 * t : 12 - 4 * t);
+      if (A.vec_store && j + 3 < A.N) {
+        *reinterpret_cast<float4 *>(dst + j) =
+            make_float4(pv[h][0], pv[h][1], pv[h][2], pv[h][3]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (j + q < A.N) dst[j + q] = pv[h][q];
+      }
     }
+  }
+  exact_bins(A, sum_p, 32 * b0, min(A.N, 32 * (b0 + 8 * MT)), dst);
+}
+
+// Events of a pixel in chunks chunk0, chunk0 + step, ... of 32 (warp w of a
+// block takes chunks w, w + nw, ...); returns how many of them are negative.
+template <int MT>
+__device__ __forceinline__ int accumulate(const uint32_t *__restrict__ evp, int cnt, int chunk0,
+                                          int step, const NdftConst &nd, uint64_t f_row,
+                                          unsigned char *stage, Acc<MT> &acc) {
+  const int lane = threadIdx.x & 31;
+  int c0 = chunk0 * kGenChunk, neg = 0;
+  uint32_t w = c0 + lane < cnt ? evp[c0 + lane] : 0u;
+  for (; c0 < cnt; c0 += step * kGenChunk) {
+    const int ne = min(kGenChunk, cnt - c0);
+    gen_chunk<MT>(w, nd, f_row, stage);
+    neg += __popc(__ballot_sync(0xffffffffu, (w & kSignBit) != 0));
+    __syncwarp();
+    const int c1 = c0 + step * kGenChunk;  // the next chunk's event word, loaded ahead
+    w = c1 + lane < cnt ? evp[c1 + lane] : 0u;
+    for (int q = 0; q < ne; q += kGroup) mma_group<MT>(q, min(kGroup, ne - q), stage, acc);
+    __syncwarp();
+  }
+  return neg;
+}
+
+// One pixel's spectrum into Pw (all passes).
+template <int MT>
+__device__ __forceinline__ void pixel_spectrum_warp(const BlockedArgs &A, const uint32_t *evp,
+                                                    int cnt, unsigned char *stage, float *Pw) {
+  for (int b0 = 0, pass = 0; b0 < A.nbr; b0 += 8 * MT, ++pass) {
+    Acc<MT> acc;
+    acc.zero();
+    const int neg = accumulate<MT>(evp, cnt, 0, 1, A.nd, A.nd.f_row[pass], stage, acc);
+    finalize_tile<MT>(acc, Pw, b0);
+    exact_bins(A, cnt - 2 * neg, 32 * b0, min(A.N, 32 * (b0 + 8 * MT)), Pw);
+    __syncwarp();
   }
 }
 
 // Light pixels of one slot, spectra to global memory. A warp takes runs of
 // `run` consecutive active pixels and, when their event lists follow one
 // another in memory (the CSR order of the binning), streams the run's events
-// through the 16-event factor chunks in that order: the factors of an event do
+// through the 32-event factor chunks in that order: the factors of an event do
 // not depend on its pixel, so one chunk serves the end of one pixel and the
 // start of the next, and a pixel's tile is stored and cleared as soon as its
-// last event is in. Events of pixels outside the run's light set (heavy ones,
-// pixels left to the hybrid path, inactive pixels) are skipped chunk-wise.
-// Runs whose lists are not in order (caller-built lists) are streamed one
-// pixel at a time. The run length is 16 pixels when there are at least eight
-// such runs per warp of the grid, and halves (down to one pixel) until there
-// are: on a sparse window the warps then share the pixels evenly instead of a
-// few runs of heavy-tailed pixels setting the kernel's time. A pixel's events
-// are accumulated in the same order whatever the run length, so the spectra
-// do not depend on it.
-template <int TB>
-__device__ __forceinline__ void light_stream(const BlockedArgs &A, float4 *stage) {
+// last event is in. A pixel's groups of 8 events count from its first one; a
+// group that does not lie in the staged chunk as a whole starts the next chunk
+// (at most 7 events are generated again). Events of pixels outside the run's
+// light set (heavy ones, pixels left to the hybrid path, inactive pixels) are
+// skipped. Runs whose lists are not in order (caller-built lists) are streamed
+// one pixel at a time. The run length is 16 pixels when there are at least
+// eight such runs per warp of the grid, and halves (down to one pixel) until
+// there are: on a sparse window the warps then share the pixels evenly instead
+// of a few runs of heavy-tailed pixels setting the kernel's time. A pixel's
+// events are accumulated in the same groups and order whatever the run length,
+// so the spectra do not depend on it.
+template <int MT>
+__device__ __forceinline__ void light_stream(const BlockedArgs &A, unsigned char *stage) {
   const int lane = threadIdx.x & 31;
-  const int e = lane & 15;
-  const GridConst &g = A.g;
   const SlotView &v = A.views[A.slot0];
   const int64_t n_act = (int64_t)v.counters[2];
-  const int rows_per_pass = 4 * TB;
   const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   int run = 16;
   while (run > 1 && (int64_t)run * n_warps * 8 > n_act) run >>= 1;
@@ -387,34 +483,40 @@ __device__ __forceinline__ void light_stream(const BlockedArgs &A, float4 *stage
       const uint32_t sub = in_order ? todo : (todo & (0u - todo));
       todo &= ~sub;
       const uint32_t e_end = __shfl_sync(0xffffffffu, q_hi, 31 - __clz(sub));
-      for (int b0 = 0; b0 < g.nbr; b0 += rows_per_pass) {
-        const uint64_t arow_mod[2] = {arow_residue(g, b0), arow_residue(g, b0 + 2 * TB)};
-        // the staged chunk holds events [c0, cend); wn: word of event cend + e
-        uint32_t c0 = 0, cend = 0, wn = 0;
-        bool have_wn = false;
+      for (int b0 = 0, pass = 0; b0 < A.nbr; b0 += 8 * MT, ++pass) {
+        // the staged chunk holds events [c0, c0 + 32) of the run (c0 = ~0: none
+        // yet), words wc; wn: the 32 words after them; sgn: their signs
+        uint32_t c0 = 0xffffffffu, wc = 0, wn = 0, sgn = 0;
         for (uint32_t rem = sub; rem; rem &= rem - 1) {
           const int p = __ffs(rem) - 1;
           const uint32_t pe0 = __shfl_sync(0xffffffffu, q_lo, p);
           const uint32_t pe1 = __shfl_sync(0xffffffffu, q_hi, p);
-          Acc<TB> acc;
+          Acc<MT> acc;
           acc.zero();
-          for (uint32_t pos = pe0; pos < pe1;) {
-            if (pos >= cend) {  // stage the chunk that starts at pos
-              const uint32_t w =
-                  have_wn && pos == cend ? wn : (pos + e < e_end ? v.ev[pos + e] : 0u);
+          int neg = 0;
+          for (uint32_t pos = pe0; pos < pe1; pos += kGroup) {
+            const int m = (int)min((uint32_t)kGroup, pe1 - pos);
+            uint32_t d = pos - c0;
+            if (c0 == 0xffffffffu || d + m > (uint32_t)kGenChunk) {  // stage from pos on
+              if (c0 != 0xffffffffu && d <= 32u) {  // among the words already loaded
+                const uint32_t x = __shfl_sync(0xffffffffu, wc, (lane + d) & 31u);
+                const uint32_t y = __shfl_sync(0xffffffffu, wn, (lane + d) & 31u);
+                wc = lane + d < 32u ? x : y;
+              } else {
+                wc = pos + lane < e_end ? v.ev[pos + lane] : 0u;
+              }
               c0 = pos;
-              cend = min(c0 + (uint32_t)kGenChunk, e_end);
+              d = 0;
               __syncwarp();  // the previous chunk's products are done
-              gen_chunk<TB>(w, c0 + e < cend, g, arow_mod, stage);
+              gen_chunk<MT>(wc, A.nd, A.nd.f_row[pass], stage);
+              sgn = __ballot_sync(0xffffffffu, (wc & kSignBit) != 0);
               __syncwarp();
-              wn = cend + e < e_end ? v.ev[cend + e] : 0u;
-              have_wn = true;
+              wn = pos + 32u + lane < e_end ? v.ev[pos + 32u + lane] : 0u;
             }
-            const uint32_t e1 = min(pe1, cend);
-            gemm_range<TB>((int)(pos - c0), (int)(e1 - c0), stage, acc);
-            pos = e1;
+            neg += __popc((sgn >> d) & (0xffu >> (kGroup - m)));
+            mma_group<MT>((int)d, m, stage, acc);
           }
-          store_tile<TB>(A, acc, (int64_t)a0 + p, b0);
+          store_tile<MT>(A, acc, (int64_t)a0 + p, b0, (int)(pe1 - pe0) - 2 * neg);
         }
         __syncwarp();
       }
@@ -434,14 +536,14 @@ __device__ __forceinline__ void store_scores(const BlockedArgs &A, const SlotVie
   }
 }
 
-template <int TB, int NW, bool FUSED>
-__global__ void __launch_bounds__(256, TB == 6 ? 2 : 1) k_blocked(BlockedArgs A) {
+template <int MT, int NW, bool FUSED>
+__global__ void __launch_bounds__(256, 2) k_blocked(BlockedArgs A) {
   extern __shared__ float4 smem4[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int warp_f4 = A.warp_bytes / 16;
-  float4 *stage = smem4 + warp * warp_f4;
-  float *Pw = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(stage) + A.pw_offset);
+  unsigned char *stage = reinterpret_cast<unsigned char *>(smem4) + warp * A.warp_bytes;
+  float *Pw = reinterpret_cast<float *>(stage + A.pw_offset);
   __shared__ uint32_t s_item;
+  __shared__ int s_neg[8];
 
   // ---------------- heavy pixels: one block each, events split over warps
   const uint32_t n_heavy = min(*A.n_heavy, A.heavy_cap);
@@ -460,63 +562,51 @@ __global__ void __launch_bounds__(256, TB == 6 ? 2 : 1) k_blocked(BlockedArgs A)
     const int cnt = (int)(v.offsets[key + 1] - o0);
     if (A.skip_min > 0 && cnt >= A.skip_min) continue;
     if (!ddhf_check((int64_t)o0 + cnt <= A.ev_cap, A.flags)) continue;
-    const int rows_per_pass = 4 * TB;
-    bool overflow = !FUSED && a >= A.cap_px;
-    if (overflow) {
+    if (!FUSED && a >= A.cap_px) {
       if (threadIdx.x == 0) raise_flag(A.flags, DDHF_FLAG_CAPACITY);
       continue;
     }
-    for (int b0 = 0; b0 < A.g.nbr; b0 += rows_per_pass) {
-      const uint64_t arow_mod[2] = {arow_residue(A.g, b0), arow_residue(A.g, b0 + 2 * TB)};
-      Acc<TB> acc;
+    for (int b0 = 0, pass = 0; b0 < A.nbr; b0 += 8 * MT, ++pass) {
+      Acc<MT> acc;
       acc.zero();
-      accumulate<TB>(v.ev + o0, cnt, warp, nw, A.g, arow_mod, stage, acc);
-      // partial sums of this warp -> its staging area, [comp][i][q][lane]
+      const int neg = accumulate<MT>(v.ev + o0, cnt, warp, nw, A.nd, A.nd.f_row[pass], stage, acc);
+      // partial sums of this warp -> its staging area, [row, column, component][lane]
       float *part = reinterpret_cast<float *>(stage);
 #pragma unroll
-      for (int i = 0; i < TB; ++i)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          part[((0 * TB + i) * 4 + q) * 32 + lane] = acc.get(0, i, q);
-          part[((1 * TB + i) * 4 + q) * 32 + lane] = acc.get(1, i, q);
-          part[((2 * TB + i) * 4 + q) * 32 + lane] = acc.get(2, i, q);
-        }
+      for (int i = 0; i < 16 * MT; ++i)
+        part[i * 32 + lane] = acc.x[i / 16][(i / 4) % 4][i % 4];
+      if (lane == 0) s_neg[warp] = neg;
       __syncthreads();
       if (warp == 0) {
+        int sum_p = cnt - 2 * neg;
         for (int w2 = 1; w2 < nw; ++w2) {
-          const float *op = reinterpret_cast<const float *>(smem4 + w2 * warp_f4);
+          const float *op = reinterpret_cast<const float *>(stage + w2 * A.warp_bytes);
 #pragma unroll
-          for (int i = 0; i < TB; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              float &x1 = acc.at(0, i, q), &x2 = acc.at(1, i, q);
-              float &x3 = acc.at(2, i, q);
-              x1 = __fadd_rn(x1, op[((0 * TB + i) * 4 + q) * 32 + lane]);
-              x2 = __fadd_rn(x2, op[((1 * TB + i) * 4 + q) * 32 + lane]);
-              x3 = __fadd_rn(x3, op[((2 * TB + i) * 4 + q) * 32 + lane]);
-            }
+          for (int i = 0; i < 16 * MT; ++i) {
+            float &x = acc.x[i / 16][(i / 4) % 4][i % 4];
+            x = __fadd_rn(x, op[i * 32 + lane]);
+          }
+          sum_p -= 2 * s_neg[w2];
         }
         if (FUSED) {
-          finalize_tile<TB>(acc, Pw, b0);
+          finalize_tile<MT>(acc, Pw, b0);
+          exact_bins(A, sum_p, 32 * b0, min(A.N, 32 * (b0 + 8 * MT)), Pw);
         } else {
-          finalize_tile<TB>(acc, Pw, 0);
-          __syncwarp();
-          const int j_begin = 32 * b0, j_end = min(A.g.N, 32 * (b0 + rows_per_pass));
-          store_row(A, a, j_begin, j_end, Pw);
+          store_tile<MT>(A, acc, a, b0, sum_p);
         }
         __syncwarp();
       }
       __syncthreads();
     }
     if (FUSED && warp == 0) {
-      CombOut o = comb_warp<NW>(Pw, A.cc, reinterpret_cast<unsigned char *>(stage));
+      CombOut o = comb_warp<NW>(Pw, A.cc, stage);
       store_scores<NW>(A, v, a, key, o);
     }
     __syncthreads();
   }
 
   if constexpr (!FUSED) {
-    light_stream<TB>(A, stage);
+    light_stream<MT>(A, stage);
     return;
   }
 
@@ -557,44 +647,34 @@ __global__ void __launch_bounds__(256, TB == 6 ? 2 : 1) k_blocked(BlockedArgs A)
       const uint32_t *evp = reinterpret_cast<const uint32_t *>(
           __shfl_sync(0xffffffffu, reinterpret_cast<uintptr_t>(m_ev), q));
       if (cnt < 0 || cnt >= A.heavy_min) continue;  // inactive, past the end, or heavy
-      if (A.skip_min > 0 && cnt >= A.skip_min) continue;  // hybrid grid path
-      if (!FUSED && a >= A.cap_px) {
-        if (lane == 0) raise_flag(A.flags, DDHF_FLAG_CAPACITY);
-        continue;
-      }
-      pixel_spectrum_warp<TB, FUSED>(A, evp, cnt, a, stage, Pw);
-      if (FUSED) {
-        CombOut o = comb_warp<NW>(Pw, A.cc, reinterpret_cast<unsigned char *>(stage));
-        store_scores<NW>(A, A.views[slot], a, key, o);
-      }
+      pixel_spectrum_warp<MT>(A, evp, cnt, stage, Pw);
+      CombOut o = comb_warp<NW>(Pw, A.cc, stage);
+      store_scores<NW>(A, A.views[slot], a, key, o);
     }
   }
 }
 
-template <int TB>
-int blocked_warp_bytes(const Ctx *c, bool fused, int NW, int *pw_offset) {
-  const int stage = WarpLayout<TB>::kStageF4 * 16;
-  const int nbr = (int)c->gconst.nbr;
-  const int pw = fused ? ((nbr + 4 * TB - 1) / (4 * TB)) * 4 * TB * 32 * 4 : 4 * TB * 32 * 4;
-  int scratch = stage;
-  const int partial = 3 * TB * 4 * 32 * 4;
-  if (partial > scratch) scratch = partial;
-  if (fused) {
-    int cb = comb_scratch_bytes(c->comb, NW);
-    if (cb > scratch) scratch = cb;
-  }
-  scratch = (scratch + 15) & ~15;
-  if (!fused) {
-    // the tile of one pass is written after that pass's last GEMM step and
-    // streamed out before the next generation step: it shares the staging area
-    *pw_offset = 0;
-    return scratch > pw ? scratch : pw;
-  }
-  *pw_offset = scratch;
-  return scratch + pw;
+// m-tiles (of 8 rows) per pass for a grid of nbr rows: rows_per_lane (4 rows of
+// a pass each) when the tuning sets it, else as few passes as MT <= 4 allows
+// (every pass generates the columns again), evenly filled.
+inline int tiles_per_pass(int nbr, int rows_per_lane) {
+  if (rows_per_lane > 0) return std::max(1, rows_per_lane / 2);
+  const int tiles = (nbr + 7) / 8, passes = (tiles + 3) / 4;
+  return (tiles + passes - 1) / passes;
 }
 
-template <int TB, int NW, bool FUSED>
+template <int MT>
+int blocked_warp_bytes(const Ctx *c, bool fused, int NW, int *pw_offset) {
+  int scratch = Stage<MT>::kBytes;
+  *pw_offset = 0;
+  if (!fused) return scratch;
+  scratch = std::max(scratch, comb_scratch_bytes(c->comb, NW));
+  scratch = (scratch + 15) & ~15;
+  *pw_offset = scratch;
+  return scratch + (((int)c->gconst.nbr + 8 * MT - 1) / (8 * MT)) * 8 * MT * 32 * 4;
+}
+
+template <int MT, int NW, bool FUSED>
 ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cudaStream_t s,
                              int slot0 = 0, int64_t ld = 0, int skip_min = 0) {
   BlockedArgs A{};
@@ -606,7 +686,9 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
   A.n_heavy = c->qctl + 0;
   A.heavy_cap = (uint32_t)std::min<int64_t>(c->heavy_cap, 0xffffffffll);
   A.cursors = c->qctl + 1;
-  A.g = c->gconst;
+  A.N = c->gconst.N;
+  A.nbr = c->gconst.nbr;
+  A.nd = make_ndft_const(c->gconst, MT);
   A.cc = c->comb;
   A.P = P;
   A.ld = ld > 0 ? ld : c->gconst.N;
@@ -614,12 +696,12 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
   A.cap_px = cap_px;
   A.heavy_min = c->tuning.heavy_min;
   A.skip_min = skip_min;
-  A.warp_bytes = blocked_warp_bytes<TB>(c, FUSED, NW, &A.pw_offset);
+  A.warp_bytes = blocked_warp_bytes<MT>(c, FUSED, NW, &A.pw_offset);
   A.flags = c->flags;
   A.ev_cap = std::max<int64_t>(c->max_events, 1);
   const int wpb = c->tuning.warps_per_block;
   const size_t smem = (size_t)A.warp_bytes * wpb;
-  auto kern = k_blocked<TB, NW, FUSED>;
+  auto kern = k_blocked<MT, NW, FUSED>;
   DDHF_CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)smem));
   int occ = 0;
@@ -635,47 +717,37 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
   return DDHF_OK;
 }
 
-// One kernel instantiation per rows-per-lane choice TB, for comb variant NW.
+// One kernel instantiation per m-tile count, for comb variant NW.
 template <int NW, bool FUSED>
-ddhf_status launch_blocked_tb(Ctx *c, int n_slots, float *P, int64_t cap_px, cudaStream_t s,
+ddhf_status launch_blocked_mt(Ctx *c, int n_slots, float *P, int64_t cap_px, cudaStream_t s,
                               int slot0, int64_t ld, int skip_min) {
-  const int nbr = c->gconst.nbr;
-  int tb = std::min(8, (nbr + 3) / 4);
-  tb = tb <= 2 ? tb : tb <= 4 ? 4 : tb <= 6 ? 6 : 8;
-  if (c->tuning.rows_per_lane > 0) tb = c->tuning.rows_per_lane;
-  switch (tb) {
-    case 1: return launch_blocked_t<1, NW, FUSED>(c, n_slots, P, cap_px, s, slot0, ld,
-                                                    skip_min);
-    case 2: return launch_blocked_t<2, NW, FUSED>(c, n_slots, P, cap_px, s, slot0, ld,
-                                                    skip_min);
-    case 4: return launch_blocked_t<4, NW, FUSED>(c, n_slots, P, cap_px, s, slot0, ld,
-                                                    skip_min);
-    case 6: return launch_blocked_t<6, NW, FUSED>(c, n_slots, P, cap_px, s, slot0, ld,
-                                                    skip_min);
-    case 8: return launch_blocked_t<8, NW, FUSED>(c, n_slots, P, cap_px, s, slot0, ld,
-                                                    skip_min);
+  switch (tiles_per_pass(c->gconst.nbr, c->tuning.rows_per_lane)) {
+    case 1: return launch_blocked_t<1, NW, FUSED>(c, n_slots, P, cap_px, s, slot0, ld, skip_min);
+    case 2: return launch_blocked_t<2, NW, FUSED>(c, n_slots, P, cap_px, s, slot0, ld, skip_min);
+    case 3: return launch_blocked_t<3, NW, FUSED>(c, n_slots, P, cap_px, s, slot0, ld, skip_min);
+    case 4: return launch_blocked_t<4, NW, FUSED>(c, n_slots, P, cap_px, s, slot0, ld, skip_min);
   }
   return DDHF_ERR_UNSUPPORTED;
 }
 
 // The fused kernels with the generic comb (1 or 8 mask words) are
 // instantiated in their own translation unit.
-extern template ddhf_status launch_blocked_tb<1, true>(Ctx *, int, float *, int64_t, cudaStream_t,
+extern template ddhf_status launch_blocked_mt<1, true>(Ctx *, int, float *, int64_t, cudaStream_t,
                                                        int, int64_t, int);
-extern template ddhf_status launch_blocked_tb<8, true>(Ctx *, int, float *, int64_t, cudaStream_t,
+extern template ddhf_status launch_blocked_mt<8, true>(Ctx *, int, float *, int64_t, cudaStream_t,
                                                        int, int64_t, int);
 
 template <bool FUSED>
 ddhf_status launch_blocked_any(Ctx *c, int n_slots, float *P, int64_t cap_px, cudaStream_t s,
                                int slot0 = 0, int64_t ld = 0, int skip_min = 0) {
   if constexpr (!FUSED) {
-    return launch_blocked_tb<1, false>(c, n_slots, P, cap_px, s, slot0, ld, skip_min);
+    return launch_blocked_mt<1, false>(c, n_slots, P, cap_px, s, slot0, ld, skip_min);
   } else {
     // the comb variant of the spectrum size: fast, or generic with 1 or 8 mask words
     switch (comb_variant(c->comb)) {
-      case 0: return launch_blocked_tb<0, true>(c, n_slots, P, cap_px, s, slot0, ld, 0);
-      case 1: return launch_blocked_tb<1, true>(c, n_slots, P, cap_px, s, slot0, ld, 0);
-      default: return launch_blocked_tb<8, true>(c, n_slots, P, cap_px, s, slot0, ld, 0);
+      case 0: return launch_blocked_mt<0, true>(c, n_slots, P, cap_px, s, slot0, ld, 0);
+      case 1: return launch_blocked_mt<1, true>(c, n_slots, P, cap_px, s, slot0, ld, 0);
+      default: return launch_blocked_mt<8, true>(c, n_slots, P, cap_px, s, slot0, ld, 0);
     }
   }
 }

@@ -17,7 +17,7 @@
 // cudaGetSymbolAddress() once per CUDA context (keyed by the context's
 // process-unique id), during the first call made with that context current.
 // That first call also loads every kernel this entry point can launch (all
-// five rows-per-lane instantiations of the spectrum kernel and the helpers),
+// four tile-count instantiations of the spectrum kernel and the helpers),
 // so that under lazy module loading no later call, whatever its grid, loads
 // code or allocates; it should therefore come before any stream capture and
 // outside any frame budget. Every call shares the array: the counters and
@@ -117,10 +117,10 @@ unsigned long long current_ctx_id() {
   return id;
 }
 
-template <int TB>
+template <int MT>
 cudaError_t load_blocked() {
   cudaFuncAttributes fa;
-  return cudaFuncGetAttributes(&fa, blocked::k_blocked<TB, 1, false>);
+  return cudaFuncGetAttributes(&fa, blocked::k_blocked<MT, 1, false>);
 }
 
 // The scratch address for the current context: looked up, and every kernel of
@@ -137,8 +137,7 @@ ddhf_status scratch_for_current(NoAllocScratch **out) {
   if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return DDHF_ERR_CUDA;
   cudaFuncAttributes fa;
   if (load_blocked<1>() != cudaSuccess || load_blocked<2>() != cudaSuccess ||
-      load_blocked<4>() != cudaSuccess || load_blocked<6>() != cudaSuccess ||
-      load_blocked<8>() != cudaSuccess ||
+      load_blocked<3>() != cudaSuccess || load_blocked<4>() != cudaSuccess ||
       cudaFuncGetAttributes(&fa, k_noalloc_prepare) != cudaSuccess ||
       cudaFuncGetAttributes(&fa, k_noalloc_heavy) != cudaSuccess ||
       cudaFuncGetAttributes(&fa, k_noalloc_finish) != cudaSuccess)
@@ -149,7 +148,7 @@ ddhf_status scratch_for_current(NoAllocScratch **out) {
   return DDHF_OK;
 }
 
-template <int TB>
+template <int MT>
 ddhf_status launch_noalloc(NoAllocScratch *sp, const GridConst &g, float *P, int64_t cap_px,
                            int64_t n_active, int64_t n_events, int num_sms, cudaStream_t s) {
   blocked::BlockedArgs A{};
@@ -161,22 +160,20 @@ ddhf_status launch_noalloc(NoAllocScratch *sp, const GridConst &g, float *P, int
   A.n_heavy = &sp->qctl[0];
   A.heavy_cap = (uint32_t)kNoAllocMaxHeavy;
   A.cursors = &sp->qctl[1];
-  A.g = g;
+  A.N = g.N;
+  A.nbr = g.nbr;
+  A.nd = blocked::make_ndft_const(g, MT);
   A.cc = CombConst{};
   A.P = P;
   A.ld = g.N;
   A.vec_store = (A.ld % 4 == 0) && (reinterpret_cast<uintptr_t>(P) % 16 == 0);
   A.cap_px = cap_px;
   A.heavy_min = kNoAllocHeavyMin;
-  const int stage = blocked::WarpLayout<TB>::kStageF4 * 16;
-  const int partial = 3 * TB * 4 * 32 * 4;
-  const int scratch = ((stage > partial ? stage : partial) + 15) & ~15;
-  A.pw_offset = scratch;
-  A.warp_bytes = scratch + 4 * TB * 32 * 4;
+  A.warp_bytes = blocked::Stage<MT>::kBytes;
   A.flags = &sp->flags;
   A.ev_cap = n_events;
   const size_t smem = (size_t)A.warp_bytes * kNoAllocWarps;
-  auto kern = blocked::k_blocked<TB, 1, false>;
+  auto kern = blocked::k_blocked<MT, 1, false>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return DDHF_ERR_CUDA;
@@ -223,15 +220,12 @@ extern "C" ddhf_status ddhf_power_spectrum_noalloc(const ddhf_grid *grid, const 
   const int blocks = (int)std::min<int64_t>(ceil_div(n_active, 256), (int64_t)num_sms * 8);
   k_noalloc_heavy<<<blocks, 256, 0, s>>>(sp, offsets, active, n_active, P, g.N);
   if (cudaGetLastError() != cudaSuccess) return DDHF_ERR_CUDA;
-  int tb = std::min(8, (g.nbr + 3) / 4);
-  tb = tb <= 2 ? tb : tb <= 4 ? 4 : tb <= 6 ? 6 : 8;
   ddhf_status st;
-  switch (tb) {
+  switch (blocked::tiles_per_pass(g.nbr, 0)) {
     case 1: st = launch_noalloc<1>(sp, g, P, cap_px, n_active, n_events, num_sms, s); break;
     case 2: st = launch_noalloc<2>(sp, g, P, cap_px, n_active, n_events, num_sms, s); break;
-    case 4: st = launch_noalloc<4>(sp, g, P, cap_px, n_active, n_events, num_sms, s); break;
-    case 6: st = launch_noalloc<6>(sp, g, P, cap_px, n_active, n_events, num_sms, s); break;
-    default: st = launch_noalloc<8>(sp, g, P, cap_px, n_active, n_events, num_sms, s); break;
+    case 3: st = launch_noalloc<3>(sp, g, P, cap_px, n_active, n_events, num_sms, s); break;
+    default: st = launch_noalloc<4>(sp, g, P, cap_px, n_active, n_events, num_sms, s); break;
   }
   if (st != DDHF_OK) return st;
   if (flags_dev) {
