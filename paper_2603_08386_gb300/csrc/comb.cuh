@@ -462,19 +462,20 @@ __device__ __forceinline__ CombOut comb_warp_generic(const float *Pw, const Comb
 
 
 // ------------------------------------------------------------------------
-// Fast variants for N <= 1024 bins, a median band of at most 32 ranks and at
-// most 32 bins in a candidate's harmonic windows (M (2d+1) <= 32).
+// Fast variants for a median band of at most 32 ranks and at most 32 bins in a
+// candidate's harmonic windows (M (2d+1) <= 32), any number of bins.
 //
 // Same results as comb_warp_generic, bit for bit, with far fewer
 // instructions per pixel:
 //  * the log sum of Eq. 7 (base 2, scaled by ln 2 once) shares its pass with
-//    a histogram of 768 buckets linear in P over [0, 1.5 mean) (values above
-//    go to the last);
+//    a histogram of 768 buckets (3072 above 4096 bins, so that the band's
+//    buckets still hold few bins beside the band) linear in P over [0, 1.5
+//    mean) (values above go to the last);
 //  * the buckets holding ranks lo_r and hi_r bound the candidate bins; at
 //    most 64 candidates (about 31 on C3's spectra) are compacted into shared
 //    memory and sorted in registers as 32-bit keys (value bits relative to
-//    the smallest candidate, above the 10-bit bin index), so that lane p
-//    holds the bin of full rank lo_r + p;
+//    the smallest candidate, above a bin index of 10 to 14 bits), so that lane
+//    p holds the bin of full rank lo_r + p;
 //  * one window maximum per centre (Eq. 8), then N(w) for every candidate,
 //    kept in shared memory;
 //  * candidates are evaluated one at a time by the whole warp: lane i <
@@ -487,39 +488,47 @@ __device__ __forceinline__ CombOut comb_warp_generic(const float *Pw, const Comb
 //    N(w) / T below that bound can neither win nor tie (on C3's spectra
 //    fewer than two candidates per pixel are evaluated on average); the rest
 //    follow in increasing w.
+// Above 1024 bins these steps took over from comb_warp_generic, which scores
+// every candidate in full: 76,800 spectra of 2000 bins 4.95 -> 0.60 ms.
 // Two forms share these steps. The register form (512 < N <= 768, M = 4,
 // d = 3: Table 2's comb on the 750-bin grid) gives each lane 24 consecutive
 // bins in registers, so every per-bin pass is a fixed, fully unrolled
 // sequence and the window maxima come from registers and six shuffles. The
 // shared-memory form takes any other size within the limits.
-// Pixels whose candidates do not fit (more than 64, or a value range above
-// 2^22 ulps) take an exact radix selection of the band instead.
-// Scratch (bytes from the scratch base, 16-byte aligned):
-//   [0, 3072)   histogram u32[768]; once the band's buckets are located, over
-//               it: candidate value bits u32[64] at 0 and their bins u16[64]
-//               at 256; once the band is in registers: N(w) of candidate
-//               w_lo + i, f32[n_cand] (-1: complement empty), when it fits
-//   [3072, +16 ceil(N/4))  window maxima f32[N]
+// Pixels whose candidates do not fit (more than 64, or a value range that the
+// key has no room for: 2^22 ulps up to 1024 bins) take an exact radix selection
+// of the band instead.
+// Scratch (bytes from the scratch base, 16-byte aligned), HB = the histogram's
+// bytes (4 per bucket):
+//   [0, HB)     histogram; once the band's buckets are located, over it:
+//               candidate value bits u32[64] at 0 and their bins u16[64] at
+//               256; once the band is in registers: N(w) of candidate w_lo +
+//               i, f32[n_cand] (-1: complement empty), when it fits
+//   [HB, +16 ceil(N/4))  window maxima f32[N]
 //   then N(w), when it does not fit over the histogram
 struct CombFast {
-  static constexpr int kBuckets = 768;
   static constexpr int kHist = 0;
-  static constexpr int kHistBytes = 3072;
   static constexpr int kCandV = 0;
   static constexpr int kCandJ = 256;
-  static constexpr int kRec = 3072;
-  __host__ __device__ static int rec_end(int N) { return kRec + ((4 * N + 15) & ~15); }
+  static constexpr int kManyBins = 4096;  // above: 96 buckets per lane instead of 24
+  __host__ __device__ static constexpr int bpl(int N) { return N > kManyBins ? 96 : 24; }
+  __host__ __device__ static constexpr int hist_bytes(int bpl) { return 32 * bpl * 4; }
+  __host__ __device__ static int rec_off(int N) { return hist_bytes(bpl(N)); }
+  __host__ __device__ static int rec_end(int N) { return rec_off(N) + ((4 * N + 15) & ~15); }
   __host__ __device__ static int nw_off(int N, int n_cand) {
-    return 4 * n_cand <= kHistBytes ? 0 : rec_end(N);
+    return 4 * n_cand <= hist_bytes(bpl(N)) ? 0 : rec_end(N);
   }
   __host__ __device__ static int bytes(int N, int n_cand) {
     const int nc = n_cand > 0 ? n_cand : 0;
     const int e = nw_off(N, nc) + 4 * nc;
     return ((e > rec_end(N) ? e : rec_end(N)) + 15) & ~15;
   }
-  static constexpr int kMaxN = 1024;
   static constexpr int kMaxBand = 32;
   static constexpr int kMaxCand = 64;
+  // bits of a bin index in a candidate's sort key
+  __host__ __device__ static int index_bits(int N) {
+    return N <= 1024 ? 10 : N <= 2048 ? 11 : N <= 4096 ? 12 : N <= 8192 ? 13 : 14;
+  }
 };
 
 // The register form's shape: bins per lane, and the comb it is written for.
@@ -527,10 +536,13 @@ struct CombReg {
   static constexpr int kBPL = 24;
   static constexpr int kM = 4;
   static constexpr int kD = 3;
-  // every candidate then has all M windows and a non-empty complement
+  // every candidate has all M windows and a non-empty complement
+  __host__ __device__ static bool comb_fits(const CombConst &cc) {
+    return cc.M == kM && cc.d == kD && kM * cc.w_hi <= cc.N - 1 - kD &&
+           cc.N > kM * (2 * kD + 1);
+  }
   __host__ __device__ static bool fits(const CombConst &cc) {
-    return cc.N > 16 * kBPL && cc.N <= 32 * kBPL && cc.M == kM && cc.d == kD &&
-           kM * cc.w_hi <= cc.N - 1 - kD && cc.N > kM * (2 * kD + 1) &&
+    return cc.N > 16 * kBPL && cc.N <= 32 * kBPL && comb_fits(cc) &&
            cc.w_hi - cc.w_lo + 1 <= 256;
   }
 };
@@ -651,28 +663,30 @@ __device__ __noinline__ static void comb_records_any_d(const float *Pw, int N, i
   }
 }
 
-// 768 linear buckets over [0, 1.5 mean) (the fast forms' histogram, with
-// scale = 512 / mean): x = v scale clamped to at most 767, bucket floor(x),
-// taken by adding 2^23 rounded down (the float bits then hold floor(x) in the
-// low mantissa bits), so no float-to-integer conversion runs on the
-// special-function pipe. Monotone in v >= 0, so the bins of a bucket range
-// are a range of full ranks, and bucket g0 <= g <= g1 exactly when g0 <= x <
-// g1 + 1. Any input (a negative value, NaN) still gives an index in [0, 1023]
-// (a histogram word index below 512: inside the scratch).
+// 32 BPL linear buckets over [0, 1.5 mean) (the fast forms' histogram, with
+// scale = 64 BPL / (3 mean)): x = v scale clamped to the last bucket, bucket
+// floor(x), taken by adding 2^23 rounded down (the float bits then hold
+// floor(x) in the low mantissa bits), so no float-to-integer conversion runs on
+// the special-function pipe. Monotone in v >= 0, so the bins of a bucket range
+// are a range of full ranks, and bucket g0 <= g <= g1 exactly when g0 <= x < g1
+// + 1. Any input (a negative value, NaN) still gives an index below 1024 (BPL
+// 24) or 4096 (96): inside the scratch (the window maxima follow).
+template <int BPL>
 __device__ __forceinline__ float bucket_x(float v, float scale) {
-  return fminf(__fmul_rn(v, scale), 767.f);
+  return fminf(__fmul_rn(v, scale), (float)(32 * BPL - 1));
 }
+template <int BPL>
 __device__ __forceinline__ uint32_t bucket_bits(float v, float scale) {
-  return __float_as_uint(__fadd_rd(bucket_x(v, scale), 0x1p23f));  // 0x4B000000 + g
+  return __float_as_uint(__fadd_rd(bucket_x<BPL>(v, scale), 0x1p23f));  // 0x4B000000 + g
 }
-__device__ __forceinline__ int bucket_of(float v, float scale) {
-  return (int)(bucket_bits(v, scale) & 1023u);
-}
+template <int BPL>
+constexpr uint32_t kBucketMask = BPL == 24 ? 1023u : 4095u;
 
 // Add one to the bucket whose bucket_bits are ybits in the histogram at
 // shared address hist_sa (one counter per bucket).
+template <int BPL>
 __device__ __forceinline__ void hist_add(uint32_t hist_sa, uint32_t ybits) {
-  const uint32_t a = hist_sa + ((ybits & 1023u) << 2);
+  const uint32_t a = hist_sa + ((ybits & kBucketMask<BPL>) << 2);
   asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(a) : "memory");
 }
 
@@ -705,21 +719,23 @@ __device__ __forceinline__ float comb_cand_nw(const float *rec, int w, const Com
 }
 
 // The buckets holding full ranks lo_r and hi_r in the histogram; lane l owns
-// buckets [24 l, 24 l + 24). Returns the first and last candidate bucket, the
-// bins below the first (cb) and the candidate count.
+// buckets [BPL l, BPL (l + 1)). Returns the first and last candidate bucket,
+// the bins below the first (cb) and the candidate count.
 struct BandBuckets {
   int g0, g1, cb, ncand;
 };
+template <int BPL>
 __device__ __forceinline__ BandBuckets comb_locate(const uint32_t *hist, int N, int lo_r,
                                                    int hi_r, bool &bad) {
   const int lane = threadIdx.x & 31;
   uint32_t lsum;
   {
-    const uint4 *h4 = reinterpret_cast<const uint4 *>(hist) + lane * 6;
+    const uint4 *h4 = reinterpret_cast<const uint4 *>(hist) + lane * (BPL / 4);
     uint32_t s2 = 0;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const uint4 t = h4[(q + (lane >> 2)) % 6];  // rotated: no bank conflicts
+    for (int q = 0; q < BPL / 4; ++q) {
+      // rotated: no bank conflicts
+      const uint4 t = h4[(q + (BPL == 24 ? lane >> 2 : lane)) % (BPL / 4)];
       s2 += t.x + t.y + t.z + t.w;
     }
     lsum = s2;
@@ -727,6 +743,7 @@ __device__ __forceinline__ BandBuckets comb_locate(const uint32_t *hist, int N, 
   uint32_t tot;
   const uint32_t lex = warp_excl_scan<uint32_t>(lsum, tot);
   if (tot != (uint32_t)N) bad = true;
+  constexpr int K = (BPL + 31) / 32;  // buckets of the found lane per lane now
   int gsel[2];
   uint32_t gbelow[2], gcount[2];
 #pragma unroll
@@ -738,15 +755,32 @@ __device__ __forceinline__ BandBuckets comb_locate(const uint32_t *hist, int N, 
       bad = true;
     }
     const uint32_t base = __shfl_sync(0xffffffffu, lex, src);
-    const uint32_t h = lane < 24 ? hist[src * 24 + lane] : 0u;
+    uint32_t hk[K], h = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      hk[k] = K * lane + k < BPL ? hist[src * BPL + K * lane + k] : 0u;
+      h += hk[k];
+    }
     uint32_t t2;
-    const uint32_t ex = warp_excl_scan<uint32_t>(h, t2) + base;
+    uint32_t ex = warp_excl_scan<uint32_t>(h, t2) + base;
     int s2 = __ffs(__ballot_sync(0xffffffffu, R >= ex && R < ex + h)) - 1;
     if (s2 < 0) {
       s2 = 0;
       bad = true;
     }
-    gsel[t] = src * 24 + s2;
+    gsel[t] = src * BPL + K * s2;
+    if constexpr (K > 1) {
+      int kk = 0;
+      h = hk[0];
+#pragma unroll
+      for (int k = 1; k < K; ++k)
+        if (R >= ex + h && kk == k - 1) {
+          ex += h;
+          h = hk[k];
+          kk = k;
+        }
+      gsel[t] += __shfl_sync(0xffffffffu, kk, s2);
+    }
     gbelow[t] = __shfl_sync(0xffffffffu, ex, s2);
     gcount[t] = __shfl_sync(0xffffffffu, h, s2);
   }
@@ -760,12 +794,12 @@ __device__ __forceinline__ BandBuckets comb_locate(const uint32_t *hist, int N, 
 
 // The band from the ncand <= 64 compacted candidates (value bits cv, bins
 // cj; element i in lane i % 32, register i / 32): sorted as 32-bit keys,
-// lane p < bw takes full rank lo_r + p (value bv, bin bj). Returns false
-// (warp-uniform) when the values span 2^22 ulps or more, so that the exact
-// selection must run instead.
+// lane p < bw takes full rank lo_r + p (value bv, bin bj). ib: bits of a bin
+// index. Returns false (warp-uniform) when the values span 2^(32 - ib) ulps or
+// more, so that the exact selection must run instead.
 __device__ __forceinline__ bool comb_band_sorted(const unsigned char *scratch, int ncand,
-                                                 int lo_r, int cb, int bw, float &bv, int &bj,
-                                                 bool &bad) {
+                                                 int lo_r, int cb, int bw, int ib, float &bv,
+                                                 int &bj, bool &bad) {
   const int lane = threadIdx.x & 31;
   const uint32_t *cv = reinterpret_cast<const uint32_t *>(scratch + CombFast::kCandV);
   const uint16_t *cj = reinterpret_cast<const uint16_t *>(scratch + CombFast::kCandJ);
@@ -774,9 +808,9 @@ __device__ __forceinline__ bool comb_band_sorted(const unsigned char *scratch, i
   const uint32_t b1 = in1 ? cv[lane + 32] : 0xFFFFFFFFu;
   const uint32_t mn = __reduce_min_sync(0xffffffffu, min(b0, b1));
   const uint32_t mx = __reduce_max_sync(0xffffffffu, max(in0 ? b0 : 0u, in1 ? b1 : 0u));
-  if (mx - mn >= (1u << 22)) return false;
-  uint32_t k0 = in0 ? (((b0 - mn) << 10) | (uint32_t)cj[lane]) : 0xFFFFFFFFu;
-  uint32_t k1 = in1 ? (((b1 - mn) << 10) | (uint32_t)cj[lane + 32]) : 0xFFFFFFFFu;
+  if (mx - mn >= (1u << (32 - ib))) return false;
+  uint32_t k0 = in0 ? (((b0 - mn) << ib) | (uint32_t)cj[lane]) : 0xFFFFFFFFu;
+  uint32_t k1 = in1 ? (((b1 - mn) << ib) | (uint32_t)cj[lane + 32]) : 0xFFFFFFFFu;
   if (ncand <= 32) k0 = warp_sort32_u32(k0);
   else warp_sort64_u32(k0, k1);
   // band position p is sorted element i = lo_r - cb + p (lane i % 32, register i / 32)
@@ -785,8 +819,8 @@ __device__ __forceinline__ bool comb_band_sorted(const unsigned char *scratch, i
   const uint32_t kk1 = __shfl_sync(0xffffffffu, k1, i & 31);
   const uint32_t kk = i < 32 ? kk0 : kk1;
   if (lane < bw && (i < 0 || i >= ncand)) bad = true;
-  bv = __uint_as_float((kk >> 10) + mn);
-  bj = (int)(kk & 1023u);
+  bv = __uint_as_float((kk >> ib) + mn);
+  bj = (int)(kk & ((1u << ib) - 1u));
   return true;
 }
 
@@ -805,9 +839,8 @@ __device__ __forceinline__ void comb_nw_all(const float *rec, float *nws, const 
     // every candidate has all KM windows and a non-empty complement: N(w) is
     // a plain sum of KM window maxima
 #pragma unroll 1
-    for (int k = 0; k < 8; ++k) {
-      const int i = lane + 32 * k;
-      if (32 * k >= n_cand) break;
+    for (int i0 = 0; i0 < n_cand; i0 += 32) {
+      const int i = i0 + lane;
       if (i < n_cand) {
         const int w = cc.w_lo + i;
         float sm = rec[w];
@@ -938,7 +971,10 @@ __device__ __forceinline__ CombOut comb_out(float best, int bestw, bool bad, flo
   return out;
 }
 
-// The shared-memory form (any size within the fast limits).
+// The shared-memory form (any size within the fast limits; BPL = CombFast::bpl(N);
+// KM, KD > 0: M and d when every candidate has all M windows and a non-empty
+// complement, which halves the instructions of the candidate sums).
+template <int BPL, int KM = 0, int KD = 0>
 __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const CombConst &cc,
                                                        unsigned char *scratch) {
   const int lane = threadIdx.x & 31;
@@ -970,7 +1006,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum = __fadd_rn(sum, __shfl_xor_sync(0xffffffffu, sum, o));
   const float fN = (float)N;
-  const float scale = __fdiv_rn(512.f, __fdiv_rn(sum, fN));
+  const float scale = __fdiv_rn(64.f * BPL / 3.f, __fdiv_rn(sum, fN));
   __syncwarp();
   float sl2 = 0.f;  // sum of log2 max(P, 1e-30)
   for (int q = lane; q < nfull; q += 32) {
@@ -988,63 +1024,68 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
   out.log_sf = sum > 0.f ? __fsub_rn(__fdiv_rn(slog, fN), __logf(__fdiv_rn(sum, fN))) : 0.f;
   if (!(out.log_sf <= cc.ln_tau_sf) || cc.w_hi < cc.w_lo) return out;
 #pragma unroll
-  for (int q = 0; q < CombFast::kHistBytes / 512; ++q)
+  for (int q = 0; q < CombFast::hist_bytes(BPL) / 512; ++q)
     reinterpret_cast<uint4 *>(hist)[q * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
   __syncwarp();
   for (int q = lane; q < nfull; q += 32) {
     const float4 v = P4[q];
-    hist_add(hist_sa, bucket_bits(v.x, scale));
-    hist_add(hist_sa, bucket_bits(v.y, scale));
-    hist_add(hist_sa, bucket_bits(v.z, scale));
-    hist_add(hist_sa, bucket_bits(v.w, scale));
+    hist_add<BPL>(hist_sa, bucket_bits<BPL>(v.x, scale));
+    hist_add<BPL>(hist_sa, bucket_bits<BPL>(v.y, scale));
+    hist_add<BPL>(hist_sa, bucket_bits<BPL>(v.z, scale));
+    hist_add<BPL>(hist_sa, bucket_bits<BPL>(v.w, scale));
   }
   if (lane == tail_lane)
-    for (int j = jt; j < N; ++j) hist_add(hist_sa, bucket_bits(Pw[j], scale));
+    for (int j = jt; j < N; ++j) hist_add<BPL>(hist_sa, bucket_bits<BPL>(Pw[j], scale));
   __syncwarp();
 
   // ---- the band: lane p < bw holds the bin at full rank lo_r + p
   const int lo_r = cc.lo_r, bw = cc.bw, hi_r = cc.lo_r + cc.bw - 1;
-  const BandBuckets bb = comb_locate(hist, N, lo_r, hi_r, bad);
+  const BandBuckets bb = comb_locate<BPL>(hist, N, lo_r, hi_r, bad);
   bool slow = bb.ncand > CombFast::kMaxCand || bad;
   float bv = 0.f;  // its value
   int bj = 0;      // its bin
   if (!slow) {
-    // this lane's candidates: bit 4k + u for element u of group lane + 32 k
-    const uint32_t g0 = (uint32_t)bb.g0, gspan = (uint32_t)(bb.g1 - bb.g0);
-    uint32_t m = 0;
+    // this lane's candidates of 1024 bins: bit 4k + u for element u of group
+    // lane + 32 k, compacted in lane order; the next 1024 bins behind them
+    const float x0 = (float)bb.g0, x1 = (float)(bb.g1 + 1);
+    uint32_t *cv = reinterpret_cast<uint32_t *>(scratch + CombFast::kCandV);
+    uint16_t *cj = reinterpret_cast<uint16_t *>(scratch + CombFast::kCandJ);
+    uint32_t run = 0;
+    __syncwarp();  // the histogram has been read
+#pragma unroll 1
+    for (int q0 = 0; q0 < ng; q0 += 256) {
+      uint32_t m = 0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int q = lane + 32 * k;
-      if (32 * k < ng && q < ng) {
-        const float4 v = P4[q];
-        const int j = 4 * q;
-        m |= ((uint32_t)(bucket_of(v.x, scale) - g0) <= gspan ? 1u : 0u) << (4 * k);
-        m |= ((uint32_t)(bucket_of(v.y, scale) - g0) <= gspan && j + 1 < N ? 1u : 0u)
-             << (4 * k + 1);
-        m |= ((uint32_t)(bucket_of(v.z, scale) - g0) <= gspan && j + 2 < N ? 1u : 0u)
-             << (4 * k + 2);
-        m |= ((uint32_t)(bucket_of(v.w, scale) - g0) <= gspan && j + 3 < N ? 1u : 0u)
-             << (4 * k + 3);
+      for (int k = 0; k < 8; ++k) {
+        const int q = q0 + lane + 32 * k;
+        if (q0 + 32 * k < ng && q < ng) {
+          const float4 v = P4[q];
+          const int j = 4 * q;
+          const float x[4] = {bucket_x<BPL>(v.x, scale), bucket_x<BPL>(v.y, scale),
+                              bucket_x<BPL>(v.z, scale), bucket_x<BPL>(v.w, scale)};
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            m |= (x[u] >= x0 && x[u] < x1 && j + u < N ? 1u : 0u) << (4 * k + u);
+        }
       }
-    }
-    uint32_t nsel;
-    uint32_t off = warp_excl_scan<uint32_t>((uint32_t)__popc(m), nsel);
-    if ((int)nsel != bb.ncand) slow = true;  // uniform (a reduction)
-    if (!slow) {
-      uint32_t *cv = reinterpret_cast<uint32_t *>(scratch + CombFast::kCandV);
-      uint16_t *cj = reinterpret_cast<uint16_t *>(scratch + CombFast::kCandJ);
-      while (m) {
+      uint32_t nsel;
+      uint32_t off = run + warp_excl_scan<uint32_t>((uint32_t)__popc(m), nsel);
+      run += nsel;
+      while (m && off < (uint32_t)CombFast::kMaxCand) {
         const int b = __ffs(m) - 1;
         m &= m - 1;
-        const int j = 4 * (lane + 32 * (b >> 2)) + (b & 3);
+        const int j = 4 * (q0 + lane + 32 * (b >> 2)) + (b & 3);
         cv[off] = __float_as_uint(Pw[j]);
         cj[off] = (uint16_t)j;
         ++off;
       }
-      __syncwarp();
-      if (!comb_band_sorted(scratch, bb.ncand, lo_r, bb.cb, bw, bv, bj, bad)) slow = true;
-      __syncwarp();
     }
+    __syncwarp();
+    if ((int)run != bb.ncand) slow = true;  // uniform (a warp total)
+    if (!slow && !comb_band_sorted(scratch, bb.ncand, lo_r, bb.cb, bw, CombFast::index_bits(N),
+                                   bv, bj, bad))
+      slow = true;
+    __syncwarp();
   }
   if (slow) {
     // exact band [lo_r, hi_r] by radix selection (a rare, out-of-line path)
@@ -1057,8 +1098,8 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
 
   // ---- window maxima: rec[c] = max of P over [c - d, c + d] (centres
   // d .. N-1-d are the ones read)
-  const int d = cc.d;
-  float *rec = reinterpret_cast<float *>(scratch + CombFast::kRec);
+  const int d = KD ? KD : cc.d;
+  float *rec = reinterpret_cast<float *>(scratch + CombFast::hist_bytes(BPL));
   if (d == 3) {
     // centre quads 4q .. 4q + 3: bins 4q - 4 .. 4q + 7 by three 16-byte loads
     for (int q = lane; q < ng; q += 32) {
@@ -1103,11 +1144,11 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
   float *nws = reinterpret_cast<float *>(scratch + CombFast::nw_off(N, cc.w_hi - cc.w_lo + 1));
   float maxnw;
   int maxi;
-  comb_nw_all<0, 0>(rec, nws, cc, uniform, maxnw, maxi);
+  comb_nw_all<KM, KD>(rec, nws, cc, uniform, maxnw, maxi);
   __syncwarp();
   float best;
   int bestw;
-  comb_best<0, 0>(Pw, nws, cc, uniform, maxnw, maxi, bv, bj, best, bestw, bad);
+  comb_best<KM, KD>(Pw, nws, cc, uniform, maxnw, maxi, bv, bj, best, bestw, bad);
   out = comb_out(best, bestw, bad, out.log_sf, cc);
   __syncwarp();
   return out;
@@ -1179,18 +1220,18 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
                          : 0.f;
   if (!(out.log_sf <= cc.ln_tau_sf) || cc.w_hi < cc.w_lo) return out;
 #pragma unroll
-  for (int q = 0; q < CombFast::kHistBytes / 512; ++q)
+  for (int q = 0; q < CombFast::hist_bytes(24) / 512; ++q)
     reinterpret_cast<uint4 *>(hist)[q * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
   __syncwarp();
 #pragma unroll
-  for (int i = 0; i < kB; ++i) hist_add(hist_sa, bucket_bits(v[i], scale));
+  for (int i = 0; i < kB; ++i) hist_add<24>(hist_sa, bucket_bits<24>(v[i], scale));
   if (npad > 0) atomicSub(&hist[0], (uint32_t)npad);  // bucket 0 is the low half of word 0
   __syncwarp();
 
   // ---- window maxima of the lane's centres from its bins and three bins of
   // each neighbour: b[i] = P[base - 3 + i], i = 0..29; centres 4k .. 4k+3 of
   // the lane need b[4k .. 4k+9]
-  float *rec = reinterpret_cast<float *>(scratch + CombFast::kRec);
+  float *rec = reinterpret_cast<float *>(scratch + CombFast::hist_bytes(24));
   {
     float lft[kD], rgt[kD];
 #pragma unroll
@@ -1219,7 +1260,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
 
   // ---- the band: lane p < bw holds the bin at full rank lo_r + p
   const int lo_r = cc.lo_r, bw = cc.bw, hi_r = cc.lo_r + cc.bw - 1;
-  const BandBuckets bb = comb_locate(hist, N, lo_r, hi_r, bad);
+  const BandBuckets bb = comb_locate<24>(hist, N, lo_r, hi_r, bad);
   bool slow = bb.ncand > CombFast::kMaxCand || bad;
   float bv = 0.f;
   int bj = 0;
@@ -1238,7 +1279,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
       const float e[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const float x = bucket_x(e[u], scale);
+        const float x = bucket_x<24>(e[u], scale);
         m |= (x >= x0 && x < x1 ? 1u : 0u) << (4 * k + u);
       }
     }
@@ -1256,7 +1297,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
     }
     __syncwarp();
     if ((int)run != bb.ncand) slow = true;  // uniform (a warp total)
-    if (!slow && !comb_band_sorted(scratch, bb.ncand, lo_r, bb.cb, bw, bv, bj, bad)) slow = true;
+    if (!slow && !comb_band_sorted(scratch, bb.ncand, lo_r, bb.cb, bw, 10, bv, bj, bad)) slow = true;
     __syncwarp();
   }
   if (slow) {
@@ -1286,26 +1327,28 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
 __device__ __forceinline__ CombOut comb_warp_fast(const float *Pw, const CombConst &cc,
                                                   unsigned char *scratch) {
   if (CombReg::fits(cc)) return comb_warp_fast_regs(Pw, cc, scratch);
-  return comb_warp_fast_smem(Pw, cc, scratch);
+  if (cc.N > CombFast::kManyBins) return comb_warp_fast_smem<96>(Pw, cc, scratch);
+  return comb_warp_fast_smem<24>(Pw, cc, scratch);
 }
 
-// Which comb variant a context uses: 0 = fast (N <= 1024, band <= 32; the
-// register or shared-memory form, chosen at run time), otherwise the generic
-// one with NW mask words per centre. A kernel that scores every pixel of one
-// context can instead take the fast form itself: 2 = register form, 3 =
-// shared-memory form (comb_fast_form).
+// Which comb variant a context uses: 0 = fast (band <= 32 and M (2d+1) <= 32;
+// the register or shared-memory form, chosen at run time), otherwise the
+// generic one with NW mask words per centre. A kernel that scores every pixel
+// of one context can instead take the fast form itself: 2 = register form, 3 =
+// shared-memory form, 4 = the latter above 4096 bins, 5 and 6 = the same two
+// for Table 2's comb shape (comb_fast_form).
 __host__ __device__ inline int comb_variant(const CombConst &cc) {
-  if (cc.N <= CombFast::kMaxN && cc.bw <= CombFast::kMaxBand && cc.M * (2 * cc.d + 1) <= 32)
-    return 0;
+  if (cc.bw <= CombFast::kMaxBand && cc.M * (2 * cc.d + 1) <= 32) return 0;
   return cc.bw <= 32 ? 1 : 8;
 }
 
 __host__ __device__ inline int comb_fast_form(const CombConst &cc) {
-  return CombReg::fits(cc) ? 2 : 3;
+  if (CombReg::fits(cc)) return 2;
+  return (cc.N > CombFast::kManyBins ? 4 : 3) + (CombReg::comb_fits(cc) ? 2 : 0);
 }
 
 __host__ __device__ inline int comb_scratch_bytes(const CombConst &cc, int variant) {
-  return (variant == 0 || variant == 2 || variant == 3)
+  return (variant == 0 || (variant >= 2 && variant <= 6))
              ? CombFast::bytes(cc.N, cc.w_hi - cc.w_lo + 1)
              : CombScratch::bytes(cc.N, variant);
 }
@@ -1317,7 +1360,12 @@ __device__ __forceinline__ CombOut comb_warp(const float *Pw, const CombConst &c
                                              unsigned char *scratch) {
   if constexpr (NW == 0) return comb_warp_fast(Pw, cc, scratch);
   else if constexpr (NW == 2) return comb_warp_fast_regs(Pw, cc, scratch);
-  else if constexpr (NW == 3) return comb_warp_fast_smem(Pw, cc, scratch);
+  else if constexpr (NW == 3) return comb_warp_fast_smem<24>(Pw, cc, scratch);
+  else if constexpr (NW == 4) return comb_warp_fast_smem<96>(Pw, cc, scratch);
+  else if constexpr (NW == 5)
+    return comb_warp_fast_smem<24, CombReg::kM, CombReg::kD>(Pw, cc, scratch);
+  else if constexpr (NW == 6)
+    return comb_warp_fast_smem<96, CombReg::kM, CombReg::kD>(Pw, cc, scratch);
   else return comb_warp_generic<NW>(Pw, cc, scratch);
 }
 

@@ -16,11 +16,11 @@ namespace ddhf {
 // comb_warp; with spec_smem = 0 (real input only: the register form on
 // 16-byte aligned rows, or the generic comb on a spectrum too large for
 // shared memory) comb_warp reads the row in global memory and shared memory
-// holds its scratch alone. 4 warps per block; the register form of the fast variant is held
-// to 80 registers (6 blocks, 24 warps per SM; its 7.4 KB of shared memory per
-// warp at 750 bins would allow 7), the shared-memory form to 64.
+// holds its scratch alone. Up to 4 warps per block; the fast variant's forms
+// are held to 80 registers (24 warps per SM; the register form's 7.4 KB of
+// shared memory per warp at 750 bins would allow 28).
 template <int NW, bool CPLX>
-__global__ void __launch_bounds__(128, NW == 2 ? 6 : (NW == 3 ? 8 : 1)) k_comb(const float *__restrict__ P, int64_t ld, int64_t cap_px,
+__global__ void __launch_bounds__(128, NW == 2 ? 6 : (NW == 3 || NW == 5 ? 6 : 1)) k_comb(const float *__restrict__ P, int64_t ld, int64_t cap_px,
                        const uint32_t *__restrict__ active, const uint64_t *__restrict__ counters,
                        unsigned long long *cursor, CombConst cc, float *log_sf, float *snr,
                        int32_t *f0, uint8_t *mask, int warp_bytes, int spec_smem, uint32_t *flags) {
@@ -145,12 +145,21 @@ ddhf_status launch_comb_t(Ctx *c, const float *P, int64_t cap_px, float *log_sf,
   while (spec_smem && wpb > 1 && (spec_b + scratch_b) * wpb > max_smem) wpb >>= 1;
   if (spec_smem && (spec_b + scratch_b) * wpb > max_smem) {
     spec_smem = 0;
-    if (CPLX || scratch_b > max_smem) {
+    if (CPLX || scratch_b > max_smem || (variant >= 3 && variant <= 6)) {
       c->last_error = "comb scratch does not fit in shared memory for this grid and comb";
       return DDHF_ERR_UNSUPPORTED;
     }
   }
   const int warp_bytes = (spec_smem ? spec_b : 0) + scratch_b;
+  // fewer warps per block when more warps then share an SM's memory (19 KB per
+  // warp at 2000 bins: 2 blocks of 4, 5 of 2)
+  int sm_smem = 0;
+  DDHF_CUDA_TRY(c, cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor,
+                                          c->device));
+  for (int w = wpb >> 1; w >= 1; w >>= 1)
+    if (sm_smem / (warp_bytes * w + 1024) * w > sm_smem / (warp_bytes * wpb + 1024) * wpb &&
+        sm_smem / (warp_bytes * wpb + 1024) * wpb < 16)
+      wpb = w;
   const size_t smem = (size_t)warp_bytes * wpb;
   DDHF_CUDA_TRY(c, cudaMemsetAsync(mask, 0, c->npx, s));
   // the pixel counter of this launch: word 6 of the slot's counters (unused
@@ -174,6 +183,9 @@ ddhf_status launch_comb_t(Ctx *c, const float *P, int64_t cap_px, float *log_sf,
   }
   if (variant == 2) DDHF_COMB_CASE(2)
   else if (variant == 3) DDHF_COMB_CASE(3)
+  else if (variant == 4) DDHF_COMB_CASE(4)
+  else if (variant == 5) DDHF_COMB_CASE(5)
+  else if (variant == 6) DDHF_COMB_CASE(6)
   else if (variant == 1) DDHF_COMB_CASE(1)
   else DDHF_COMB_CASE(8)
 #undef DDHF_COMB_CASE
