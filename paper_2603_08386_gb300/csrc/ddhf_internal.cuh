@@ -295,6 +295,19 @@ __device__ __forceinline__ float2 phasor_of_residue(uint64_t r, float two_over_d
   return make_float2(c, -s);
 }
 
+// e^{-2 pi i phi}, phi given as the top 32 bits of a 64-bit fraction of a turn:
+// split into the nearest quarter turn and a signed remainder of at most 1/8
+// turn, which converts to FP32 with an absolute error below 2^-28 of a turn.
+__device__ __forceinline__ float2 phasor_of_turn32(uint32_t turn) {
+  const uint32_t q = (turn + 0x20000000u) >> 30;
+  const int32_t rem = (int32_t)(turn - (q << 30));
+  float sy, cy;
+  sincospi_reduced(__fmul_rn((float)rem, 0x1p-31f), sy, cy);
+  const float a = (q & 1u) ? sy : cy, b = (q & 1u) ? cy : sy;
+  return make_float2(__uint_as_float(__float_as_uint(a) ^ (((q + 1u) & 2u) << 30)),
+                     __uint_as_float(__float_as_uint(b) ^ (((q & 2u) ^ 2u) << 30)));
+}
+
 // Complex product with a fixed rounding sequence (no compiler contraction), so
 // every kernel that generates the same phasors gets the same bits.
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {

@@ -102,18 +102,8 @@ inline NdftConst make_ndft_const(const GridConst &g, int mt) {
 __device__ __forceinline__ void raise_flag(uint32_t *flags, uint32_t f) { atomicOr(flags, f); }
 
 // e^{-2 pi i phi}, phi = f tau as a fraction of a turn (f in units of 2^-64).
-// The turn's top 32 bits are split into the nearest quarter turn and a signed
-// remainder of at most 1/8 turn, which converts to FP32 with an absolute error
-// below 2^-28 of a turn.
 __device__ __forceinline__ float2 phasor_of_turn(uint64_t f, uint32_t tau) {
-  const uint32_t turn = __umulhi((uint32_t)f, tau) + (uint32_t)(f >> 32) * tau;
-  const uint32_t q = (turn + 0x20000000u) >> 30;
-  const int32_t rem = (int32_t)(turn - (q << 30));
-  float sy, cy;
-  sincospi_reduced(__fmul_rn((float)rem, 0x1p-31f), sy, cy);
-  const float a = (q & 1u) ? sy : cy, b = (q & 1u) ? cy : sy;
-  return make_float2(__uint_as_float(__float_as_uint(a) ^ (((q + 1u) & 2u) << 30)),
-                     __uint_as_float(__float_as_uint(b) ^ (((q & 2u) ^ 2u) << 30)));
+  return phasor_of_turn32(__umulhi((uint32_t)f, tau) + (uint32_t)(f >> 32) * tau);
 }
 
 // x = hi + lo as two FP16 values, hi in the low half: hi is x cut to 11
