@@ -78,6 +78,7 @@ struct CombConst {
   float ln_tau_sf;  // log(tau_sf) in FP32
   float tau_comb;
   float inv_N;      // 1 / N in FP32
+  int32_t ib;       // bits of a bin index in the comb's sort keys
 };
 
 struct GridConst {
@@ -261,10 +262,12 @@ __device__ __forceinline__ uint64_t mod_barrett(uint64_t x, uint64_t D, uint64_t
 // rint does), whose float bits then hold q mod 4 in their lowest bits, so
 // no conversion runs on the special-function pipe.
 // Error within 2 ulp of the exact values (checked against sincospif).
+// QUARTER: |x| <= 1/4 already (q = 0).
+template <bool QUARTER = false>
 __device__ __forceinline__ void sincospi_reduced(float x, float &s, float &c) {
   const float mq = __fadd_rn(__fmul_rn(2.f, x), 0x1.8p23f);
   const float q = __fsub_rn(mq, 0x1.8p23f);
-  const float y = __fmaf_rn(-0.5f, q, x);
+  const float y = QUARTER ? x : __fmaf_rn(-0.5f, q, x);
   const float t = __fmul_rn(y, y);
   float p = 0.0810556039f;
   p = __fmaf_rn(p, t, -0.599208117f);
@@ -277,6 +280,11 @@ __device__ __forceinline__ void sincospi_reduced(float x, float &s, float &c) {
   k = __fmaf_rn(k, t, 4.05870819f);
   k = __fmaf_rn(k, t, -4.93480206f);
   const float cy = __fmaf_rn(k, t, 1.f);
+  if (QUARTER) {
+    s = sy;
+    c = cy;
+    return;
+  }
   const int iq = __float_as_int(mq) & 3;  // 0: (sy, cy), 1: (cy, -sy), 2: (-sy, -cy), 3: (-cy, sy)
   const float s0 = (iq & 1) ? cy : sy, c0 = (iq & 1) ? sy : cy;
   s = (iq & 2) ? -s0 : s0;
@@ -302,7 +310,7 @@ __device__ __forceinline__ float2 phasor_of_turn32(uint32_t turn) {
   const uint32_t q = (turn + 0x20000000u) >> 30;
   const int32_t rem = (int32_t)(turn - (q << 30));
   float sy, cy;
-  sincospi_reduced(__fmul_rn((float)rem, 0x1p-31f), sy, cy);
+  sincospi_reduced<true>(__fmul_rn((float)rem, 0x1p-31f), sy, cy);
   const float a = (q & 1u) ? sy : cy, b = (q & 1u) ? cy : sy;
   return make_float2(__uint_as_float(__float_as_uint(a) ^ (((q + 1u) & 2u) << 30)),
                      __uint_as_float(__float_as_uint(b) ^ (((q & 2u) ^ 2u) << 30)));

@@ -36,8 +36,9 @@
 // before it, with its longer rotation chains: 8.1e-7 and 1.3e-6).
 //
 // Measured (one 1280x720 window of 19.9M events, 750 bins, default tuning):
-// 2.58 -> 1.55 ms (FMA pipe -> issue 65 %, tensor pipe 32 %, 1,227 warp
-// instructions per pixel); 640x480 at 2000 bins 1.79 -> 0.99 ms.
+// 2.58 -> 1.49 ms (issue 61 % at 16 warps per SM, tensor pipe 34 %, 1,095 warp
+// instructions per pixel; 1.55 ms and 1,227 before the rotation chains were
+// paired); 640x480 at 2000 bins 1.79 -> 0.99 ms.
 //
 // Bins whose frequency is a multiple of D (in practice bin 0 of a grid that
 // starts at 0 Hz) have the phase 0 for every event: their power is the squared
@@ -106,15 +107,31 @@ __device__ __forceinline__ float2 phasor_of_turn(uint64_t f, uint32_t tau) {
   return phasor_of_turn32(__umulhi((uint32_t)f, tau) + (uint32_t)(f >> 32) * tau);
 }
 
-// x = hi + lo as two FP16 values, hi in the low half: hi is x cut to 11
-// significant bits, lo the rest rounded to FP16.
-__device__ __forceinline__ uint32_t split_half2(float x) {
-  const float hi = __uint_as_float(__float_as_uint(x) & 0xffffe000u);
-  const float lo = __fsub_rn(x, hi);
-  uint32_t w;
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(lo), "f"(hi));
-  return w;
+// Each element of v (|v| <= 1) as two FP16 values, hi in the low half of its
+// word: hi is v rounded to a multiple of 2^-11 (exact in FP16), lo the rest
+// (|lo| <= 2^-12) rounded to FP16.
+__device__ __forceinline__ void split_half2(float2 v, uint32_t &wx, uint32_t &wy) {
+  const float2 m = make_float2(6144.f, 6144.f), nm = make_float2(-6144.f, -6144.f);
+  const float2 hi = __fadd2_rn(__fadd2_rn(v, m), nm);
+  const float2 lo = __ffma2_rn(hi, make_float2(-1.f, -1.f), v);
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(wx) : "f"(lo.x), "f"(hi.x));
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(wy) : "f"(lo.y), "f"(hi.y));
 }
+
+// Two rotation chains in paired FP32 instructions (each element rounded as
+// cmul rounds it): `up` steps by r, `dn` by its conjugate.
+struct ChainPair {
+  float2 x, y;          // (up, dn) real and imaginary parts
+  float2 rx, ry, nry;   // (rx, rx), (ry, -ry), (-ry, ry)
+  __device__ __forceinline__ ChainPair(float2 up, float2 dn, float2 r)
+      : x(make_float2(up.x, dn.x)), y(make_float2(up.y, dn.y)), rx(make_float2(r.x, r.x)),
+        ry(make_float2(r.y, -r.y)), nry(make_float2(-r.y, r.y)) {}
+  __device__ __forceinline__ void step() {
+    const float2 a = __fmul2_rn(y, nry), b = __fmul2_rn(y, rx);
+    y = __ffma2_rn(x, ry, b);
+    x = __ffma2_rn(x, rx, a);
+  }
+};
 
 // Shared-memory layout of one warp's staged factors, per event: B (32 columns)
 // as eight 16-byte units of four words, A as one such array per two m-tiles and
@@ -145,23 +162,19 @@ __device__ __forceinline__ void gen_chunk(uint32_t w, const NdftConst &nd, uint6
                                           unsigned char *stage) {
   const int e = threadIdx.x & 31;
   const uint32_t tau = w & 0x7fffffffu, sg = w & kSignBit;
-  const float2 u = phasor_of_turn(nd.f_u, tau);
-  const float2 uc = make_float2(u.x, -u.y);
   // columns: k = 8 exact, 9..15 and 7..0 by rotation
   {
-    float2 up = phasor_of_turn(nd.f_k8, tau), dn = up;
+    const float2 u = phasor_of_turn(nd.f_u, tau), k8 = phasor_of_turn(nd.f_k8, tau);
+    ChainPair z(k8, cmul(k8, make_float2(u.x, -u.y)), u);
     uint4 *b = reinterpret_cast<uint4 *>(stage + Stage<MT>::kB + e * 144);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       uint32_t c[4], d[4], c2[4], d2[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        if (h + i > 0) up = cmul(up, u);
-        c[i] = split_half2(up.x);  // k = 8 + 4 h + i
-        d[i] = split_half2(up.y);
-        dn = cmul(dn, uc);
-        c2[3 - i] = split_half2(dn.x);  // k = 7 - 4 h - i
-        d2[3 - i] = split_half2(dn.y);
+        if (h + i > 0) z.step();
+        split_half2(z.x, c[i], c2[3 - i]);  // k = 8 + 4 h + i and 7 - 4 h - i
+        split_half2(z.y, d[i], d2[3 - i]);
       }
       b[2 + h] = make_uint4(c[0], c[1], c[2], c[3]);
       b[6 + h] = make_uint4(d[0], d[1], d[2], d[3]);
@@ -172,22 +185,19 @@ __device__ __forceinline__ void gen_chunk(uint32_t w, const NdftConst &nd, uint6
   // rows: 4 MT exact (the polarity's sign on it), the others by rotation
   {
     const float2 v = phasor_of_turn(nd.f_v, tau);
-    const float2 vc = make_float2(v.x, -v.y);
-    float2 up = phasor_of_turn(f_row, tau);
-    up.x = __uint_as_float(__float_as_uint(up.x) ^ sg);
-    up.y = __uint_as_float(__float_as_uint(up.y) ^ sg);
-    float2 dn = up;
+    float2 s = phasor_of_turn(f_row, tau);
+    s.x = __uint_as_float(__float_as_uint(s.x) ^ sg);
+    s.y = __uint_as_float(__float_as_uint(s.y) ^ sg);
+    ChainPair z(s, cmul(s, make_float2(v.x, -v.y)), v);
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
       uint32_t r[2 * MT], r2[2 * MT];
 #pragma unroll
       for (int i = 0; i < MT; ++i) {
-        if (h + i > 0) up = cmul(up, v);
-        r[2 * i] = split_half2(up.x);  // row MT (4 + h) + i
-        r[2 * i + 1] = split_half2(up.y);
-        dn = cmul(dn, vc);
-        r2[2 * (MT - 1 - i)] = split_half2(dn.x);  // row MT (3 - h) + MT - 1 - i
-        r2[2 * (MT - 1 - i) + 1] = split_half2(dn.y);
+        if (h + i > 0) z.step();
+        // rows MT (4 + h) + i and MT (3 - h) + MT - 1 - i
+        split_half2(z.x, r[2 * i], r2[2 * (MT - 1 - i)]);
+        split_half2(z.y, r[2 * i + 1], r2[2 * (MT - 1 - i) + 1]);
       }
       const int gu = 4 + h, gd = 3 - h;
 #pragma unroll
@@ -241,22 +251,35 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
         "f"(c[2]), "f"(c[3]));
 }
 
-// Staged events q .. q + m - 1 (m <= 8, q + m <= 32) into the accumulators. A
-// pixel's events enter in groups of 8 counted from its first one, whatever the
-// chunk they were staged in, so its sums do not depend on how the work is split.
-template <int MT>
+// Staged events q .. q + m - 1 (m <= 8, q + m <= 32) into the accumulators
+// (FIRST: which take their values instead of adding them). A pixel's events
+// enter in groups of 8 counted from its first one, whatever the chunk they were
+// staged in, so its sums do not depend on how the work is split.
+//
+// A word of A against the same event's word of B gives hi hi + lo lo, against
+// the word with its halves swapped hi lo + lo hi. The tensor core cuts its sums
+// off instead of rounding them, so a long chain of steps through one accumulator
+// drifts towards zero (1.5e-5 of the spectra at 2000 bins, 25 times the FP32
+// product's error): each group is summed on its own (the small products first)
+// and added to the accumulators in FP32.
+template <int MT, bool FIRST>
 __device__ __forceinline__ void mma_group(int q, int m, const unsigned char *stage, Acc<MT> &acc) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int e0 = min(q + t, kGenChunk - 1), e1 = min(q + t + 4, kGenChunk - 1);
-  const unsigned char *sb = stage + Stage<MT>::kB + 16 * unit16(g);
-  uint4 b0 = *reinterpret_cast<const uint4 *>(sb + e0 * 144);
-  uint4 b1 = *reinterpret_cast<const uint4 *>(sb + e1 * 144);
+  int e0 = q + t, e1 = q + t + 4;
+  if (m < kGroup) {  // a slot past the chunk
+    e0 = min(e0, kGenChunk - 1);
+    e1 = min(e1, kGenChunk - 1);
+  }
+  const unsigned char *s0 = stage + 16 * unit16(g) + e0 * 144;
+  const unsigned char *s1 = stage + 16 * unit16(g) + e1 * 144;
+  uint4 b0 = *reinterpret_cast<const uint4 *>(s0 + Stage<MT>::kB);
+  uint4 b1 = *reinterpret_cast<const uint4 *>(s1 + Stage<MT>::kB);
   uint32_t a[MT][4];
 #pragma unroll
   for (int p = 0; p < Stage<MT>::kPairs; ++p) {
-    const unsigned char *sa = stage + Stage<MT>::kA + p * Stage<MT>::kArray + 16 * unit16(g);
-    const uint4 x = *reinterpret_cast<const uint4 *>(sa + e0 * 144);
-    const uint4 y = *reinterpret_cast<const uint4 *>(sa + e1 * 144);
+    const int o = Stage<MT>::kA + p * Stage<MT>::kArray;
+    const uint4 x = *reinterpret_cast<const uint4 *>(s0 + o);
+    const uint4 y = *reinterpret_cast<const uint4 *>(s1 + o);
     a[2 * p][0] = x.x, a[2 * p][1] = x.y, a[2 * p][2] = y.x, a[2 * p][3] = y.y;
     a[2 * p + 1][0] = x.z, a[2 * p + 1][1] = x.w, a[2 * p + 1][2] = y.z, a[2 * p + 1][3] = y.w;
   }
@@ -270,29 +293,27 @@ __device__ __forceinline__ void mma_group(int q, int m, const unsigned char *sta
     if (t >= m) b0 = make_uint4(0u, 0u, 0u, 0u);
     if (t + 4 >= m) b1 = make_uint4(0u, 0u, 0u, 0u);
   }
-  // The tensor core cuts its sums off instead of rounding them, so a long chain
-  // of steps through one accumulator drifts towards zero (1.5e-5 of the spectra
-  // at 2000 bins, 25 times the FP32 product's error). Each group is summed on
-  // its own (against lo of B, then hi) and added to the accumulators in FP32.
   const uint32_t w0[4] = {b0.x, b0.y, b0.z, b0.w}, w1[4] = {b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    const uint32_t l0 = __byte_perm(w0[c], 0u, 0x3232u), l1 = __byte_perm(w1[c], 0u, 0x3232u);
-    const uint32_t h0 = __byte_perm(w0[c], 0u, 0x1010u), h1 = __byte_perm(w1[c], 0u, 0x1010u);
+    const uint32_t x0 = __byte_perm(w0[c], 0u, 0x1032u), x1 = __byte_perm(w1[c], 0u, 0x1032u);
     float d[MT][4];
     const float zero[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int i = 0; i < MT; ++i) mma16816(d[i], a[i], l0, l1, zero);
+    for (int i = 0; i < MT; ++i) mma16816(d[i], a[i], x0, x1, zero);
 #pragma unroll
-    for (int i = 0; i < MT; ++i) mma16816(d[i], a[i], h0, h1, d[i]);
+    for (int i = 0; i < MT; ++i) mma16816(FIRST ? acc.x[i][c] : d[i], a[i], w0[c], w1[c], d[i]);
+    if (!FIRST) {
 #pragma unroll
-    for (int i = 0; i < MT; ++i) {
-      float *x = acc.x[i][c];
+      for (int i = 0; i < MT; ++i) {
+        float *x = acc.x[i][c];
 #pragma unroll
-      for (int k = 0; k < 4; k += 2) {
-        const float2 r = __fadd2_rn(make_float2(x[k], x[k + 1]), make_float2(d[i][k], d[i][k + 1]));
-        x[k] = r.x;
-        x[k + 1] = r.y;
+        for (int k = 0; k < 4; k += 2) {
+          const float2 r =
+              __fadd2_rn(make_float2(x[k], x[k + 1]), make_float2(d[i][k], d[i][k + 1]));
+          x[k] = r.x;
+          x[k + 1] = r.y;
+        }
       }
     }
   }
@@ -357,18 +378,20 @@ __device__ __forceinline__ void store_tile(const BlockedArgs &A, const Acc<MT> &
                                            int b0, int sum_p) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   float *dst = A.P + prow * A.ld;
+  const int row = b0 + MT * g, whole = A.vec_store ? A.N >> 5 : 0;  // rows below it: 16-byte stores
+  float *up = dst + 32 * row + 16 + 4 * t, *dn = dst + 32 * row + 12 - 4 * t;
 #pragma unroll
   for (int i = 0; i < MT; ++i) {
     float pv[2][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc.powers(i, q, pv[1][q], pv[0][3 - q]);
+    if (row + i < whole) {
+      *reinterpret_cast<float4 *>(up + 32 * i) = make_float4(pv[1][0], pv[1][1], pv[1][2], pv[1][3]);
+      *reinterpret_cast<float4 *>(dn + 32 * i) = make_float4(pv[0][0], pv[0][1], pv[0][2], pv[0][3]);
+    } else {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int j = 32 * (b0 + MT * g + i) + (h ? 16 + 4 * t : 12 - 4 * t);
-      if (A.vec_store && j + 3 < A.N) {
-        *reinterpret_cast<float4 *>(dst + j) =
-            make_float4(pv[h][0], pv[h][1], pv[h][2], pv[h][3]);
-      } else {
+      for (int h = 0; h < 2; ++h) {
+        const int j = 32 * (row + i) + (h ? 16 + 4 * t : 12 - 4 * t);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
           if (j + q < A.N) dst[j + q] = pv[h][q];
@@ -394,7 +417,7 @@ __device__ __forceinline__ int accumulate(const uint32_t *__restrict__ evp, int 
     __syncwarp();
     const int c1 = c0 + step * kGenChunk;  // the next chunk's event word, loaded ahead
     w = c1 + lane < cnt ? evp[c1 + lane] : 0u;
-    for (int q = 0; q < ne; q += kGroup) mma_group<MT>(q, min(kGroup, ne - q), stage, acc);
+    for (int q = 0; q < ne; q += kGroup) mma_group<MT, false>(q, min(kGroup, ne - q), stage, acc);
     __syncwarp();
   }
   return neg;
@@ -477,13 +500,14 @@ __device__ __forceinline__ void light_stream(const BlockedArgs &A, unsigned char
         // the staged chunk holds events [c0, c0 + 32) of the run (c0 = ~0: none
         // yet), words wc; wn: the 32 words after them; sgn: their signs
         uint32_t c0 = 0xffffffffu, wc = 0, wn = 0, sgn = 0;
+        const bool has_dc = A.nd.dc_first >= 0 && A.nd.dc_first < 32 * (b0 + 8 * MT);
         for (uint32_t rem = sub; rem; rem &= rem - 1) {
           const int p = __ffs(rem) - 1;
           const uint32_t pe0 = __shfl_sync(0xffffffffu, q_lo, p);
           const uint32_t pe1 = __shfl_sync(0xffffffffu, q_hi, p);
           Acc<MT> acc;
-          acc.zero();
           int neg = 0;
+          if (pe0 >= pe1) acc.zero();
           for (uint32_t pos = pe0; pos < pe1; pos += kGroup) {
             const int m = (int)min((uint32_t)kGroup, pe1 - pos);
             uint32_t d = pos - c0;
@@ -503,8 +527,9 @@ __device__ __forceinline__ void light_stream(const BlockedArgs &A, unsigned char
               __syncwarp();
               wn = pos + 32u + lane < e_end ? v.ev[pos + 32u + lane] : 0u;
             }
-            neg += __popc((sgn >> d) & (0xffu >> (kGroup - m)));
-            mma_group<MT>((int)d, m, stage, acc);
+            if (has_dc) neg += __popc((sgn >> d) & (0xffu >> (kGroup - m)));
+            if (pos == pe0) mma_group<MT, true>((int)d, m, stage, acc);
+            else mma_group<MT, false>((int)d, m, stage, acc);
           }
           store_tile<MT>(A, acc, (int64_t)a0 + p, b0, (int)(pe1 - pe0) - 2 * neg);
         }
