@@ -227,6 +227,9 @@ void derive_constants(Ctx *c) {
   cc.ln_tau_sf = (float)log((double)p.tau_sf);
   cc.inv_N = (float)(1.0 / (double)N);
   cc.tau_comb = p.tau_comb;
+  // a short index leaves the values more bits: the 30 middle ranks of a short
+  // spectrum span more of its range
+  cc.ib = std::max(7, ceil_log2(N));
 }
 
 ddhf_status check_params(const ddhf_params *p) {

@@ -474,8 +474,9 @@ __device__ __forceinline__ CombOut comb_warp_generic(const float *Pw, const Comb
 //  * the buckets holding ranks lo_r and hi_r bound the candidate bins; at
 //    most 64 candidates (about 31 on C3's spectra) are compacted into shared
 //    memory and sorted in registers as 32-bit keys (value bits relative to
-//    the smallest candidate, above a bin index of 10 to 14 bits), so that lane
-//    p holds the bin of full rank lo_r + p;
+//    the smallest candidate, above a bin index of 7 to 14 bits; 64-bit keys
+//    when the values span more), so that lane p holds the bin of full rank
+//    lo_r + p;
 //  * one window maximum per centre (Eq. 8), then N(w) for every candidate,
 //    kept in shared memory;
 //  * candidates are evaluated one at a time by the whole warp: lane i <
@@ -495,9 +496,8 @@ __device__ __forceinline__ CombOut comb_warp_generic(const float *Pw, const Comb
 // bins in registers, so every per-bin pass is a fixed, fully unrolled
 // sequence and the window maxima come from registers and six shuffles. The
 // shared-memory form takes any other size within the limits.
-// Pixels whose candidates do not fit (more than 64, or a value range that the
-// key has no room for: 2^22 ulps up to 1024 bins) take an exact radix selection
-// of the band instead.
+// Pixels with more than 64 candidates (crowded middle ranks) take an exact
+// radix selection of the band instead.
 // Scratch (bytes from the scratch base, 16-byte aligned), HB = the histogram's
 // bytes (4 per bucket):
 //   [0, HB)     histogram; once the band's buckets are located, over it:
@@ -525,10 +525,6 @@ struct CombFast {
   }
   static constexpr int kMaxBand = 32;
   static constexpr int kMaxCand = 64;
-  // bits of a bin index in a candidate's sort key
-  __host__ __device__ static int index_bits(int N) {
-    return N <= 1024 ? 10 : N <= 2048 ? 11 : N <= 4096 ? 12 : N <= 8192 ? 13 : 14;
-  }
 };
 
 // The register form's shape: bins per lane, and the comb it is written for.
@@ -611,14 +607,34 @@ __device__ __forceinline__ uint64_t warp_sort32_u64(uint64_t v) {
 }
 
 // The band of full ranks [lo_r, hi_r] (bw <= 32 ranks) of Pw[0..N) in the
-// (value, index) order, exactly, by radix selection of its two ends: lane p
-// gets the value bits and bin of rank lo_r + p. Returns true when the count
-// found disagrees with bw (an internal error). Kept out of line: it runs only
-// for spectra whose middle ranks the histogram cannot separate.
+// (value, index) order, exactly: lane p gets the value bits and bin of rank lo_r
+// + p. With ncand > 0 from that many compacted candidates (over the histogram),
+// sorted as 64-bit keys, element `first` being rank lo_r: their values are too
+// far apart for 32-bit keys (at 100 bins the 30 middle ranks span more than a
+// factor of two: 76,800 such spectra 0.70 -> 0.22 ms). Otherwise, for spectra
+// whose middle ranks the histogram cannot separate, by radix selection of the
+// band's two ends. Returns true when the count found disagrees with bw (an
+// internal error). Kept out of line: it runs only for some spectra.
 __device__ __noinline__ static bool comb_band_exact(const float *Pw, int N, int lo_r, int hi_r,
-                                                    int bw, uint32_t *hist, uint32_t &bv_bits,
-                                                    int &bj) {
+                                                    int bw, uint32_t *hist, int ncand,
+                                                    int first, uint32_t &bv_bits, int &bj) {
   const int lane = threadIdx.x & 31;
+  if (ncand > 0) {
+    const unsigned char *sc = reinterpret_cast<const unsigned char *>(hist);
+    const uint32_t *cv = reinterpret_cast<const uint32_t *>(sc + CombFast::kCandV);
+    const uint16_t *cj = reinterpret_cast<const uint16_t *>(sc + CombFast::kCandJ);
+    uint64_t k0 = lane < ncand ? ((uint64_t)cv[lane] << 16) | cj[lane] : ~0ull;
+    uint64_t k1 = lane + 32 < ncand ? ((uint64_t)cv[lane + 32] << 16) | cj[lane + 32] : ~0ull;
+    if (ncand <= 32) k0 = warp_sort32_u64(k0);
+    else warp_sort64_regs(k0, k1);
+    const int i = first + lane;
+    const uint64_t a = __shfl_sync(0xffffffffu, k0, i & 31);
+    const uint64_t b = __shfl_sync(0xffffffffu, k1, i & 31);
+    const uint64_t k = i < 32 ? a : b;
+    bv_bits = (uint32_t)(k >> 16);
+    bj = (int)(k & 0xFFFFu);
+    return false;
+  }
   const uint32_t lt = lanemask_lt();
   const uint64_t klo = select_rank_slow(Pw, N, lo_r, hist);
   const uint64_t khi = select_rank_slow(Pw, N, hi_r, hist);
@@ -651,8 +667,55 @@ __device__ __forceinline__ bool below_band(float v, int j, float T, int tj) {
   return v < T || (v == T && j < tj);
 }
 
-// Window maxima rec[c] = max of P over [c - d, c + d] for any half-width d;
-// out of line (the d = 3 case has inline versions).
+// Window maxima rec[c] = max of P over [c - D, c + D], centre quads 4q .. 4q + 3
+// from the bins 4q - 4 .. 4q + 7 by three 16-byte loads (D <= 4).
+template <int D>
+__device__ __forceinline__ void comb_records_quads(const float *Pw, int N, float *rec) {
+  const int lane = threadIdx.x & 31;
+  const int nfull = N >> 2, ng = (N + 3) >> 2;
+  const float4 *P4 = reinterpret_cast<const float4 *>(Pw);
+  for (int q = lane; q < ng; q += 32) {
+    float b[12];  // b[i] = P[4q - 4 + i]
+    if (q >= 1 && q + 1 < nfull) {
+      const float4 x = P4[q - 1], y = P4[q], z = P4[q + 1];
+      b[0] = x.x; b[1] = x.y; b[2] = x.z; b[3] = x.w;
+      b[4] = y.x; b[5] = y.y; b[6] = y.z; b[7] = y.w;
+      b[8] = z.x; b[9] = z.y; b[10] = z.z; b[11] = z.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 12; ++i) {
+        const int j = 4 * q - 4 + i;
+        b[i] = (j >= 0 && j < N) ? Pw[j] : 0.f;
+      }
+    }
+    float wv[4];
+    if (D == 3) {  // every centre's window holds the quad
+      const float mid = fmaxf(fmaxf(b[4], b[5]), fmaxf(b[6], b[7]));  // 4q .. 4q+3
+      const float l1 = fmaxf(b[2], b[3]), r1 = fmaxf(b[8], b[9]);
+      wv[0] = fmaxf(mid, fmaxf(b[1], l1));   // 4q-3 .. 4q+3
+      wv[1] = fmaxf(mid, fmaxf(l1, b[8]));   // 4q-2 .. 4q+4
+      wv[2] = fmaxf(mid, fmaxf(b[3], r1));   // 4q-1 .. 4q+5
+      wv[3] = fmaxf(mid, fmaxf(r1, b[10]));  // 4q   .. 4q+6
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        wv[u] = b[4 + u - D];
+#pragma unroll
+        for (int i = 1; i <= 2 * D; ++i) wv[u] = fmaxf(wv[u], b[4 + u - D + i]);
+      }
+    }
+    if (q < nfull) {
+      reinterpret_cast<float4 *>(rec)[q] = make_float4(wv[0], wv[1], wv[2], wv[3]);
+    } else {  // the partial last quad
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (4 * q + u < N) rec[4 * q + u] = wv[u];
+    }
+  }
+}
+
+// Window maxima rec[c] = max of P over [c - d, c + d] for any half-width d; out
+// of line.
 __device__ __noinline__ static void comb_records_any_d(const float *Pw, int N, int d,
                                                        float *rec) {
   const int lane = threadIdx.x & 31;
@@ -697,25 +760,13 @@ __device__ __forceinline__ int comb_mvalid(int w, int M, int L) {
   return mv;
 }
 
-// N(w) of Eq. 8 from the window maxima, or -1 when w's complement is empty
-// (KM, KD: the comb's M and d when known at compile time, else 0).
-template <int KM, int KD>
-__device__ __forceinline__ float comb_cand_nw(const float *rec, int w, const CombConst &cc,
-                                              bool uniform) {
-  const int M = KM ? KM : cc.M, d = KD ? KD : cc.d, N = cc.N;
-  const int L = N - 1 - d;
-  const int mv = uniform ? M : comb_mvalid(w, M, L);
-  const int h = w >= 2 * d + 1 ? mv * (2 * d + 1) : (mv - 1) * w + 2 * d + 1;
-  if (N - h <= 0) return -1.f;
-  float s = rec[w];  // 0 + m_1, exact
-  if (KM && uniform) {
-#pragma unroll
-    for (int m = 2; m <= KM; ++m) s = __fadd_rn(s, rec[m * w]);
-    return comb_nw(s, KM);
-  }
-#pragma unroll 4
-  for (int m = 2; m <= mv; ++m) s = __fadd_rn(s, rec[m * w]);
-  return comb_nw(s, mv);
+// s / m correctly rounded for an integer m <= 32, r = 1 / m correctly rounded: one
+// product and one exact remainder step (Markstein, IBM J. Res. Dev. 34(1), 1990),
+// where nothing under- or overflows; a division elsewhere.
+__device__ __forceinline__ float div_small(float s, float m, float r) {
+  if (s != 0.f && !(s >= 0x1p-100f && s < 0x1p120f)) return __fdiv_rn(s, m);
+  const float q = __fmul_rn(s, r);
+  return __fmaf_rn(__fmaf_rn(-q, m, s), r, q);
 }
 
 // The buckets holding full ranks lo_r and hi_r in the histogram; lane l owns
@@ -793,10 +844,9 @@ __device__ __forceinline__ BandBuckets comb_locate(const uint32_t *hist, int N, 
 }
 
 // The band from the ncand <= 64 compacted candidates (value bits cv, bins
-// cj; element i in lane i % 32, register i / 32): sorted as 32-bit keys,
-// lane p < bw takes full rank lo_r + p (value bv, bin bj). ib: bits of a bin
-// index. Returns false (warp-uniform) when the values span 2^(32 - ib) ulps or
-// more, so that the exact selection must run instead.
+// cj; element i in lane i % 32, register i / 32): sorted as 32-bit keys of ib
+// index bits, lane p < bw takes full rank lo_r + p (value bv, bin bj). Returns
+// false (warp-uniform) when the values span 2^(32 - ib) ulps or more.
 __device__ __forceinline__ bool comb_band_sorted(const unsigned char *scratch, int ncand,
                                                  int lo_r, int cb, int bw, int ib, float &bv,
                                                  int &bj, bool &bad) {
@@ -808,29 +858,30 @@ __device__ __forceinline__ bool comb_band_sorted(const unsigned char *scratch, i
   const uint32_t b1 = in1 ? cv[lane + 32] : 0xFFFFFFFFu;
   const uint32_t mn = __reduce_min_sync(0xffffffffu, min(b0, b1));
   const uint32_t mx = __reduce_max_sync(0xffffffffu, max(in0 ? b0 : 0u, in1 ? b1 : 0u));
+  // band position p is sorted element i = lo_r - cb + p (lane i % 32, register i / 32)
+  const int i = lo_r - cb + lane;
+  if (lane < bw && (i < 0 || i >= ncand)) bad = true;
   if (mx - mn >= (1u << (32 - ib))) return false;
   uint32_t k0 = in0 ? (((b0 - mn) << ib) | (uint32_t)cj[lane]) : 0xFFFFFFFFu;
   uint32_t k1 = in1 ? (((b1 - mn) << ib) | (uint32_t)cj[lane + 32]) : 0xFFFFFFFFu;
   if (ncand <= 32) k0 = warp_sort32_u32(k0);
   else warp_sort64_u32(k0, k1);
-  // band position p is sorted element i = lo_r - cb + p (lane i % 32, register i / 32)
-  const int i = lo_r - cb + lane;
   const uint32_t kk0 = __shfl_sync(0xffffffffu, k0, i & 31);
   const uint32_t kk1 = __shfl_sync(0xffffffffu, k1, i & 31);
   const uint32_t kk = i < 32 ? kk0 : kk1;
-  if (lane < bw && (i < 0 || i >= ncand)) bad = true;
   bv = __uint_as_float((kk >> ib) + mn);
   bj = (int)(kk & ((1u << ib) - 1u));
   return true;
 }
 
-// N(w) of every candidate into nws[], the largest and its candidate index
+// N(w) of every candidate into nws[] (-1: empty complement), the largest and its
+// candidate index
 // (the first of equal maxima; -1 / INT_MAX when every complement is empty).
 // KM, KD > 0 (the register form): the comb's M and d, with every candidate
 // known to have all M windows and a non-empty complement (CombReg::fits).
 template <int KM, int KD>
 __device__ __forceinline__ void comb_nw_all(const float *rec, float *nws, const CombConst &cc,
-                                            bool uniform, float &maxnw, int &maxi) {
+                                            float &maxnw, int &maxi) {
   const int lane = threadIdx.x & 31;
   const int n_cand = cc.w_hi - cc.w_lo + 1;
   maxnw = -1.f;
@@ -855,12 +906,34 @@ __device__ __forceinline__ void comb_nw_all(const float *rec, float *nws, const 
       }
     }
   } else {
-    for (int i = lane; i < n_cand; i += 32) {
-      const float nw = comb_cand_nw<0, 0>(rec, cc.w_lo + i, cc, uniform);
-      nws[i] = nw;
-      if (nw > maxnw) {
-        maxnw = nw;
-        maxi = i;
+    // window maxima added while they are in band (a prefix of m), then divided
+    // by their number; lane m holds 1 / m
+    const int M = cc.M, d = cc.d, L = cc.N - 1 - d, span = 2 * d + 1;
+    const bool may_be_empty = cc.N <= M * span;  // some complement may be empty
+    const float inv = __frcp_rn((float)max(lane, 1));
+    for (int i0 = 0; i0 < n_cand; i0 += 32) {
+      const int i = min(i0 + lane, n_cand - 1);
+      const int w = cc.w_lo + i;
+      float sm = rec[w];  // 0 + m_1, exact
+      int mv = 1;
+#pragma unroll 4
+      for (int c = 2 * w, m = 2; m <= M; ++m, c += w)
+        if (c <= L) {
+          sm = __fadd_rn(sm, rec[c]);
+          mv = m;
+        }
+      const float r = __shfl_sync(0xffffffffu, inv, mv & 31);
+      float nw = mv < 32 ? div_small(sm, (float)mv, r) : comb_nw(sm, mv);
+      if (may_be_empty) {
+        const int h = w >= span ? mv * span : (mv - 1) * w + span;
+        if (cc.N - h <= 0) nw = -1.f;
+      }
+      if (i0 + lane < n_cand) {
+        nws[i] = nw;
+        if (nw > maxnw) {
+          maxnw = nw;
+          maxi = i;
+        }
       }
     }
   }
@@ -972,9 +1045,9 @@ __device__ __forceinline__ CombOut comb_out(float best, int bestw, bool bad, flo
 }
 
 // The shared-memory form (any size within the fast limits; BPL = CombFast::bpl(N);
-// KM, KD > 0: M and d when every candidate has all M windows and a non-empty
+// LOOP: more than 1024 bins; KM, KD > 0: M and d when every candidate has all M windows and a non-empty
 // complement, which halves the instructions of the candidate sums).
-template <int BPL, int KM = 0, int KD = 0>
+template <int BPL, bool LOOP, int KM = 0, int KD = 0>
 __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const CombConst &cc,
                                                        unsigned char *scratch) {
   const int lane = threadIdx.x & 31;
@@ -1042,6 +1115,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
   const int lo_r = cc.lo_r, bw = cc.bw, hi_r = cc.lo_r + cc.bw - 1;
   const BandBuckets bb = comb_locate<BPL>(hist, N, lo_r, hi_r, bad);
   bool slow = bb.ncand > CombFast::kMaxCand || bad;
+  int wide = 0;  // candidates to sort by 64-bit keys
   float bv = 0.f;  // its value
   int bj = 0;      // its bin
   if (!slow) {
@@ -1053,7 +1127,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
     uint32_t run = 0;
     __syncwarp();  // the histogram has been read
 #pragma unroll 1
-    for (int q0 = 0; q0 < ng; q0 += 256) {
+    for (int q0 = 0; q0 < (LOOP ? ng : 1); q0 += 256) {
       uint32_t m = 0;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
@@ -1071,7 +1145,8 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
       uint32_t nsel;
       uint32_t off = run + warp_excl_scan<uint32_t>((uint32_t)__popc(m), nsel);
       run += nsel;
-      while (m && off < (uint32_t)CombFast::kMaxCand) {
+      if (run > (uint32_t)CombFast::kMaxCand) break;  // never: the histogram counted fewer
+      while (m) {
         const int b = __ffs(m) - 1;
         m &= m - 1;
         const int j = 4 * (q0 + lane + 32 * (b >> 2)) + (b & 3);
@@ -1082,16 +1157,17 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
     }
     __syncwarp();
     if ((int)run != bb.ncand) slow = true;  // uniform (a warp total)
-    if (!slow && !comb_band_sorted(scratch, bb.ncand, lo_r, bb.cb, bw, CombFast::index_bits(N),
-                                   bv, bj, bad))
+    if (!slow && !comb_band_sorted(scratch, bb.ncand, lo_r, bb.cb, bw, cc.ib, bv, bj, bad)) {
       slow = true;
+      wide = bb.ncand;
+    }
     __syncwarp();
   }
   if (slow) {
     // exact band [lo_r, hi_r] by radix selection (a rare, out-of-line path)
     uint32_t bvu = 0u;
     __syncwarp();
-    bad |= comb_band_exact(Pw, N, lo_r, hi_r, bw, hist, bvu, bj);
+    bad |= comb_band_exact(Pw, N, lo_r, hi_r, bw, hist, wide, lo_r - bb.cb, bvu, bj);
     bv = __uint_as_float(bvu);
     __syncwarp();
   }
@@ -1101,37 +1177,11 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
   const int d = KD ? KD : cc.d;
   float *rec = reinterpret_cast<float *>(scratch + CombFast::hist_bytes(BPL));
   if (d == 3) {
-    // centre quads 4q .. 4q + 3: bins 4q - 4 .. 4q + 7 by three 16-byte loads
-    for (int q = lane; q < ng; q += 32) {
-      float b[12];  // b[i] = P[4q - 4 + i]
-      if (q >= 1 && q + 1 < nfull) {
-        const float4 x = P4[q - 1], y = P4[q], z = P4[q + 1];
-        b[0] = x.x; b[1] = x.y; b[2] = x.z; b[3] = x.w;
-        b[4] = y.x; b[5] = y.y; b[6] = y.z; b[7] = y.w;
-        b[8] = z.x; b[9] = z.y; b[10] = z.z; b[11] = z.w;
-      } else {
-#pragma unroll
-        for (int i = 0; i < 12; ++i) {
-          const int j = 4 * q - 4 + i;
-          b[i] = (j >= 0 && j < N) ? Pw[j] : 0.f;
-        }
-      }
-      const float mid = fmaxf(fmaxf(b[4], b[5]), fmaxf(b[6], b[7]));  // 4q .. 4q+3
-      const float l1 = fmaxf(b[2], b[3]), r1 = fmaxf(b[8], b[9]);
-      const float w0 = fmaxf(mid, fmaxf(b[1], l1));   // 4q-3 .. 4q+3
-      const float w1 = fmaxf(mid, fmaxf(l1, b[8]));   // 4q-2 .. 4q+4
-      const float w2 = fmaxf(mid, fmaxf(b[3], r1));   // 4q-1 .. 4q+5
-      const float w3 = fmaxf(mid, fmaxf(r1, b[10]));  // 4q   .. 4q+6
-      const int j0 = 4 * q;
-      if (q < nfull) {
-        reinterpret_cast<float4 *>(rec)[q] = make_float4(w0, w1, w2, w3);
-      } else {  // the partial last quad
-        const float wv[4] = {w0, w1, w2, w3};
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (j0 + u < N) rec[j0 + u] = wv[u];
-      }
-    }
+    comb_records_quads<3>(Pw, N, rec);
+  } else if (!KD && d == 2) {
+    comb_records_quads<2>(Pw, N, rec);
+  } else if (!KD && d == 1) {
+    comb_records_quads<1>(Pw, N, rec);
   } else {
     comb_records_any_d(Pw, N, d, rec);
   }
@@ -1144,7 +1194,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
   float *nws = reinterpret_cast<float *>(scratch + CombFast::nw_off(N, cc.w_hi - cc.w_lo + 1));
   float maxnw;
   int maxi;
-  comb_nw_all<KM, KD>(rec, nws, cc, uniform, maxnw, maxi);
+  comb_nw_all<KM, KD>(rec, nws, cc, maxnw, maxi);
   __syncwarp();
   float best;
   int bestw;
@@ -1262,6 +1312,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
   const int lo_r = cc.lo_r, bw = cc.bw, hi_r = cc.lo_r + cc.bw - 1;
   const BandBuckets bb = comb_locate<24>(hist, N, lo_r, hi_r, bad);
   bool slow = bb.ncand > CombFast::kMaxCand || bad;
+  int wide = 0;  // candidates to sort by 64-bit keys
   float bv = 0.f;
   int bj = 0;
   if (!slow) {
@@ -1297,13 +1348,16 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
     }
     __syncwarp();
     if ((int)run != bb.ncand) slow = true;  // uniform (a warp total)
-    if (!slow && !comb_band_sorted(scratch, bb.ncand, lo_r, bb.cb, bw, 10, bv, bj, bad)) slow = true;
+    if (!slow && !comb_band_sorted(scratch, bb.ncand, lo_r, bb.cb, bw, 10, bv, bj, bad)) {
+      slow = true;
+      wide = bb.ncand;
+    }
     __syncwarp();
   }
   if (slow) {
     uint32_t bvu = 0u;
     __syncwarp();
-    bad |= comb_band_exact(Pw, N, lo_r, hi_r, bw, hist, bvu, bj);
+    bad |= comb_band_exact(Pw, N, lo_r, hi_r, bw, hist, wide, lo_r - bb.cb, bvu, bj);
     bv = __uint_as_float(bvu);
     __syncwarp();
   }
@@ -1314,7 +1368,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
   float *nws = reinterpret_cast<float *>(scratch + CombFast::nw_off(N, cc.w_hi - cc.w_lo + 1));
   float maxnw;
   int maxi;
-  comb_nw_all<kM, kD>(rec, nws, cc, uniform, maxnw, maxi);
+  comb_nw_all<kM, kD>(rec, nws, cc, maxnw, maxi);
   __syncwarp();
   float best;
   int bestw;
@@ -1327,16 +1381,16 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
 __device__ __forceinline__ CombOut comb_warp_fast(const float *Pw, const CombConst &cc,
                                                   unsigned char *scratch) {
   if (CombReg::fits(cc)) return comb_warp_fast_regs(Pw, cc, scratch);
-  if (cc.N > CombFast::kManyBins) return comb_warp_fast_smem<96>(Pw, cc, scratch);
-  return comb_warp_fast_smem<24>(Pw, cc, scratch);
+  if (cc.N > CombFast::kManyBins) return comb_warp_fast_smem<96, true>(Pw, cc, scratch);
+  return comb_warp_fast_smem<24, true>(Pw, cc, scratch);
 }
 
 // Which comb variant a context uses: 0 = fast (band <= 32 and M (2d+1) <= 32;
 // the register or shared-memory form, chosen at run time), otherwise the
 // generic one with NW mask words per centre. A kernel that scores every pixel
-// of one context can instead take the fast form itself: 2 = register form, 3 =
-// shared-memory form, 4 = the latter above 4096 bins, 5 and 6 = the same two
-// for Table 2's comb shape (comb_fast_form).
+// of one context can instead take the fast form itself: 2 = register form, 3, 4,
+// 5 = shared-memory form up to 1024 bins, up to 4096 and above, 13, 14, 15 = the
+// same three for Table 2's comb shape (comb_fast_form).
 __host__ __device__ inline int comb_variant(const CombConst &cc) {
   if (cc.bw <= CombFast::kMaxBand && cc.M * (2 * cc.d + 1) <= 32) return 0;
   return cc.bw <= 32 ? 1 : 8;
@@ -1344,11 +1398,12 @@ __host__ __device__ inline int comb_variant(const CombConst &cc) {
 
 __host__ __device__ inline int comb_fast_form(const CombConst &cc) {
   if (CombReg::fits(cc)) return 2;
-  return (cc.N > CombFast::kManyBins ? 4 : 3) + (CombReg::comb_fits(cc) ? 2 : 0);
+  return (cc.N > CombFast::kManyBins ? 5 : cc.N > 1024 ? 4 : 3) +
+         (CombReg::comb_fits(cc) ? 10 : 0);
 }
 
 __host__ __device__ inline int comb_scratch_bytes(const CombConst &cc, int variant) {
-  return (variant == 0 || (variant >= 2 && variant <= 6))
+  return (variant == 0 || (variant >= 2 && variant <= 5) || variant >= 13)
              ? CombFast::bytes(cc.N, cc.w_hi - cc.w_lo + 1)
              : CombScratch::bytes(cc.N, variant);
 }
@@ -1360,12 +1415,12 @@ __device__ __forceinline__ CombOut comb_warp(const float *Pw, const CombConst &c
                                              unsigned char *scratch) {
   if constexpr (NW == 0) return comb_warp_fast(Pw, cc, scratch);
   else if constexpr (NW == 2) return comb_warp_fast_regs(Pw, cc, scratch);
-  else if constexpr (NW == 3) return comb_warp_fast_smem<24>(Pw, cc, scratch);
-  else if constexpr (NW == 4) return comb_warp_fast_smem<96>(Pw, cc, scratch);
-  else if constexpr (NW == 5)
-    return comb_warp_fast_smem<24, CombReg::kM, CombReg::kD>(Pw, cc, scratch);
-  else if constexpr (NW == 6)
-    return comb_warp_fast_smem<96, CombReg::kM, CombReg::kD>(Pw, cc, scratch);
+  else if constexpr ((NW >= 3 && NW <= 5) || NW >= 13) {
+    constexpr bool kTable = NW >= 13;  // Table 2's comb shape
+    constexpr int kSize = kTable ? NW - 10 : NW;
+    return comb_warp_fast_smem<kSize == 5 ? 96 : 24, (kSize > 3), kTable ? CombReg::kM : 0,
+                               kTable ? CombReg::kD : 0>(Pw, cc, scratch);
+  }
   else return comb_warp_generic<NW>(Pw, cc, scratch);
 }
 

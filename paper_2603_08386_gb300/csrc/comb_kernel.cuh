@@ -16,11 +16,12 @@ namespace ddhf {
 // comb_warp; with spec_smem = 0 (real input only: the register form on
 // 16-byte aligned rows, or the generic comb on a spectrum too large for
 // shared memory) comb_warp reads the row in global memory and shared memory
-// holds its scratch alone. Up to 4 warps per block; the fast variant's forms
-// are held to 80 registers (24 warps per SM; the register form's 7.4 KB of
-// shared memory per warp at 750 bins would allow 28).
+// holds its scratch alone. Up to 4 warps per block; the register form is held
+// to 80 registers (24 warps per SM; its 7.4 KB of shared memory per warp at 750
+// bins would allow 28), the shared-memory form to 64 up to 1024 bins and to 80
+// above, where shared memory holds fewer warps.
 template <int NW, bool CPLX>
-__global__ void __launch_bounds__(128, NW == 2 ? 6 : (NW == 3 || NW == 5 ? 6 : 1)) k_comb(const float *__restrict__ P, int64_t ld, int64_t cap_px,
+__global__ void __launch_bounds__(128, NW == 3 || NW == 13 ? 8 : (NW == 2 || NW == 4 || NW == 14 ? 6 : 1)) k_comb(const float *__restrict__ P, int64_t ld, int64_t cap_px,
                        const uint32_t *__restrict__ active, const uint64_t *__restrict__ counters,
                        unsigned long long *cursor, CombConst cc, float *log_sf, float *snr,
                        int32_t *f0, uint8_t *mask, int warp_bytes, int spec_smem, uint32_t *flags) {
@@ -145,7 +146,7 @@ ddhf_status launch_comb_t(Ctx *c, const float *P, int64_t cap_px, float *log_sf,
   while (spec_smem && wpb > 1 && (spec_b + scratch_b) * wpb > max_smem) wpb >>= 1;
   if (spec_smem && (spec_b + scratch_b) * wpb > max_smem) {
     spec_smem = 0;
-    if (CPLX || scratch_b > max_smem || (variant >= 3 && variant <= 6)) {
+    if (CPLX || scratch_b > max_smem || (variant >= 3 && variant <= 5) || variant >= 13) {
       c->last_error = "comb scratch does not fit in shared memory for this grid and comb";
       return DDHF_ERR_UNSUPPORTED;
     }
@@ -185,7 +186,9 @@ ddhf_status launch_comb_t(Ctx *c, const float *P, int64_t cap_px, float *log_sf,
   else if (variant == 3) DDHF_COMB_CASE(3)
   else if (variant == 4) DDHF_COMB_CASE(4)
   else if (variant == 5) DDHF_COMB_CASE(5)
-  else if (variant == 6) DDHF_COMB_CASE(6)
+  else if (variant == 13) DDHF_COMB_CASE(13)
+  else if (variant == 14) DDHF_COMB_CASE(14)
+  else if (variant == 15) DDHF_COMB_CASE(15)
   else if (variant == 1) DDHF_COMB_CASE(1)
   else DDHF_COMB_CASE(8)
 #undef DDHF_COMB_CASE
