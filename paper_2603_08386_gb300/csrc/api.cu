@@ -288,7 +288,7 @@ ddhf_status run_detect(Ctx *c, const ddhf_window *wins, int nw, ddhf_box *boxes,
   if (c->timing) DDHF_CUDA_TRY(c, record_stage(c, 0, s));
   const bool fused = c->tuning.fuse != 0 || !c->pbuf;
   if (fused) {
-    DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, sizeof(uint32_t), s));  // heavy count
+    DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, 2 * sizeof(uint32_t), s));  // heavy and big counts
     for (int w = 0; w < nw; ++w) {
       const ddhf_window &W = wins[w];
       NvtxRange r("ddhf binning");
@@ -316,7 +316,7 @@ ddhf_status run_detect(Ctx *c, const ddhf_window *wins, int nw, ddhf_box *boxes,
       if (we) DDHF_CUDA_TRY(c, record_event(we[0], s));
       {
         NvtxRange r("ddhf binning");
-        DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, sizeof(uint32_t), s));
+        DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, 2 * sizeof(uint32_t), s));
         if (ready) DDHF_CUDA_TRY(c, cudaStreamWaitEvent(s, ready[w], 0));
       DDHF_TRY(bin_into(c, w, W.x, W.y, W.t_us, W.p, W.n, W.t0_us, W.window_us, s));
       }
@@ -349,7 +349,7 @@ ddhf_status run_detect(Ctx *c, const ddhf_window *wins, int nw, ddhf_box *boxes,
       if (we) DDHF_CUDA_TRY(c, record_event(we[0], s));
       {
         NvtxRange r("ddhf binning");
-        DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, sizeof(uint32_t), s));
+        DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, 2 * sizeof(uint32_t), s));
         if (ready) DDHF_CUDA_TRY(c, cudaStreamWaitEvent(s, ready[w], 0));
       DDHF_TRY(bin_into(c, w, W.x, W.y, W.t_us, W.p, W.n, W.t0_us, W.window_us, s));
       }
@@ -667,7 +667,7 @@ ddhf_status ddhf_bin_events(ddhf_ctx *h, const int16_t *x, const int16_t *y, con
   DDHF_TRY(check_window(c, x, y, t_us, p, n, window_us));
   cudaStream_t s = (cudaStream_t)stream;
   c->last_stream = s;
-  DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, sizeof(uint32_t), s));
+  DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, 2 * sizeof(uint32_t), s));
   DDHF_TRY(bin_into(c, 0, x, y, t_us, p, n, t0_us, window_us, s));
   c->binned = true;
   return DDHF_OK;

@@ -17,6 +17,8 @@
 // Per-pixel counts come from segment boundaries of the sorted keys, and one
 // 64-bit scan of (count << 32 | active flag) gives both the CSR offsets and
 // the active-pixel list.
+#include <algorithm>
+
 #include "ddhf_internal.cuh"
 
 namespace ddhf {
@@ -446,9 +448,10 @@ __global__ void k_pack(const uint32_t *__restrict__ seg_lo, const uint32_t *__re
 __global__ void k_finish(const uint64_t *__restrict__ scanned, const uint32_t *__restrict__ seg_lo,
                          const uint32_t *__restrict__ seg_hi, uint32_t *__restrict__ offsets,
                          uint32_t *__restrict__ active, uint64_t *__restrict__ counters,
-                         int64_t npx, int n_min, int heavy_min, int64_t n_in, int64_t n_bins,
-                         uint64_t *__restrict__ heavy_list, uint32_t *heavy_count,
-                         uint32_t slot, int64_t heavy_cap, uint32_t *flags) {
+                         int64_t npx, int n_min, int heavy_min, int big_min, int64_t n_in,
+                         int64_t n_bins, uint64_t *__restrict__ heavy_list,
+                         uint32_t *heavy_count, uint32_t slot, int64_t heavy_cap,
+                         uint32_t *flags) {
   uint64_t terms = 0;
   uint32_t heavy = 0;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k <= npx;
@@ -462,9 +465,12 @@ __global__ void k_finish(const uint64_t *__restrict__ scanned, const uint32_t *_
         terms += (uint64_t)cnt * (uint64_t)n_bins;
         if (cnt >= (uint32_t)heavy_min) {
           heavy += 1u;
-          const uint32_t pos = atomicAdd(heavy_count, 1u);
+          // heavy pixels from the list's front, big ones from its back (the list
+          // holds every pixel of at least heavy_min events)
+          const bool big = cnt >= (uint32_t)big_min;
+          const uint32_t pos = atomicAdd(heavy_count + (big ? 1 : 0), 1u);
           if ((int64_t)pos < heavy_cap)
-            heavy_list[pos] = ((uint64_t)slot << 32) | (uint32_t)v;
+            heavy_list[big ? heavy_cap - 1 - pos : pos] = ((uint64_t)slot << 32) | (uint32_t)v;
           else
             atomicOr(flags, DDHF_FLAG_CAPACITY);
         }
@@ -652,7 +658,7 @@ void scatter_attributes() {
   }
 }
 
-ddhf_status bin_core(Ctx *c, Slot &sl, const RawIn &raw, int n_min, int heavy_min,
+ddhf_status bin_core(Ctx *c, Slot &sl, const RawIn &raw, int n_min, int heavy_min, int big_min,
                      uint64_t *heavy_list, uint32_t *heavy_count, uint32_t slot_tag,
                      int64_t heavy_cap, cudaStream_t s) {
   const int64_t n = raw.n;
@@ -723,8 +729,8 @@ ddhf_status bin_core(Ctx *c, Slot &sl, const RawIn &raw, int n_min, int heavy_mi
   DDHF_CUDA_TRY(c, scan_rec<uint64_t>(c->packed, c->packed, npx + 1,
                                       reinterpret_cast<uint64_t *>(c->scan_part), nullptr, s));
   k_finish<<<pb, 256, 0, s>>>(c->packed, c->seg_lo, c->seg_hi, sl.offsets, sl.active,
-                              sl.counters, npx, n_min, heavy_min, n, c->grid.n_bins, heavy_list,
-                              heavy_count, slot_tag, heavy_cap, c->flags);
+                              sl.counters, npx, n_min, heavy_min, big_min, n, c->grid.n_bins,
+                              heavy_list, heavy_count, slot_tag, heavy_cap, c->flags);
   DDHF_CUDA_TRY(c, cudaGetLastError());
   return DDHF_OK;
 }
@@ -735,8 +741,9 @@ ddhf_status bin_window(Ctx *c, int slot_i, const int16_t *x, const int16_t *y, c
   sl.t0 = t0;
   sl.window_us = win;
   RawIn raw{x, y, t, p, n, t0, (uint64_t)win, c->W, c->H, c->params.polarity_01, c->row0};
-  return bin_core(c, sl, raw, c->params.n_min, c->tuning.heavy_min, c->work, c->qctl,
-                  (uint32_t)slot_i, c->heavy_cap, s);
+  return bin_core(c, sl, raw, c->params.n_min, std::min(c->tuning.heavy_min, kTeamPixel),
+                  std::max(c->tuning.heavy_min, kBigPixel), c->work, c->qctl, (uint32_t)slot_i,
+                  c->heavy_cap, s);
 }
 
 // Stable sort of pre-packed (key, value) pairs into a slot's per-pixel list;
@@ -745,7 +752,8 @@ ddhf_status bin_packed(Ctx *c, Slot &sl, const uint32_t *keys, const uint32_t *v
                        int n_min, int heavy_min, uint64_t *heavy_list, uint32_t *heavy_count,
                        int64_t heavy_cap, cudaStream_t s) {
   RawIn raw{nullptr, nullptr, nullptr, nullptr, n, 0, 0, c->W, c->H, 0, 0, keys, vals};
-  return bin_core(c, sl, raw, n_min, heavy_min, heavy_list, heavy_count, 0u, heavy_cap, s);
+  return bin_core(c, sl, raw, n_min, heavy_min, INT32_MAX, heavy_list, heavy_count, 0u,
+                  heavy_cap, s);
 }
 
 void set_bin_attributes() {

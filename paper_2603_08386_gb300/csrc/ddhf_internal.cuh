@@ -23,6 +23,8 @@ constexpr int kMaxBandWords = 8;   // comb rank band up to 256 positions
 constexpr uint32_t kSignBit = 0x80000000u;
 constexpr size_t kCanaryBytes = 256;        // guard region on each side of a buffer
 constexpr unsigned char kCanaryByte = 0xA5;
+constexpr int kTeamPixel = 256;             // events from which four warps take a pixel
+constexpr int kBigPixel = 2048;             // events from which a cluster of blocks takes it
 constexpr uint32_t kDropKey = 0xffffffffu;  // pre-packed sort input: pair not kept
 
 // Invariant checks of the debug build (-DDDHF_BOUNDS_CHECK, made by
@@ -159,7 +161,8 @@ struct Ctx {
   // work queue of the persistent kernel
   uint64_t *work = nullptr;      // [heavy_cap] heavy items (slot << 32 | active index)
   int64_t heavy_cap = 0;
-  uint32_t *qctl = nullptr;      // [16] queue counters: [0] heavy count, [1-2] spectrum cursors,
+  uint32_t *qctl = nullptr;      // [16] queue counters: [0] heavy count, [1] big count, [5-7]
+                                 // spectrum cursors (heavy, light, big),
                                  // [4] soft-comb cursor, [8] kept events of a binning, [9]
                                  // label count, [12-13] hybrid lists, [14] hybrid cursor
   // labelling / boxes scratch

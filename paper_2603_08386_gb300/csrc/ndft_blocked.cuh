@@ -36,18 +36,34 @@
 // before it, with its longer rotation chains: 8.1e-7 and 1.3e-6).
 //
 // Measured (one 1280x720 window of 19.9M events, 750 bins, default tuning):
-// 2.58 -> 1.49 ms (issue 61 % at 16 warps per SM, tensor pipe 34 %, 1,095 warp
-// instructions per pixel; 1.55 ms and 1,227 before the rotation chains were
-// paired); 640x480 at 2000 bins 1.79 -> 0.99 ms.
+// 2.58 -> 1.33 ms (issue 55 % at 16 warps per SM, tensor pipe 38 %, 920 warp
+// instructions per pixel; bound by the latency of its dependent chains at the
+// occupancy that 128 registers allow); 640x480 at 2000 bins 1.79 -> 0.82 ms,
+// 320x180 at 10,000 bins 7.4 -> 2.7 ms, a sparse 1280x720 window (1.06M events)
+// 190 -> 80 us.
 //
 // Bins whose frequency is a multiple of D (in practice bin 0 of a grid that
 // starts at 0 Hz) have the phase 0 for every event: their power is the squared
 // integer sum of the polarities, counted exactly (Eq. 7 takes the logarithm of
 // it, and a sum of zero must be exactly zero).
 //
-// Light pixels take one warp, heavy pixels a whole block (events split over
-// warps, partial sums reduced in a fixed order), heavy first.
+// Who takes a pixel, and in which order its events are summed, both by its event
+// count n alone:
+//   n < 256 (kTeamPixel)   one warp, group after group (unless the tuning's
+//                          heavy_min lists it);
+//   n >= 256, or listed    four sums over every fourth chunk of 32 events, added
+//                          in order, by a team of four warps (or of two): one
+//                          warp needs 1.6 us per chunk, so that a 1000-event
+//                          pixel alone took 62 us, longer than the rest of a
+//                          sparse window; by a team 19 us;
+//   n >= 2048 (kBigPixel)  (and heavy_min) a cluster of four blocks, one sum per
+//                          warp, added in order through shared memory: 20,000
+//                          events are 156 chunks per warp of a block.
+// Big pixels first, then the listed ones, then the light. When several passes
+// cover the bins, each (pixel, pass) of the first two is an item of its own.
 #pragma once
+
+#include <cooperative_groups.h>
 
 #include <algorithm>
 
@@ -133,25 +149,28 @@ struct ChainPair {
   }
 };
 
-// Shared-memory layout of one warp's staged factors, per event: B (32 columns)
-// as eight 16-byte units of four words, A as one such array per two m-tiles and
-// an array of eight 8-byte units for an odd one (MT m-tiles of 8 rows; the words
-// of lane group g belong to rows MT g .. MT g + MT - 1, Re and Im). Events are
-// nine units apart and the units permuted, so that neither the generating
-// lanes (one event each) nor the multiplying ones (lane (g, t): unit g of
-// events t and t + 4) meet a bank twice (8-byte units: one extra wavefront).
+// Shared-memory record of one event's factors: the 32 words of B, word 8 c + g
+// for lane group g (columns k = 4 (g / 2) + c, real part c_k for an even g,
+// imaginary d_k for an odd one), then A's rows in order, Re and Im, and 32 bytes
+// of padding: lane (g, t) of a step reads word 8 c + g and row 8 i + g of events
+// t and t + 4, and with this stride no two lanes of a load share a bank. The
+// words are loaded one and two at a time, straight into the register pairs that
+// the tensor instruction takes: 16-byte loads cost 18-27 % more instructions in
+// moves.
 template <int MT>
 struct Stage {
-  static constexpr int kPairs = MT / 2;                 // 16-byte A arrays
-  static constexpr int kB = 0;                          // bytes
-  static constexpr int kA = 144 * kGenChunk;
-  static constexpr int kArray = 144 * kGenChunk;        // per 16-byte array
-  static constexpr int kA64 = kA + kPairs * kArray;
-  static constexpr int kBytes = kA64 + (MT & 1) * 72 * kGenChunk;
+  static constexpr int kRows = 128;                   // byte offset of the rows
+  static constexpr int kRec = 128 + 64 * MT + 32;     // bytes per event
+  static constexpr int kBytes = kRec * kGenChunk;
 };
-__device__ __forceinline__ int unit16(int g) { return (g >> 1) + 4 * (g & 1); }
-__device__ __forceinline__ int unit8(int g) {
-  return ((g >> 2) << 1) + ((g & 1) << 2) + ((g >> 1) & 1);
+
+__device__ __forceinline__ uint32_t lds32(uint32_t sa) {
+  uint32_t x;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x) : "r"(sa) : "memory");
+  return x;
+}
+__device__ __forceinline__ void lds64(uint32_t sa, uint32_t &x, uint32_t &y) {
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(sa) : "memory");
 }
 
 // The factors of event word w (lane = event of the chunk) into the warp's
@@ -160,26 +179,27 @@ __device__ __forceinline__ int unit8(int g) {
 template <int MT>
 __device__ __forceinline__ void gen_chunk(uint32_t w, const NdftConst &nd, uint64_t f_row,
                                           unsigned char *stage) {
-  const int e = threadIdx.x & 31;
   const uint32_t tau = w & 0x7fffffffu, sg = w & kSignBit;
+  unsigned char *rec = stage + (threadIdx.x & 31) * Stage<MT>::kRec;
   // columns: k = 8 exact, 9..15 and 7..0 by rotation
   {
     const float2 u = phasor_of_turn(nd.f_u, tau), k8 = phasor_of_turn(nd.f_k8, tau);
     ChainPair z(k8, cmul(k8, make_float2(u.x, -u.y)), u);
-    uint4 *b = reinterpret_cast<uint4 *>(stage + Stage<MT>::kB + e * 144);
+    uint4 *b = reinterpret_cast<uint4 *>(rec);
+    uint32_t up[4][2], dn[4][2];  // columns 8 + c and 4 + c
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      uint32_t c[4], d[4], c2[4], d2[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (h + i > 0) z.step();
-        split_half2(z.x, c[i], c2[3 - i]);  // k = 8 + 4 h + i and 7 - 4 h - i
-        split_half2(z.y, d[i], d2[3 - i]);
+    for (int i = 0; i < 8; ++i) {
+      if (i > 0) z.step();  // k = 8 + i and 7 - i
+      uint32_t cu, cd, du, dd;
+      split_half2(z.x, cu, cd);
+      split_half2(z.y, du, dd);
+      if (i < 4) {
+        up[i][0] = cu, up[i][1] = du;
+        dn[3 - i][0] = cd, dn[3 - i][1] = dd;
+      } else {
+        b[2 * (i - 4) + 1] = make_uint4(up[i - 4][0], up[i - 4][1], cu, du);
+        b[2 * (7 - i)] = make_uint4(cd, dd, dn[7 - i][0], dn[7 - i][1]);
       }
-      b[2 + h] = make_uint4(c[0], c[1], c[2], c[3]);
-      b[6 + h] = make_uint4(d[0], d[1], d[2], d[3]);
-      b[1 - h] = make_uint4(c2[0], c2[1], c2[2], c2[3]);
-      b[5 - h] = make_uint4(d2[0], d2[1], d2[2], d2[3]);
     }
   }
   // rows: 4 MT exact (the polarity's sign on it), the others by rotation
@@ -189,34 +209,23 @@ __device__ __forceinline__ void gen_chunk(uint32_t w, const NdftConst &nd, uint6
     s.x = __uint_as_float(__float_as_uint(s.x) ^ sg);
     s.y = __uint_as_float(__float_as_uint(s.y) ^ sg);
     ChainPair z(s, cmul(s, make_float2(v.x, -v.y)), v);
+    uint4 *a = reinterpret_cast<uint4 *>(rec + Stage<MT>::kRows);  // two rows each
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      uint32_t r[2 * MT], r2[2 * MT];
+    for (int i = 0; i < 2 * MT; ++i) {
+      uint32_t u[4], d[4];
 #pragma unroll
-      for (int i = 0; i < MT; ++i) {
-        if (h + i > 0) z.step();
-        // rows MT (4 + h) + i and MT (3 - h) + MT - 1 - i
-        split_half2(z.x, r[2 * i], r2[2 * (MT - 1 - i)]);
-        split_half2(z.y, r[2 * i + 1], r2[2 * (MT - 1 - i) + 1]);
+      for (int j = 0; j < 2; ++j) {
+        if (i + j > 0) z.step();  // rows 4 MT + 2 i + j and 4 MT - 1 - 2 i - j
+        split_half2(z.x, u[2 * j], d[2 - 2 * j]);
+        split_half2(z.y, u[2 * j + 1], d[3 - 2 * j]);
       }
-      const int gu = 4 + h, gd = 3 - h;
-#pragma unroll
-      for (int p = 0; p < Stage<MT>::kPairs; ++p) {
-        uint4 *a = reinterpret_cast<uint4 *>(stage + Stage<MT>::kA + p * Stage<MT>::kArray +
-                                             e * 144);
-        a[unit16(gu)] = make_uint4(r[4 * p], r[4 * p + 1], r[4 * p + 2], r[4 * p + 3]);
-        a[unit16(gd)] = make_uint4(r2[4 * p], r2[4 * p + 1], r2[4 * p + 2], r2[4 * p + 3]);
-      }
-      if (MT & 1) {
-        uint2 *a = reinterpret_cast<uint2 *>(stage + Stage<MT>::kA64 + e * 72);
-        a[unit8(gu)] = make_uint2(r[2 * MT - 2], r[2 * MT - 1]);
-        a[unit8(gd)] = make_uint2(r2[2 * MT - 2], r2[2 * MT - 1]);
-      }
+      a[2 * MT + i] = make_uint4(u[0], u[1], u[2], u[3]);
+      a[2 * MT - 1 - i] = make_uint4(d[0], d[1], d[2], d[3]);
     }
   }
 }
 
-// A lane's accumulators: x[i][q] = (X1, X4, X3, X2) of row MT g + i and column
+// A lane's accumulators: x[i][q] = (X1, X4, X3, X2) of row 8 i + g and column
 // pair k = 4 t + q (lane (g, t) = (lane / 4, lane % 4)): the C fragment of an
 // m16n8k16 step whose rows g and g + 8 are Re and Im of A and whose columns 2 t
 // and 2 t + 1 are c and d.
@@ -270,30 +279,26 @@ __device__ __forceinline__ void mma_group(int q, int m, const unsigned char *sta
     e0 = min(e0, kGenChunk - 1);
     e1 = min(e1, kGenChunk - 1);
   }
-  const unsigned char *s0 = stage + 16 * unit16(g) + e0 * 144;
-  const unsigned char *s1 = stage + 16 * unit16(g) + e1 * 144;
-  uint4 b0 = *reinterpret_cast<const uint4 *>(s0 + Stage<MT>::kB);
-  uint4 b1 = *reinterpret_cast<const uint4 *>(s1 + Stage<MT>::kB);
-  uint32_t a[MT][4];
+  const uint32_t sa = (uint32_t)__cvta_generic_to_shared(stage);
+  const uint32_t s0 = sa + e0 * Stage<MT>::kRec, s1 = sa + e1 * Stage<MT>::kRec;
+  uint32_t w0[4], w1[4], a[MT][4];
 #pragma unroll
-  for (int p = 0; p < Stage<MT>::kPairs; ++p) {
-    const int o = Stage<MT>::kA + p * Stage<MT>::kArray;
-    const uint4 x = *reinterpret_cast<const uint4 *>(s0 + o);
-    const uint4 y = *reinterpret_cast<const uint4 *>(s1 + o);
-    a[2 * p][0] = x.x, a[2 * p][1] = x.y, a[2 * p][2] = y.x, a[2 * p][3] = y.y;
-    a[2 * p + 1][0] = x.z, a[2 * p + 1][1] = x.w, a[2 * p + 1][2] = y.z, a[2 * p + 1][3] = y.w;
+  for (int c = 0; c < 4; ++c) {
+    w0[c] = lds32(s0 + 4 * g + 32 * c);
+    w1[c] = lds32(s1 + 4 * g + 32 * c);
   }
-  if (MT & 1) {
-    const unsigned char *sa = stage + Stage<MT>::kA64 + 8 * unit8(g);
-    const uint2 x = *reinterpret_cast<const uint2 *>(sa + e0 * 72);
-    const uint2 y = *reinterpret_cast<const uint2 *>(sa + e1 * 72);
-    a[MT - 1][0] = x.x, a[MT - 1][1] = x.y, a[MT - 1][2] = y.x, a[MT - 1][3] = y.y;
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+    lds64(s0 + 8 * g + Stage<MT>::kRows + 64 * i, a[i][0], a[i][1]);
+    lds64(s1 + 8 * g + Stage<MT>::kRows + 64 * i, a[i][2], a[i][3]);
   }
   if (m < kGroup) {  // past the pixel's last event
-    if (t >= m) b0 = make_uint4(0u, 0u, 0u, 0u);
-    if (t + 4 >= m) b1 = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (t >= m) w0[c] = 0u;
+      if (t + 4 >= m) w1[c] = 0u;
+    }
   }
-  const uint32_t w0[4] = {b0.x, b0.y, b0.z, b0.w}, w1[4] = {b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const uint32_t x0 = __byte_perm(w0[c], 0u, 0x1032u), x1 = __byte_perm(w1[c], 0u, 0x1032u);
@@ -325,16 +330,17 @@ struct BlockedArgs {
   int n_slots;
   int64_t npx;
   const uint64_t *heavy;     // heavy work items (slot << 32 | active index)
-  const uint32_t *n_heavy;   // count of heavy items
+  const uint32_t *n_heavy;   // [0] heavy items, from the list's front, [1] big ones, from its back
   uint32_t heavy_cap;        // capacity of the heavy list
-  uint32_t *cursors;         // [0] heavy cursor, [1] light cursor
+  uint32_t *cursors;         // [0] heavy cursor, [1] light cursor, [2] big cursor
   int N, nbr;                // bins, rows of 32 bins
   CombConst cc;
   float *P;                  // spectra (write mode), rows in active order of slot 0
   int64_t ld;                // row stride of P in floats (>= N)
   int vec_store;             // P and ld 16-byte aligned
   int64_t cap_px;
-  int heavy_min;
+  int heavy_min;             // events from which the list holds a pixel
+  int light_max;             // the light path takes pixels of fewer events (<= heavy_min)
   int skip_min;              // > 0: pixels with at least this many events are left to the
                              // hybrid grid path (their rows are written there)
   int warp_bytes;            // per-warp shared memory (bytes)
@@ -364,7 +370,7 @@ __device__ __forceinline__ void finalize_tile(const Acc<MT> &acc, float *Pw, int
     float pp[4], pm[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc.powers(i, q, pp[q], pm[q]);
-    float *row = Pw + (row_base + MT * g + i) * 32;
+    float *row = Pw + (row_base + 8 * i + g) * 32;
     *reinterpret_cast<float4 *>(row + 16 + 4 * t) = make_float4(pp[0], pp[1], pp[2], pp[3]);
     *reinterpret_cast<float4 *>(row + 12 - 4 * t) = make_float4(pm[3], pm[2], pm[1], pm[0]);
   }
@@ -378,20 +384,20 @@ __device__ __forceinline__ void store_tile(const BlockedArgs &A, const Acc<MT> &
                                            int b0, int sum_p) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   float *dst = A.P + prow * A.ld;
-  const int row = b0 + MT * g, whole = A.vec_store ? A.N >> 5 : 0;  // rows below it: 16-byte stores
+  const int row = b0 + g, whole = A.vec_store ? A.N >> 5 : 0;  // rows below it: 16-byte stores
   float *up = dst + 32 * row + 16 + 4 * t, *dn = dst + 32 * row + 12 - 4 * t;
 #pragma unroll
   for (int i = 0; i < MT; ++i) {
     float pv[2][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc.powers(i, q, pv[1][q], pv[0][3 - q]);
-    if (row + i < whole) {
-      *reinterpret_cast<float4 *>(up + 32 * i) = make_float4(pv[1][0], pv[1][1], pv[1][2], pv[1][3]);
-      *reinterpret_cast<float4 *>(dn + 32 * i) = make_float4(pv[0][0], pv[0][1], pv[0][2], pv[0][3]);
+    if (row + 8 * i < whole) {
+      *reinterpret_cast<float4 *>(up + 256 * i) = make_float4(pv[1][0], pv[1][1], pv[1][2], pv[1][3]);
+      *reinterpret_cast<float4 *>(dn + 256 * i) = make_float4(pv[0][0], pv[0][1], pv[0][2], pv[0][3]);
     } else {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int j = 32 * (row + i) + (h ? 16 + 4 * t : 12 - 4 * t);
+        const int j = 32 * (row + 8 * i) + (h ? 16 + 4 * t : 12 - 4 * t);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
           if (j + q < A.N) dst[j + q] = pv[h][q];
@@ -476,14 +482,14 @@ __device__ __forceinline__ void light_stream(const BlockedArgs &A, unsigned char
       q_lo = v.offsets[key];
       q_hi = v.offsets[key + 1];
       const int cnt = (int)(q_hi - q_lo);
-      q_ok = cnt < A.heavy_min && !(A.skip_min > 0 && cnt >= A.skip_min) &&
+      q_ok = cnt < A.light_max && !(A.skip_min > 0 && cnt >= A.skip_min) &&
              ddhf_check((int64_t)q_hi <= A.ev_cap, A.flags);
       if (q_ok && aq >= A.cap_px) {
         raise_flag(A.flags, DDHF_FLAG_CAPACITY);
         q_ok = false;
       }
     }
-    uint32_t okm = __ballot_sync(0xffffffffu, q_ok);
+    const uint32_t okm = __ballot_sync(0xffffffffu, q_ok);
     if (!okm) continue;
     // in order: every light pixel's list starts at or after the previous one's end
     const uint32_t lower = okm & lanemask_lt();
@@ -507,7 +513,11 @@ __device__ __forceinline__ void light_stream(const BlockedArgs &A, unsigned char
           const uint32_t pe1 = __shfl_sync(0xffffffffu, q_hi, p);
           Acc<MT> acc;
           int neg = 0;
-          if (pe0 >= pe1) acc.zero();
+          // a step of its own for the first group saves the clearing and adding,
+          // but costs registers: 834 against 867 us at 2000 bins (MT 4), 1.38
+          // against 1.33 ms at 750 (MT 3)
+          constexpr bool kFirst = MT == 4;
+          if (!kFirst || pe0 >= pe1) acc.zero();
           for (uint32_t pos = pe0; pos < pe1; pos += kGroup) {
             const int m = (int)min((uint32_t)kGroup, pe1 - pos);
             uint32_t d = pos - c0;
@@ -528,7 +538,7 @@ __device__ __forceinline__ void light_stream(const BlockedArgs &A, unsigned char
               wn = pos + 32u + lane < e_end ? v.ev[pos + 32u + lane] : 0u;
             }
             if (has_dc) neg += __popc((sgn >> d) & (0xffu >> (kGroup - m)));
-            if (pos == pe0) mma_group<MT, true>((int)d, m, stage, acc);
+            if (kFirst && pos == pe0) mma_group<MT, true>((int)d, m, stage, acc);
             else mma_group<MT, false>((int)d, m, stage, acc);
           }
           store_tile<MT>(A, acc, (int64_t)a0 + p, b0, (int)(pe1 - pe0) - 2 * neg);
@@ -551,74 +561,234 @@ __device__ __forceinline__ void store_scores(const BlockedArgs &A, const SlotVie
   }
 }
 
+// Barrier of a team of TW warps (team `id` of the block).
+template <int TW>
+__device__ __forceinline__ void team_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id + 1), "n"(32 * TW) : "memory");
+}
+
+// The four sums of a pixel's events (chunks r, r + 4, ... of 32), added in order
+// by a team of TW warps (this one: warp tw), into the accumulators of warp 0;
+// returns the number of negative events there. s_neg: four words per team.
+template <int MT, int TW>
+__device__ __forceinline__ int team_sum(const uint32_t *evp, int cnt, const NdftConst &nd,
+                                        uint64_t f_row, unsigned char *stage, int warp_bytes,
+                                        int tw, int id, int *s_neg, Acc<MT> &acc) {
+  const int lane = threadIdx.x & 31;
+  float *part = reinterpret_cast<float *>(stage);
+  float tot[16 * MT];  // the sum so far, when the team takes several rounds
+  int neg_tot = 0;
+#pragma unroll 1
+  for (int r0 = 0; r0 < 4; r0 += TW) {
+    acc.zero();
+    const int neg = accumulate<MT>(evp, cnt, r0 + tw, 4, nd, f_row, stage, acc);
+    // partial sums of this warp -> its staging area, [row, column, component][lane]
+#pragma unroll
+    for (int i = 0; i < 16 * MT; ++i) part[i * 32 + lane] = acc.x[i / 16][(i / 4) % 4][i % 4];
+    if (lane == 0) s_neg[tw] = neg;
+    team_sync<TW>(id);
+    if (tw == 0) {
+      neg_tot += neg;
+      if (r0 > 0)
+#pragma unroll
+        for (int i = 0; i < 16 * MT; ++i) {
+          float &x = acc.x[i / 16][(i / 4) % 4][i % 4];
+          x = __fadd_rn(tot[i], x);
+        }
+      for (int w2 = 1; w2 < TW; ++w2) {
+        const float *op = reinterpret_cast<const float *>(stage + w2 * warp_bytes);
+#pragma unroll
+        for (int i = 0; i < 16 * MT; ++i) {
+          float &x = acc.x[i / 16][(i / 4) % 4][i % 4];
+          x = __fadd_rn(x, op[i * 32 + lane]);
+        }
+        neg_tot += s_neg[w2];
+      }
+      if (TW < 4)
+#pragma unroll
+        for (int i = 0; i < 16 * MT; ++i) tot[i] = acc.x[i / 16][(i / 4) % 4][i % 4];
+    }
+    team_sync<TW>(id);  // the partial sums have been read
+  }
+  return neg_tot;
+}
+
+// Warp 0 of a team or cluster: the finished sums of pass ps to the spectrum row,
+// or to Pw (FUSED).
+template <int MT, bool FUSED>
+__device__ __forceinline__ void heavy_store(const BlockedArgs &A, const Acc<MT> &acc, int64_t a,
+                                            int ps, int sum_p, float *Pw) {
+  const int b0 = ps * 8 * MT;
+  if (FUSED) {
+    finalize_tile<MT>(acc, Pw, b0);
+    exact_bins(A, sum_p, 32 * b0, min(A.N, 32 * (b0 + 8 * MT)), Pw);
+  } else {
+    store_tile<MT>(A, acc, a, b0, sum_p);
+  }
+  __syncwarp();
+}
+
+// An item of the heavy list: its active index, slot, events; false when the
+// item is not this kernel's.
+struct HeavyPixel {
+  int64_t a;
+  const SlotView *v;
+  uint32_t key, o0;
+  int cnt;
+};
+template <bool FUSED>
+__device__ __forceinline__ bool heavy_pixel(const BlockedArgs &A, uint64_t it, HeavyPixel &h) {
+  h.a = (int64_t)(uint32_t)it;
+  h.v = &A.views[it >> 32];
+  h.key = h.v->active[h.a];
+  h.o0 = h.v->offsets[h.key];
+  h.cnt = (int)(h.v->offsets[h.key + 1] - h.o0);
+  if (A.skip_min > 0 && h.cnt >= A.skip_min) return false;
+  if (!ddhf_check((int64_t)h.o0 + h.cnt <= A.ev_cap, A.flags)) return false;
+  if (!FUSED && h.a >= A.cap_px) {
+    raise_flag(A.flags, DDHF_FLAG_CAPACITY);
+    return false;
+  }
+  return true;
+}
+
+// A listed pixel (pass >= 0: that pass of the bins alone, else all of them, and
+// the pixel is scored, FUSED) by a team of TW warps. Out of line, so that its
+// registers do not count against the light pixels' loop.
+template <int MT, int NW, bool FUSED, int TW>
+__device__ __noinline__ void team_item(const BlockedArgs &A, uint64_t it, int pass,
+                                       unsigned char *stage, int tw, int id, int *s_neg) {
+  HeavyPixel h;
+  if (!heavy_pixel<FUSED>(A, it, h)) return;
+  float *Pw = reinterpret_cast<float *>(stage + A.pw_offset);
+  const int p0 = pass >= 0 ? pass : 0;
+  const int p1 = pass >= 0 ? pass + 1 : (A.nbr + 8 * MT - 1) / (8 * MT);
+  for (int ps = p0; ps < p1; ++ps) {
+    Acc<MT> acc;
+    const int neg = team_sum<MT, TW>(h.v->ev + h.o0, h.cnt, A.nd, A.nd.f_row[ps], stage,
+                                     A.warp_bytes, tw, id, s_neg, acc);
+    if (tw == 0) heavy_store<MT, FUSED>(A, acc, h.a, ps, h.cnt - 2 * neg, Pw);
+  }
+  if (FUSED && tw == 0) {
+    CombOut o = comb_warp<NW>(Pw, A.cc, stage);
+    store_scores<NW>(A, *h.v, h.a, h.key, o);
+  }
+}
+
+// A big pixel by the blocks of a cluster: warp w of block r takes chunks r nw +
+// w, + blocks nw, ...; warp 0 of each block adds its warps' sums, that of the
+// first block the other blocks'.
 template <int MT, int NW, bool FUSED>
-__global__ void __launch_bounds__(256, 2) k_blocked(BlockedArgs A) {
-  extern __shared__ float4 smem4[];
+__device__ __noinline__ void cluster_item(const BlockedArgs &A, uint64_t it, int pass,
+                                          unsigned char *stage, int *s_neg) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int blocks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  HeavyPixel h;
+  if (!heavy_pixel<FUSED>(A, it, h)) return;  // the same answer in every block
+  float *Pw = reinterpret_cast<float *>(stage + A.pw_offset);
+  float *part = reinterpret_cast<float *>(stage);
+  const int p0 = pass >= 0 ? pass : 0;
+  const int p1 = pass >= 0 ? pass + 1 : (A.nbr + 8 * MT - 1) / (8 * MT);
+  for (int ps = p0; ps < p1; ++ps) {
+    Acc<MT> acc;
+    acc.zero();
+    int neg = accumulate<MT>(h.v->ev + h.o0, h.cnt, rank * nw + warp, blocks * nw, A.nd,
+                             A.nd.f_row[ps], stage, acc);
+#pragma unroll
+    for (int i = 0; i < 16 * MT; ++i) part[i * 32 + lane] = acc.x[i / 16][(i / 4) % 4][i % 4];
+    if (lane == 0) s_neg[warp] = neg;
+    __syncthreads();
+    if (warp == 0) {
+      for (int w2 = 1; w2 < nw; ++w2) {
+        const float *op = reinterpret_cast<const float *>(stage + w2 * A.warp_bytes);
+#pragma unroll
+        for (int i = 0; i < 16 * MT; ++i) {
+          float &x = acc.x[i / 16][(i / 4) % 4][i % 4];
+          x = __fadd_rn(x, op[i * 32 + lane]);
+        }
+        neg += s_neg[w2];
+      }
+      if (rank != 0) {
+#pragma unroll
+        for (int i = 0; i < 16 * MT; ++i) part[i * 32 + lane] = acc.x[i / 16][(i / 4) % 4][i % 4];
+        if (lane == 0) s_neg[0] = neg;
+      }
+    }
+    cluster.sync();
+    if (warp == 0 && rank == 0) {
+      for (int r = 1; r < blocks; ++r) {
+        const float *op = cluster.map_shared_rank(part, r);
+#pragma unroll
+        for (int i = 0; i < 16 * MT; ++i) {
+          float &x = acc.x[i / 16][(i / 4) % 4][i % 4];
+          x = __fadd_rn(x, op[i * 32 + lane]);
+        }
+        neg += *cluster.map_shared_rank(s_neg, r);
+      }
+      heavy_store<MT, FUSED>(A, acc, h.a, ps, h.cnt - 2 * neg, Pw);
+    }
+    cluster.sync();  // the other blocks' sums have been read
+  }
+  if (FUSED && warp == 0 && rank == 0) {
+    CombOut o = comb_warp<NW>(Pw, A.cc, stage);
+    store_scores<NW>(A, *h.v, h.a, h.key, o);
+  }
+}
+
+// The listed pixels, item by item, by teams of TW warps.
+template <int MT, int NW, bool FUSED, int TW>
+__device__ __forceinline__ void team_loop(const BlockedArgs &A, uint32_t per_px,
+                                          unsigned char *stage, uint32_t *s_item, int *s_neg) {
+  const int warp = threadIdx.x >> 5, tw = warp % TW, id = warp / TW;
+  const uint32_t n_heavy = min(A.n_heavy[0], A.heavy_cap);
+  if (n_heavy == 0) return;
+  for (;;) {
+    if (tw == 0 && (threadIdx.x & 31) == 0) s_item[id] = atomicAdd(&A.cursors[0], 1u);
+    team_sync<TW>(id);
+    const uint32_t item = s_item[id];
+    team_sync<TW>(id);
+    if (item / per_px >= n_heavy) break;
+    team_item<MT, NW, FUSED, TW>(A, A.heavy[item / per_px], FUSED ? -1 : (int)(item % per_px),
+                                 stage, tw, id, s_neg + 4 * id);
+  }
+}
+
+// Big pixels, one cluster each, then the other listed ones, a team of warps each.
+template <int MT, int NW, bool FUSED>
+__device__ __noinline__ void listed_pixels(const BlockedArgs &A, unsigned char *stage,
+                                           uint32_t *s_item, int *s_neg) {
+  namespace cg = cooperative_groups;
+  // items of a pixel: its passes (a fused pixel is scored once all are in)
+  const uint32_t per_px = FUSED ? 1u : (uint32_t)((A.nbr + 8 * MT - 1) / (8 * MT));
+  const uint32_t n_big = min(A.n_heavy[1], A.heavy_cap);
+  if (n_big > 0) {
+    const cg::cluster_group cluster = cg::this_cluster();
+    for (;;) {
+      if (cluster.block_rank() == 0 && threadIdx.x == 0) s_item[0] = atomicAdd(&A.cursors[2], 1u);
+      cluster.sync();
+      const uint32_t item = *cluster.map_shared_rank(&s_item[0], 0);
+      cluster.sync();
+      if (item / per_px >= n_big) break;
+      cluster_item<MT, NW, FUSED>(A, A.heavy[A.heavy_cap - 1 - item / per_px],
+                                  FUSED ? -1 : (int)(item % per_px), stage, s_neg);
+    }
+  }
+  if (blockDim.x >= 128) team_loop<MT, NW, FUSED, 4>(A, per_px, stage, s_item, s_neg);
+  else team_loop<MT, NW, FUSED, 2>(A, per_px, stage, s_item, s_neg);
+  __syncwarp();
+}
+
+template <int MT, int NW, bool FUSED>
+__global__ void __launch_bounds__(256, 2) k_blocked(const __grid_constant__ BlockedArgs A) {
+  extern __shared__ float4 smem4[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned char *stage = reinterpret_cast<unsigned char *>(smem4) + warp * A.warp_bytes;
   float *Pw = reinterpret_cast<float *>(stage + A.pw_offset);
-  __shared__ uint32_t s_item;
+  __shared__ uint32_t s_item[2];
   __shared__ int s_neg[8];
-
-  // ---------------- heavy pixels: one block each, events split over warps
-  const uint32_t n_heavy = min(*A.n_heavy, A.heavy_cap);
-  for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(&A.cursors[0], 1u);
-    __syncthreads();
-    const uint32_t item = s_item;
-    __syncthreads();
-    if (item >= n_heavy) break;
-    const uint64_t it = A.heavy[item];
-    const int slot = (int)(it >> 32);
-    const int64_t a = (int64_t)(uint32_t)it;
-    const SlotView v = A.views[slot];
-    const uint32_t key = v.active[a];
-    const uint32_t o0 = v.offsets[key];
-    const int cnt = (int)(v.offsets[key + 1] - o0);
-    if (A.skip_min > 0 && cnt >= A.skip_min) continue;
-    if (!ddhf_check((int64_t)o0 + cnt <= A.ev_cap, A.flags)) continue;
-    if (!FUSED && a >= A.cap_px) {
-      if (threadIdx.x == 0) raise_flag(A.flags, DDHF_FLAG_CAPACITY);
-      continue;
-    }
-    for (int b0 = 0, pass = 0; b0 < A.nbr; b0 += 8 * MT, ++pass) {
-      Acc<MT> acc;
-      acc.zero();
-      const int neg = accumulate<MT>(v.ev + o0, cnt, warp, nw, A.nd, A.nd.f_row[pass], stage, acc);
-      // partial sums of this warp -> its staging area, [row, column, component][lane]
-      float *part = reinterpret_cast<float *>(stage);
-#pragma unroll
-      for (int i = 0; i < 16 * MT; ++i)
-        part[i * 32 + lane] = acc.x[i / 16][(i / 4) % 4][i % 4];
-      if (lane == 0) s_neg[warp] = neg;
-      __syncthreads();
-      if (warp == 0) {
-        int sum_p = cnt - 2 * neg;
-        for (int w2 = 1; w2 < nw; ++w2) {
-          const float *op = reinterpret_cast<const float *>(stage + w2 * A.warp_bytes);
-#pragma unroll
-          for (int i = 0; i < 16 * MT; ++i) {
-            float &x = acc.x[i / 16][(i / 4) % 4][i % 4];
-            x = __fadd_rn(x, op[i * 32 + lane]);
-          }
-          sum_p -= 2 * s_neg[w2];
-        }
-        if (FUSED) {
-          finalize_tile<MT>(acc, Pw, b0);
-          exact_bins(A, sum_p, 32 * b0, min(A.N, 32 * (b0 + 8 * MT)), Pw);
-        } else {
-          store_tile<MT>(A, acc, a, b0, sum_p);
-        }
-        __syncwarp();
-      }
-      __syncthreads();
-    }
-    if (FUSED && warp == 0) {
-      CombOut o = comb_warp<NW>(Pw, A.cc, stage);
-      store_scores<NW>(A, v, a, key, o);
-    }
-    __syncthreads();
-  }
+  listed_pixels<MT, NW, FUSED>(A, stage, s_item, s_neg);
 
   if constexpr (!FUSED) {
     light_stream<MT>(A, stage);
@@ -661,11 +831,35 @@ __global__ void __launch_bounds__(256, 2) k_blocked(BlockedArgs A) {
       const uint32_t key = __shfl_sync(0xffffffffu, m_key, q);
       const uint32_t *evp = reinterpret_cast<const uint32_t *>(
           __shfl_sync(0xffffffffu, reinterpret_cast<uintptr_t>(m_ev), q));
-      if (cnt < 0 || cnt >= A.heavy_min) continue;  // inactive, past the end, or heavy
+      if (cnt < 0 || cnt >= A.light_max) continue;  // inactive, past the end, or listed
       pixel_spectrum_warp<MT>(A, evp, cnt, stage, Pw);
       CombOut o = comb_warp<NW>(Pw, A.cc, stage);
       store_scores<NW>(A, A.views[slot], a, key, o);
     }
+  }
+}
+
+// Pixels of kTeamPixel events and fewer than A.heavy_min, which no list holds
+// (the no-allocation entry point, whose fixed scratch lists the larger ones), by
+// teams of four warps, one team per block: each takes 32 active pixels at a time.
+template <int MT>
+__global__ void __launch_bounds__(128, 4) k_team_scan(const __grid_constant__ BlockedArgs A) {
+  extern __shared__ float4 smem4[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned char *stage = reinterpret_cast<unsigned char *>(smem4) + warp * A.warp_bytes;
+  __shared__ int s_neg[4];
+  const SlotView &v = A.views[0];
+  const int64_t n_act = (int64_t)v.counters[2];
+  for (int64_t a0 = 32 * (int64_t)blockIdx.x; a0 < n_act; a0 += 32 * (int64_t)gridDim.x) {
+    int cnt = 0;
+    if (a0 + lane < n_act) {
+      const uint32_t key = v.active[a0 + lane];
+      cnt = (int)(v.offsets[key + 1] - v.offsets[key]);
+    }
+    for (uint32_t m = __ballot_sync(0xffffffffu, cnt >= kTeamPixel && cnt < A.heavy_min); m;
+         m &= m - 1)  // the same pixels in every warp of the block
+      for (int ps = 0; ps < (A.nbr + 8 * MT - 1) / (8 * MT); ++ps)
+        team_item<MT, 1, false, 4>(A, (uint64_t)(a0 + __ffs(m) - 1), ps, stage, warp, 0, s_neg);
   }
 }
 
@@ -689,6 +883,27 @@ int blocked_warp_bytes(const Ctx *c, bool fused, int NW, int *pw_offset) {
   return scratch + (((int)c->gconst.nbr + 8 * MT - 1) / (8 * MT)) * 8 * MT * 32 * 4;
 }
 
+// A grid of `blocks` blocks (rounded down to whole clusters) in clusters of four:
+// with four blocks per SM a cluster divides every GPC's blocks evenly, so none
+// of them is lost.
+constexpr int kCluster = 4;
+template <typename K>
+cudaError_t launch_clusters(K kern, int blocks, int threads, size_t smem, cudaStream_t s,
+                            const BlockedArgs &A) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)std::max(kCluster, blocks / kCluster * kCluster));
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kCluster;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, A);
+}
+
 template <int MT, int NW, bool FUSED>
 ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cudaStream_t s,
                              int slot0 = 0, int64_t ld = 0, int skip_min = 0) {
@@ -700,7 +915,7 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
   A.heavy = c->work;
   A.n_heavy = c->qctl + 0;
   A.heavy_cap = (uint32_t)std::min<int64_t>(c->heavy_cap, 0xffffffffll);
-  A.cursors = c->qctl + 1;
+  A.cursors = c->qctl + 5;
   A.N = c->gconst.N;
   A.nbr = c->gconst.nbr;
   A.nd = make_ndft_const(c->gconst, MT);
@@ -709,7 +924,7 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
   A.ld = ld > 0 ? ld : c->gconst.N;
   A.vec_store = (A.ld % 4 == 0) && (reinterpret_cast<uintptr_t>(P) % 16 == 0);
   A.cap_px = cap_px;
-  A.heavy_min = c->tuning.heavy_min;
+  A.heavy_min = A.light_max = std::min(c->tuning.heavy_min, kTeamPixel);  // as binning lists them
   A.skip_min = skip_min;
   A.warp_bytes = blocked_warp_bytes<MT>(c, FUSED, NW, &A.pw_offset);
   A.flags = c->flags;
@@ -726,9 +941,8 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
     return DDHF_ERR_UNSUPPORTED;
   }
   int bps = c->tuning.blocks_per_sm > 0 ? std::min(occ, c->tuning.blocks_per_sm) : occ;
-  DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl + 1, 0, 2 * sizeof(uint32_t), s));
-  kern<<<c->num_sms * bps, wpb * 32, smem, s>>>(A);
-  DDHF_CUDA_TRY(c, cudaGetLastError());
+  DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl + 5, 0, 3 * sizeof(uint32_t), s));
+  DDHF_CUDA_TRY(c, launch_clusters(kern, c->num_sms * bps, wpb * 32, smem, s, A));
   return DDHF_OK;
 }
 

@@ -17,7 +17,7 @@
 // cudaGetSymbolAddress() once per CUDA context (keyed by the context's
 // process-unique id), during the first call made with that context current.
 // That first call also loads every kernel this entry point can launch (all
-// four tile-count instantiations of the spectrum kernel and the helpers),
+// four tile-count instantiations of the spectrum kernels and the helpers),
 // so that under lazy module loading no later call, whatever its grid, loads
 // code or allocates; it should therefore come before any stream capture and
 // outside any frame budget. Every call shares the array: the counters and
@@ -42,7 +42,7 @@ constexpr int kMaxContexts = 64;
 struct NoAllocScratch {
   SlotView view;
   uint64_t counters[8];  // [2] = number of active pixels
-  uint32_t qctl[4];      // [0] heavy count, [1] heavy cursor, [2] light cursor
+  uint32_t qctl[8];      // [0] heavy count, [1] big count, [2-4] cursors (heavy, light, big)
   uint32_t flags;
   uint32_t pad[3];
   uint64_t heavy[kNoAllocMaxHeavy];  // heavy work items (slot 0 << 32 | active index)
@@ -57,7 +57,7 @@ __global__ void k_noalloc_prepare(NoAllocScratch *s, const uint32_t *ev, const u
     s->view = SlotView{ev, offsets, active, s->counters, nullptr, nullptr, nullptr, nullptr};
     for (int i = 0; i < 8; ++i) s->counters[i] = 0;
     s->counters[2] = (uint64_t)n_active;
-    for (int i = 0; i < 4; ++i) s->qctl[i] = 0;
+    for (int i = 0; i < 8; ++i) s->qctl[i] = 0;
     s->flags = 0;
   }
 }
@@ -71,10 +71,14 @@ __global__ void k_noalloc_heavy(NoAllocScratch *s, const uint32_t *offsets, cons
   for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n_active;
        a += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t k = active[a];
-    if (offsets[k + 1] - offsets[k] >= (uint32_t)kNoAllocHeavyMin) {
-      const uint32_t pos = atomicAdd(&s->qctl[0], 1u);
+    const uint32_t cnt = offsets[k + 1] - offsets[k];
+    if (cnt >= (uint32_t)kNoAllocHeavyMin) {
+      // from the list's front, or (big pixels) from its back: it holds all of
+      // a call whose offsets stay within its events
+      const bool big = cnt >= (uint32_t)kBigPixel;
+      const uint32_t pos = atomicAdd(&s->qctl[big ? 1 : 0], 1u);
       if ((int64_t)pos < kNoAllocMaxHeavy) {
-        s->heavy[pos] = (uint32_t)a;
+        s->heavy[big ? kNoAllocMaxHeavy - 1 - pos : pos] = (uint32_t)a;
       } else {
         atomicOr(&s->flags, DDHF_FLAG_CAPACITY);
         for (int j = 0; j < n_bins; ++j) P[a * n_bins + j] = __int_as_float(0x7fc00000);
@@ -120,7 +124,8 @@ unsigned long long current_ctx_id() {
 template <int MT>
 cudaError_t load_blocked() {
   cudaFuncAttributes fa;
-  return cudaFuncGetAttributes(&fa, blocked::k_blocked<MT, 1, false>);
+  const cudaError_t e = cudaFuncGetAttributes(&fa, blocked::k_blocked<MT, 1, false>);
+  return e != cudaSuccess ? e : cudaFuncGetAttributes(&fa, blocked::k_team_scan<MT>);
 }
 
 // The scratch address for the current context: looked up, and every kernel of
@@ -159,7 +164,7 @@ ddhf_status launch_noalloc(NoAllocScratch *sp, const GridConst &g, float *P, int
   A.heavy = sp->heavy;
   A.n_heavy = &sp->qctl[0];
   A.heavy_cap = (uint32_t)kNoAllocMaxHeavy;
-  A.cursors = &sp->qctl[1];
+  A.cursors = &sp->qctl[2];
   A.N = g.N;
   A.nbr = g.nbr;
   A.nd = blocked::make_ndft_const(g, MT);
@@ -169,6 +174,7 @@ ddhf_status launch_noalloc(NoAllocScratch *sp, const GridConst &g, float *P, int
   A.vec_store = (A.ld % 4 == 0) && (reinterpret_cast<uintptr_t>(P) % 16 == 0);
   A.cap_px = cap_px;
   A.heavy_min = kNoAllocHeavyMin;
+  A.light_max = kTeamPixel;
   A.warp_bytes = blocked::Stage<MT>::kBytes;
   A.flags = &sp->flags;
   A.ev_cap = n_events;
@@ -182,7 +188,14 @@ ddhf_status launch_noalloc(NoAllocScratch *sp, const GridConst &g, float *P, int
           cudaSuccess ||
       occ < 1)
     return DDHF_ERR_CUDA;
-  kern<<<num_sms * occ, kNoAllocWarps * 32, smem, s>>>(A);
+  if (blocked::launch_clusters(kern, num_sms * occ, kNoAllocWarps * 32, smem, s, A) != cudaSuccess)
+    return DDHF_ERR_CUDA;
+  auto scan = blocked::k_team_scan<MT>;
+  if (cudaFuncSetAttribute(scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+      cudaSuccess)
+    return DDHF_ERR_CUDA;
+  const int64_t blocks = std::min<int64_t>(ceil_div(n_active, 32), (int64_t)num_sms * 4);
+  scan<<<(unsigned)blocks, kNoAllocWarps * 32, smem, s>>>(A);
   return cudaGetLastError() == cudaSuccess ? DDHF_OK : DDHF_ERR_CUDA;
 }
 
