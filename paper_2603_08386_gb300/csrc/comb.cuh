@@ -490,7 +490,8 @@ __device__ __forceinline__ CombOut comb_warp_generic(const float *Pw, const Comb
 //    fewer than two candidates per pixel are evaluated on average); the rest
 //    follow in increasing w.
 // Above 1024 bins these steps took over from comb_warp_generic, which scores
-// every candidate in full: 76,800 spectra of 2000 bins 4.95 -> 0.60 ms.
+// every candidate in full: 76,800 spectra of 2000 bins 4.95 -> 0.56 ms, 3,072 of
+// 10,000 bins 3.66 -> 0.38 ms.
 // Two forms share these steps. The register form (512 < N <= 768, M = 4,
 // d = 3: Table 2's comb on the 750-bin grid) gives each lane 24 consecutive
 // bins in registers, so every per-bin pass is a fixed, fully unrolled
@@ -727,29 +728,22 @@ __device__ __noinline__ static void comb_records_any_d(const float *Pw, int N, i
 }
 
 // 32 BPL linear buckets over [0, 1.5 mean) (the fast forms' histogram, with
-// scale = 64 BPL / (3 mean)): x = v scale clamped to the last bucket, bucket
-// floor(x), taken by adding 2^23 rounded down (the float bits then hold
-// floor(x) in the low mantissa bits), so no float-to-integer conversion runs on
-// the special-function pipe. Monotone in v >= 0, so the bins of a bucket range
-// are a range of full ranks, and bucket g0 <= g <= g1 exactly when g0 <= x < g1
-// + 1. Any input (a negative value, NaN) still gives an index below 1024 (BPL
-// 24) or 4096 (96): inside the scratch (the window maxima follow).
+// scale = 64 BPL / (3 mean)): bucket g = floor(v scale) clamped to the last one,
+// as the float 2^23 + g, from one multiply-add to 2^23 rounded down, so no
+// float-to-integer conversion runs on the special-function pipe. Monotone in v
+// >= 0, so the bins of a bucket range are a range of full ranks. Any input (a
+// negative value, NaN) still gives an index below 1024 (BPL 24) or 4096 (96) to
+// hist_add: inside the scratch (the window maxima follow).
 template <int BPL>
-__device__ __forceinline__ float bucket_x(float v, float scale) {
-  return fminf(__fmul_rn(v, scale), (float)(32 * BPL - 1));
+__device__ __forceinline__ float bucket_y(float v, float scale) {
+  return fminf(__fmaf_rd(v, scale, 0x1p23f), 0x1p23f + (float)(32 * BPL - 1));
 }
-template <int BPL>
-__device__ __forceinline__ uint32_t bucket_bits(float v, float scale) {
-  return __float_as_uint(__fadd_rd(bucket_x<BPL>(v, scale), 0x1p23f));  // 0x4B000000 + g
-}
-template <int BPL>
-constexpr uint32_t kBucketMask = BPL == 24 ? 1023u : 4095u;
 
-// Add one to the bucket whose bucket_bits are ybits in the histogram at
-// shared address hist_sa (one counter per bucket).
+// Add one to bucket y in the histogram at shared address hist_sa (one counter
+// per bucket).
 template <int BPL>
-__device__ __forceinline__ void hist_add(uint32_t hist_sa, uint32_t ybits) {
-  const uint32_t a = hist_sa + ((ybits & kBucketMask<BPL>) << 2);
+__device__ __forceinline__ void hist_add(uint32_t hist_sa, float y) {
+  const uint32_t a = hist_sa + ((__float_as_uint(y) & (BPL == 24 ? 1023u : 4095u)) << 2);
   asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(a) : "memory");
 }
 
@@ -795,45 +789,51 @@ __device__ __forceinline__ BandBuckets comb_locate(const uint32_t *hist, int N, 
   const uint32_t lex = warp_excl_scan<uint32_t>(lsum, tot);
   if (tot != (uint32_t)N) bad = true;
   constexpr int K = (BPL + 31) / 32;  // buckets of the found lane per lane now
-  int gsel[2];
-  uint32_t gbelow[2], gcount[2];
+  int src[2], gsel[2];
+  uint32_t gbelow[2], gcount[2], base[2], hk[2][K], h[2];
 #pragma unroll
   for (int t = 0; t < 2; ++t) {
     const uint32_t R = t == 0 ? (uint32_t)lo_r : (uint32_t)hi_r;
-    int src = __ffs(__ballot_sync(0xffffffffu, R >= lex && R < lex + lsum)) - 1;
-    if (src < 0) {
-      src = 0;
+    src[t] = __ffs(__ballot_sync(0xffffffffu, R >= lex && R < lex + lsum)) - 1;
+    if (src[t] < 0) {
+      src[t] = 0;
       bad = true;
     }
-    const uint32_t base = __shfl_sync(0xffffffffu, lex, src);
-    uint32_t hk[K], h = 0;
+    base[t] = __shfl_sync(0xffffffffu, lex, src[t]);
+    h[t] = 0;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      hk[k] = K * lane + k < BPL ? hist[src * BPL + K * lane + k] : 0u;
-      h += hk[k];
+      hk[t][k] = K * lane + k < BPL ? hist[src[t] * BPL + K * lane + k] : 0u;
+      h[t] += hk[t][k];
     }
-    uint32_t t2;
-    uint32_t ex = warp_excl_scan<uint32_t>(h, t2) + base;
-    int s2 = __ffs(__ballot_sync(0xffffffffu, R >= ex && R < ex + h)) - 1;
+  }
+  // both ends' counts (at most 16,384 each) in one scan
+  uint32_t both_tot;
+  const uint32_t both = warp_excl_scan<uint32_t>(h[0] | (h[1] << 16), both_tot);
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    const uint32_t R = t == 0 ? (uint32_t)lo_r : (uint32_t)hi_r;
+    uint32_t ex = (t == 0 ? both & 0xffffu : both >> 16) + base[t], hh = h[t];
+    int s2 = __ffs(__ballot_sync(0xffffffffu, R >= ex && R < ex + hh)) - 1;
     if (s2 < 0) {
       s2 = 0;
       bad = true;
     }
-    gsel[t] = src * BPL + K * s2;
+    gsel[t] = src[t] * BPL + K * s2;
     if constexpr (K > 1) {
       int kk = 0;
-      h = hk[0];
+      hh = hk[t][0];
 #pragma unroll
       for (int k = 1; k < K; ++k)
-        if (R >= ex + h && kk == k - 1) {
-          ex += h;
-          h = hk[k];
+        if (R >= ex + hh && kk == k - 1) {
+          ex += hh;
+          hh = hk[t][k];
           kk = k;
         }
       gsel[t] += __shfl_sync(0xffffffffu, kk, s2);
     }
     gbelow[t] = __shfl_sync(0xffffffffu, ex, s2);
-    gcount[t] = __shfl_sync(0xffffffffu, h, s2);
+    gcount[t] = __shfl_sync(0xffffffffu, hh, s2);
   }
   BandBuckets r;
   r.g0 = gsel[0];
@@ -937,15 +937,10 @@ __device__ __forceinline__ void comb_nw_all(const float *rec, float *nws, const 
       }
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float on = __shfl_xor_sync(0xffffffffu, maxnw, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, maxi, o);
-    if (on > maxnw || (on == maxnw && oi < maxi)) {
-      maxnw = on;
-      maxi = oi;
-    }
-  }
+  // N(w) >= 0 (or -1): its bits order as a signed integer
+  const int top = __reduce_max_sync(0xffffffffu, __float_as_int(maxnw));
+  maxi = __reduce_min_sync(0xffffffffu, __float_as_int(maxnw) == top ? maxi : 0x7fffffff);
+  maxnw = __int_as_float(top);
 }
 
 // Eq. 9-10 for the candidates, each by the whole warp: the one with the
@@ -1102,13 +1097,13 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
   __syncwarp();
   for (int q = lane; q < nfull; q += 32) {
     const float4 v = P4[q];
-    hist_add<BPL>(hist_sa, bucket_bits<BPL>(v.x, scale));
-    hist_add<BPL>(hist_sa, bucket_bits<BPL>(v.y, scale));
-    hist_add<BPL>(hist_sa, bucket_bits<BPL>(v.z, scale));
-    hist_add<BPL>(hist_sa, bucket_bits<BPL>(v.w, scale));
+    hist_add<BPL>(hist_sa, bucket_y<BPL>(v.x, scale));
+    hist_add<BPL>(hist_sa, bucket_y<BPL>(v.y, scale));
+    hist_add<BPL>(hist_sa, bucket_y<BPL>(v.z, scale));
+    hist_add<BPL>(hist_sa, bucket_y<BPL>(v.w, scale));
   }
   if (lane == tail_lane)
-    for (int j = jt; j < N; ++j) hist_add<BPL>(hist_sa, bucket_bits<BPL>(Pw[j], scale));
+    for (int j = jt; j < N; ++j) hist_add<BPL>(hist_sa, bucket_y<BPL>(Pw[j], scale));
   __syncwarp();
 
   // ---- the band: lane p < bw holds the bin at full rank lo_r + p
@@ -1121,7 +1116,7 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
   if (!slow) {
     // this lane's candidates of 1024 bins: bit 4k + u for element u of group
     // lane + 32 k, compacted in lane order; the next 1024 bins behind them
-    const float x0 = (float)bb.g0, x1 = (float)(bb.g1 + 1);
+    const float y0 = 0x1p23f + (float)bb.g0, y1 = 0x1p23f + (float)bb.g1;
     uint32_t *cv = reinterpret_cast<uint32_t *>(scratch + CombFast::kCandV);
     uint16_t *cj = reinterpret_cast<uint16_t *>(scratch + CombFast::kCandJ);
     uint32_t run = 0;
@@ -1135,11 +1130,11 @@ __device__ __forceinline__ CombOut comb_warp_fast_smem(const float *Pw, const Co
         if (q0 + 32 * k < ng && q < ng) {
           const float4 v = P4[q];
           const int j = 4 * q;
-          const float x[4] = {bucket_x<BPL>(v.x, scale), bucket_x<BPL>(v.y, scale),
-                              bucket_x<BPL>(v.z, scale), bucket_x<BPL>(v.w, scale)};
+          const float y[4] = {bucket_y<BPL>(v.x, scale), bucket_y<BPL>(v.y, scale),
+                              bucket_y<BPL>(v.z, scale), bucket_y<BPL>(v.w, scale)};
 #pragma unroll
           for (int u = 0; u < 4; ++u)
-            m |= (x[u] >= x0 && x[u] < x1 && j + u < N ? 1u : 0u) << (4 * k + u);
+            m |= (y[u] >= y0 && y[u] <= y1 && j + u < N ? 1u : 0u) << (4 * k + u);
         }
       }
       uint32_t nsel;
@@ -1273,9 +1268,6 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
   for (int q = 0; q < CombFast::hist_bytes(24) / 512; ++q)
     reinterpret_cast<uint4 *>(hist)[q * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
   __syncwarp();
-#pragma unroll
-  for (int i = 0; i < kB; ++i) hist_add<24>(hist_sa, bucket_bits<24>(v[i], scale));
-  if (npad > 0) atomicSub(&hist[0], (uint32_t)npad);  // bucket 0 is the low half of word 0
   __syncwarp();
 
   // ---- window maxima of the lane's centres from its bins and three bins of
@@ -1308,6 +1300,15 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
     }
   }
 
+  // ---- the histogram; each bin's bucket (2^23 + g) takes its place in v
+#pragma unroll
+  for (int i = 0; i < kB; ++i) {
+    v[i] = bucket_y<24>(v[i], scale);
+    hist_add<24>(hist_sa, v[i]);
+  }
+  if (npad > 0) atomicSub(&hist[0], (uint32_t)npad);
+  __syncwarp();
+
   // ---- the band: lane p < bw holds the bin at full rank lo_r + p
   const int lo_r = cc.lo_r, bw = cc.bw, hi_r = cc.lo_r + cc.bw - 1;
   const BandBuckets bb = comb_locate<24>(hist, N, lo_r, hi_r, bad);
@@ -1316,24 +1317,15 @@ __device__ __forceinline__ CombOut comb_warp_fast_regs(const float *Pw, const Co
   float bv = 0.f;
   int bj = 0;
   if (!slow) {
-    // the lane's candidates as a bit mask over its 24 bins (read back from
-    // shared memory, so that its registers are free for the selection), then
-    // compacted in bin order
+    // the lane's candidates as a bit mask over its 24 bins, then compacted in bin
+    // order (their values read back from the row; reading every bin back instead of
+    // keeping its bucket in a register: 575 against 552 us on 230,400 spectra)
     uint32_t *cv = reinterpret_cast<uint32_t *>(scratch + CombFast::kCandV);
     uint16_t *cj = reinterpret_cast<uint16_t *>(scratch + CombFast::kCandJ);
-    const float x0 = (float)bb.g0, x1 = (float)(bb.g1 + 1);
-    const float4 *P4 = reinterpret_cast<const float4 *>(Pw) + base / 4;
+    const float y0 = 0x1p23f + (float)bb.g0, y1 = 0x1p23f + (float)bb.g1;
     uint32_t m = 0;
 #pragma unroll
-    for (int k = 0; k < kB / 4; ++k) {
-      const float4 t = 4 * k < nval ? P4[k] : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float e[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float x = bucket_x<24>(e[u], scale);
-        m |= (x >= x0 && x < x1 ? 1u : 0u) << (4 * k + u);
-      }
-    }
+    for (int i = 0; i < kB; ++i) m |= (v[i] >= y0 && v[i] <= y1 ? 1u : 0u) << i;
     m &= nval >= kB ? 0xFFFFFFu : (nval > 0 ? (1u << nval) - 1u : 0u);
     uint32_t run;
     uint32_t off = warp_excl_scan<uint32_t>((uint32_t)__popc(m), run);

@@ -13,8 +13,8 @@ namespace ddhf {
 
 // The row is copied to shared memory with all of a lane's loads in flight at
 // once (16-byte loads when the rows are 16-byte aligned), then scored by
-// comb_warp; with spec_smem = 0 (real input only: the register form on
-// 16-byte aligned rows, or the generic comb on a spectrum too large for
+// comb_warp; with spec_smem = 0 (real input only: the register form and
+// the shared-memory form above 1024 bins on 16-byte aligned rows, or the generic comb on a spectrum too large for
 // shared memory) comb_warp reads the row in global memory and shared memory
 // holds its scratch alone. Up to 4 warps per block; the register form is held
 // to 80 registers (24 warps per SM; its 7.4 KB of shared memory per warp at 750
@@ -139,9 +139,12 @@ ddhf_status launch_comb_t(Ctx *c, const float *P, int64_t cap_px, float *log_sf,
   const int spec_b = (c->grid.n_bins * 4 + 15) & ~15;
   int wpb = 4, spec_smem = 1;
   // the register form reads its rows where they are when they are 16-byte
-  // aligned (each lane loads its 96 contiguous bytes; the row stays in L1)
+  // aligned (each lane loads its 96 contiguous bytes; the row stays in L1), and
+  // so does the shared-memory form above 1024 bins, where the row's copy would
+  // halve the warps per SM (76,800 spectra of 2000 bins 596 -> 575 us)
   const int64_t ldv = ld > 0 ? ld : c->grid.n_bins;
-  if (variant == 2 && !CPLX && ldv % 4 == 0 && (reinterpret_cast<uintptr_t>(P) & 15) == 0)
+  const bool in_place = variant == 2 || variant == 4 || variant == 5 || variant >= 14;
+  if (in_place && !CPLX && ldv % 4 == 0 && (reinterpret_cast<uintptr_t>(P) & 15) == 0)
     spec_smem = 0;
   while (spec_smem && wpb > 1 && (spec_b + scratch_b) * wpb > max_smem) wpb >>= 1;
   if (spec_smem && (spec_b + scratch_b) * wpb > max_smem) {
