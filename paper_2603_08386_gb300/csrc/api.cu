@@ -375,8 +375,8 @@ ddhf_status run_detect(Ctx *c, const ddhf_window *wins, int nw, ddhf_box *boxes,
   for (int w = 0; w < nw; ++w) {
     Slot &sl = c->slots[w];
     NvtxRange r("ddhf labels + boxes");
-    DDHF_TRY(launch_label(c, sl.mask, sl.labels, sl.counters + 7, s));
-    DDHF_TRY(launch_boxes(c, sl.labels, boxes + (int64_t)w * cap, cap, sl.nbox, s));
+    DDHF_TRY(launch_label(c, sl.mask, sl.labels, sl.counters + 7, s, true));
+    DDHF_TRY(launch_boxes(c, sl.labels, boxes + (int64_t)w * cap, cap, sl.nbox, s, true));
     DDHF_CUDA_TRY(c, cudaMemcpyAsync(n_boxes_dev + w, sl.nbox, sizeof(int32_t),
                                      cudaMemcpyDeviceToDevice, s));
     if (masks_out)

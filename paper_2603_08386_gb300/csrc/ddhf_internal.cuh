@@ -361,15 +361,17 @@ ddhf_status launch_fused(Ctx *c, int n_slots, bool write_p, float *P, int64_t ca
                          cudaStream_t s);
 void set_bin_attributes();
 // ccl.cu
+// boxes_follow / after_label: the labelling leaves the box slots initialised in
+// the box workspace for a launch_boxes that comes next
 ddhf_status launch_label(Ctx *c, const uint8_t *mask, int32_t *labels, uint64_t *n_fg,
-                         cudaStream_t s);
+                         cudaStream_t s, bool boxes_follow = false);
 ddhf_status launch_box_f0(Ctx *c, int slot, const ddhf_box *boxes, const int32_t *n_boxes,
                           int32_t cap, int32_t *f0_out, float *snr_out, float *med_hz,
                           cudaStream_t s);
 ddhf_status launch_components(Ctx *c, const int32_t *labels, int32_t row0, ddhf_component *out,
                               int32_t cap, int32_t *n_out, cudaStream_t s);
 ddhf_status launch_boxes(Ctx *c, const int32_t *labels, ddhf_box *boxes, int32_t cap,
-                         int32_t *n_boxes, cudaStream_t s);
+                         int32_t *n_boxes, cudaStream_t s, bool after_label = false);
 
 }  // namespace ddhf
 

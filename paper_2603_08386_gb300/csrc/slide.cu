@@ -658,8 +658,8 @@ ddhf_status ddhf_slide_detect(ddhf_ctx *h, ddhf_box *boxes, int32_t cap, int32_t
   Slot &sl = c->slots[0];
   DDHF_TRY_S(slide_active(c, S, s));
   DDHF_TRY_S(launch_comb_cplx(c, S->F, S->ldF, sl.log_sf, sl.snr, sl.f0, sl.mask, s));
-  DDHF_TRY_S(launch_label(c, sl.mask, sl.labels, sl.counters + 7, s));
-  DDHF_TRY_S(launch_boxes(c, sl.labels, boxes, cap, sl.nbox, s));
+  DDHF_TRY_S(launch_label(c, sl.mask, sl.labels, sl.counters + 7, s, true));
+  DDHF_TRY_S(launch_boxes(c, sl.labels, boxes, cap, sl.nbox, s, true));
   DDHF_CUDA_TRY(c, cudaMemcpyAsync(n_boxes_dev, sl.nbox, sizeof(int32_t),
                                    cudaMemcpyDeviceToDevice, s));
   if (mask_out)
