@@ -124,7 +124,6 @@ void free_all(Ctx *c) {
   F(c->hist);
   F(c->scan_part);
   F(c->seg_lo);
-  F(c->seg_hi);
   F(c->packed);
   for (auto &s : c->slots) {
     F(s.ev);
@@ -480,7 +479,12 @@ ddhf_status ddhf_create(int32_t W, int32_t H, const ddhf_grid *grid, const ddhf_
   derive_constants(c);
   const int64_t npx = c->npx;
   const int64_t nev = std::max<int64_t>(max_events, 1);
-  const int64_t hist_n = (int64_t)(1 << kMaxDigitBits) * c->nchunks;
+  // chunks of a binning: of kBinChunk events, or of kSmallChunk up to half of
+  // the former per SM
+  const int64_t small_chunks = std::min<int64_t>(
+      ceil_div(max_events, kSmallChunk), (int64_t)c->num_sms / 2 * (kBinChunk / kSmallChunk));
+  const int64_t hist_n =
+      (int64_t)(1 << kMaxDigitBits) * std::max<int64_t>(c->nchunks, small_chunks);
   const int64_t scan_n = std::max<int64_t>(hist_n, 2 * (npx + 1));
   const int64_t heavy_cap = (int64_t)max_windows * std::min<int64_t>(npx, ceil_div(nev, 32));
   ddhf_status st = DDHF_OK;
@@ -492,8 +496,8 @@ ddhf_status ddhf_create(int32_t W, int32_t H, const ddhf_grid *grid, const ddhf_
   A(c->valsB, nev);
   A(c->hist, hist_n);
   A(c->scan_part, scan_n / 4000 + 256);
-  A(c->seg_lo, npx);
-  A(c->seg_hi, npx);
+  A(c->seg_lo, 2 * npx);
+  c->seg_hi = c->seg_lo + npx;
   A(c->packed, npx + 1);
   c->slots.resize(max_windows);
   for (int i = 0; i < max_windows && st == DDHF_OK; ++i) {

@@ -4,7 +4,7 @@
 //
 // Design: least-significant-digit radix sort over the key bits in 1-3 passes
 // of <= 11 bits. Each pass is reduce-then-scan: a histogram kernel writes one
-// count per (digit, chunk of 8192 events) in digit-major order, an exclusive
+// count per (digit, chunk of 8192 or 2048 events) in digit-major order, an exclusive
 // scan of that table gives every (digit, chunk) its output offset, and a
 // scatter kernel re-reads its chunk and places each element at
 // offset + (its rank among equal digits earlier in the chunk). The in-chunk
@@ -15,9 +15,10 @@
 // reads the raw (x, y, t, p) arrays directly and packs each kept event into
 // one 32-bit word: tau = t - t0 in bits 0-30, bit 31 set for polarity -1.
 // Per-pixel counts come from segment boundaries of the sorted keys, and one
-// 64-bit scan of (count << 32 | active flag) gives both the CSR offsets and
-// the active-pixel list.
+// 64-bit scan of (count << 32 | active flag), formed as it is scanned, gives both
+// the CSR offsets and the active-pixel list.
 #include <algorithm>
+#include <type_traits>
 
 #include "ddhf_internal.cuh"
 
@@ -62,19 +63,19 @@ template <bool RAW>
 __global__ void __launch_bounds__(kBinThreads) k_hist(RawIn raw, const uint32_t *__restrict__ kin,
                                                       const uint32_t *__restrict__ n_dev,
                                                       uint32_t *__restrict__ hist, int64_t nchunks,
-                                                      int shift, int nb) {
+                                                      int chunk_n, int shift, int nb) {
   __shared__ uint32_t sh[1 << kMaxDigitBits];
   constexpr int kU = 8;  // elements per thread with their loads in flight together
   const int64_t n = RAW ? raw.n : (int64_t)*n_dev;
   const int64_t chunk = blockIdx.x;
-  const int64_t c0 = chunk * kBinChunk;
+  const int64_t c0 = chunk * chunk_n;
   for (int d = threadIdx.x; d < nb; d += blockDim.x) sh[d] = 0;
   __syncthreads();
-  const int64_t c1 = min(n, c0 + (int64_t)kBinChunk);
-  if (!RAW && c1 - c0 == kBinChunk && (reinterpret_cast<uintptr_t>(kin) & 15) == 0) {
+  const int64_t c1 = min(n, c0 + (int64_t)chunk_n);
+  if (!RAW && c1 - c0 == chunk_n && (reinterpret_cast<uintptr_t>(kin) & 15) == 0) {
     // a whole chunk of sort words: 16-byte loads, 4 keys each, 8 per thread and step
     const uint4 *k4 = reinterpret_cast<const uint4 *>(kin + c0);
-    for (int q = threadIdx.x; q < kBinChunk / 4; q += 2 * kBinThreads) {
+    for (int q = threadIdx.x; q < chunk_n / 4; q += 2 * kBinThreads) {
       const uint4 a = k4[q];
       const uint4 b = k4[q + kBinThreads];
       const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
@@ -117,16 +118,16 @@ template <bool VEC>
 __global__ void __launch_bounds__(kBinThreads) k_hist_pack(RawIn raw, uint32_t *__restrict__ pk,
                                                            uint32_t *__restrict__ pv,
                                                            uint32_t *__restrict__ hist,
-                                                           int64_t nchunks, int nb) {
+                                                           int64_t nchunks, int chunk_n, int nb) {
   __shared__ uint32_t sh[1 << kMaxDigitBits];
   const int64_t n = raw.n;
   const int64_t chunk = blockIdx.x;
-  const int64_t c0 = chunk * kBinChunk;
+  const int64_t c0 = chunk * chunk_n;
   for (int d = threadIdx.x; d < nb; d += blockDim.x) sh[d] = 0;
   __syncthreads();
-  const int64_t c1 = min(n, c0 + (int64_t)kBinChunk);
+  const int64_t c1 = min(n, c0 + (int64_t)chunk_n);
   const uint32_t mask = (uint32_t)(nb - 1);
-  // 4 consecutive events per thread and step; 8 steps cover the chunk
+  // 4 consecutive events per thread and step
   for (int64_t e0 = c0 + 4 * (int64_t)threadIdx.x; e0 < c1; e0 += 4 * kBinThreads) {
     uint32_t key[4], val[4];
     bool kept[4];
@@ -229,13 +230,13 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t *a, int n, uint32_t
 // warp's rows): one; splitting the rows into two interleaved chains measured
 // slower.
 __host__ __device__ constexpr int scatter_chains(int) { return 1; }
-__host__ __device__ constexpr int scatter_union_words(int nb) {
-  return (kScatThreads / 32) * scatter_chains(nb) * nb / 2 > 2 * kBinChunk
+__host__ __device__ constexpr int scatter_union_words(int nb, int chunk) {
+  return (kScatThreads / 32) * scatter_chains(nb) * nb / 2 > 2 * chunk
              ? (kScatThreads / 32) * scatter_chains(nb) * nb / 2
-             : 2 * kBinChunk;
+             : 2 * chunk;
 }
-__host__ __device__ constexpr int scatter_smem_bytes(int nb) {
-  return (scatter_union_words(nb) + 2 * nb + kBinChunk) * 4;
+__host__ __device__ constexpr int scatter_smem_bytes(int nb, int chunk) {
+  return (scatter_union_words(nb, chunk) + 2 * nb + chunk) * 4;
 }
 
 // Asynchronous global -> shared copies (cp.async), `bytes` of `size` read.
@@ -251,9 +252,10 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// Stable scatter of one chunk of 8192 (key, value) elements. Warp w holds the
-// chunk's keys [512 w, 512 (w + 1)) as 16 rows of 32 consecutive keys (lane l
-// of row i: element 512 w + 32 i + l), so the order (warp, row, lane) is input
+// Stable scatter of one chunk of 512 ITEMS (key, value) elements (8192, or 2048
+// for few events, see bin_core). Warp w holds the chunk's keys [32 ITEMS w, 32
+// ITEMS (w + 1)) as ITEMS rows of 32 consecutive keys (lane l of row i: element
+// 32 ITEMS w + 32 i + l), so the order (warp, row, lane) is input
 // order; the values go to shared memory in input order by asynchronous copies
 // meanwhile. Ranking: row by row, each element's rank among the warp's earlier
 // elements of its digit is a per-warp counter (shared memory, 16 bits) plus
@@ -268,31 +270,32 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // marks one that is not kept; otherwise all n_total elements are kept.
 // n_total: kept elements of the whole array (the table's sum). BITS: digit
 // width (nb = 2^BITS), a template argument so that the ballots unroll.
-template <bool DROP, int BITS>
+template <bool DROP, int BITS, int ITEMS>
 __global__ void __launch_bounds__(kScatThreads, 2) k_scatter(
     const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, int64_t n_in,
     const uint32_t *__restrict__ n_total, uint32_t *__restrict__ kout,
     uint32_t *__restrict__ vout, const uint32_t *__restrict__ hscan, int64_t nchunks,
     int shift, uint32_t *flags) {
   constexpr int kWarps = kScatThreads / 32;
+  constexpr int kChunk = kScatThreads * ITEMS;
   constexpr int nb = 1 << BITS;
   constexpr int kCh = scatter_chains(nb);            // counter tables per warp
   constexpr int kVW = kWarps * kCh;                   // virtual warps, in input order
-  constexpr int kRows = kScatItems / kCh;             // rows per chain
+  constexpr int kRows = ITEMS / kCh;             // rows per chain
   constexpr uint32_t mask = (uint32_t)(nb - 1);
   extern __shared__ uint32_t sm[];
   uint16_t *cnt = reinterpret_cast<uint16_t *>(sm);  // [kVW][nb], then chunk positions
-  uint32_t *sk = sm;                                  // [kBinChunk] staged keys
-  uint32_t *sv = sm + kBinChunk;                      // [kBinChunk] staged values
-  uint32_t *lst = sm + scatter_union_words(nb);       // [nb] start of each digit in the chunk
+  uint32_t *sk = sm;                                  // [kChunk] staged keys
+  uint32_t *sv = sm + kChunk;                      // [kChunk] staged values
+  uint32_t *lst = sm + scatter_union_words(nb, kChunk);       // [nb] start of each digit in the chunk
   uint32_t *gofs = lst + nb;                          // [nb] output offset minus the start
-  uint32_t *vbuf = gofs + nb;                         // [kBinChunk] values in input order
+  uint32_t *vbuf = gofs + nb;                         // [kChunk] values in input order
   __shared__ uint32_t scan_tmp[kWarps];
   const int64_t n = DROP ? n_in : (int64_t)*n_total;
   const int64_t chunk = blockIdx.x;
-  const int64_t c0 = chunk * kBinChunk;
+  const int64_t c0 = chunk * kChunk;
   if (c0 >= n) return;
-  const int nloc = (int)min((int64_t)kBinChunk, n - c0);  // elements of this chunk
+  const int nloc = (int)min((int64_t)kChunk, n - c0);  // elements of this chunk
   // values -> vbuf (16-byte copies when the array is aligned for them)
   const uint32_t vbuf_sa = (uint32_t)__cvta_generic_to_shared(vbuf);
   if ((reinterpret_cast<uintptr_t>(vin) & 15) == 0) {
@@ -316,11 +319,11 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_scatter(
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1;
   uint16_t *my = cnt + warp * kCh * nb;  // chain h of this warp: my + h * nb
-  const int wloc = warp * (32 * kScatItems) + lane;  // local index of row 0
+  const int wloc = warp * (32 * ITEMS) + lane;  // local index of row 0
   // ps: two 16-bit ranks (then chunk positions, < 8192) per register
-  uint32_t kk[kScatItems], ps[kScatItems / 2], ok = 0;
+  uint32_t kk[ITEMS], ps[ITEMS / 2], ok = 0;
 #pragma unroll
-  for (int i = 0; i < kScatItems; ++i) {
+  for (int i = 0; i < ITEMS; ++i) {
     const int l = wloc + 32 * i;
     const uint32_t key = l < nloc ? kin[c0 + l] : kDropKey;
     const bool kept = l < nloc && (!DROP || key != kDropKey);
@@ -367,22 +370,22 @@ __global__ void __launch_bounds__(kScatThreads, 2) k_scatter(
   }
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < kScatItems; ++i)
+  for (int i = 0; i < ITEMS; ++i)
     if ((ok >> i) & 1u)
       ps[i / 2] += (uint32_t)my[(i / kRows) * nb + ((kk[i] >> shift) & mask)] << (16 * (i & 1));
   cp_async_wait_all();
   __syncthreads();  // counters read, values arrived
 #pragma unroll
-  for (int i = 0; i < kScatItems; ++i) {
+  for (int i = 0; i < ITEMS; ++i) {
     const uint32_t pos = (ps[i / 2] >> (16 * (i & 1))) & 0xffffu;
-    if (((ok >> i) & 1u) && ddhf_check(pos < (uint32_t)kBinChunk, flags)) {
+    if (((ok >> i) & 1u) && ddhf_check(pos < (uint32_t)kChunk, flags)) {
       sk[pos] = kk[i];
       sv[pos] = vbuf[wloc + 32 * i];
     }
   }
   __syncthreads();
   // staged chunk out: consecutive slots of one digit go to consecutive addresses
-  for (uint32_t sl = threadIdx.x; sl < m && sl < (uint32_t)kBinChunk; sl += kScatThreads) {
+  for (uint32_t sl = threadIdx.x; sl < m && sl < (uint32_t)kChunk; sl += kScatThreads) {
     const uint32_t key = sk[sl];
     const uint32_t dest = gofs[(key >> shift) & mask] + sl;
     if (dest < total) {  // always true when the counts agree with the table
@@ -429,66 +432,6 @@ __global__ void k_seg(const uint32_t *__restrict__ keys, const uint32_t *__restr
       if (i == 0 || k[u - 1] != kk) seg_lo[kk] = (uint32_t)i;
       if (i == n - 1 || k[u + 1] != kk) seg_hi[kk] = (uint32_t)(i + 1);
     }
-  }
-}
-
-__global__ void k_pack(const uint32_t *__restrict__ seg_lo, const uint32_t *__restrict__ seg_hi,
-                       uint64_t *__restrict__ packed, int64_t npx, int n_min) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k <= npx;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t v = 0;
-    if (k < npx) {
-      uint32_t cnt = seg_hi[k] - seg_lo[k];
-      v = ((uint64_t)cnt << 32) | (cnt >= (uint32_t)n_min ? 1u : 0u);
-    }
-    packed[k] = v;
-  }
-}
-
-__global__ void k_finish(const uint64_t *__restrict__ scanned, const uint32_t *__restrict__ seg_lo,
-                         const uint32_t *__restrict__ seg_hi, uint32_t *__restrict__ offsets,
-                         uint32_t *__restrict__ active, uint64_t *__restrict__ counters,
-                         int64_t npx, int n_min, int heavy_min, int big_min, int64_t n_in,
-                         int64_t n_bins, uint64_t *__restrict__ heavy_list,
-                         uint32_t *heavy_count, uint32_t slot, int64_t heavy_cap,
-                         uint32_t *flags) {
-  uint64_t terms = 0;
-  uint32_t heavy = 0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k <= npx;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t v = scanned[k];
-    offsets[k] = (uint32_t)(v >> 32);
-    if (k < npx) {
-      uint32_t cnt = seg_hi[k] - seg_lo[k];
-      if (cnt >= (uint32_t)n_min) {
-        active[(uint32_t)v] = (uint32_t)k;
-        terms += (uint64_t)cnt * (uint64_t)n_bins;
-        if (cnt >= (uint32_t)heavy_min) {
-          heavy += 1u;
-          // heavy pixels from the list's front, big ones from its back (the list
-          // holds every pixel of at least heavy_min events)
-          const bool big = cnt >= (uint32_t)big_min;
-          const uint32_t pos = atomicAdd(heavy_count + (big ? 1 : 0), 1u);
-          if ((int64_t)pos < heavy_cap)
-            heavy_list[big ? heavy_cap - 1 - pos : pos] = ((uint64_t)slot << 32) | (uint32_t)v;
-          else
-            atomicOr(flags, DDHF_FLAG_CAPACITY);
-        }
-      }
-    } else {
-      counters[0] = v >> 32;                       // n_valid
-      counters[1] = (uint64_t)n_in - (v >> 32);    // n_dropped
-      counters[2] = (uint32_t)v;                   // n_active
-      counters[3] = (uint64_t)n_in;
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    terms += __shfl_xor_sync(0xffffffffu, terms, o);
-    heavy += __shfl_xor_sync(0xffffffffu, heavy, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    if (terms) atomicAdd((unsigned long long *)&counters[5], (unsigned long long)terms);
-    if (heavy) atomicAdd((unsigned long long *)&counters[4], (unsigned long long)heavy);
   }
 }
 
@@ -598,6 +541,96 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_prefixed(const T *in, T *
     *total_out = pre_total + tile_total;
 }
 
+// Per pixel (count << 32 | active flag) from the segment bounds; entry npx is 0.
+__device__ __forceinline__ uint64_t seg_word(const uint32_t *seg_lo, const uint32_t *seg_hi,
+                                             int64_t k, int64_t npx, int n_min) {
+  if (k >= npx) return 0;
+  const uint32_t cnt = seg_hi[k] - seg_lo[k];
+  return ((uint64_t)cnt << 32) | (cnt >= (uint32_t)n_min ? 1u : 0u);
+}
+
+// Sum of each tile of kScanTile pixels' words.
+__global__ void __launch_bounds__(kScanThreads) k_seg_sum(const uint32_t *__restrict__ seg_lo,
+                                                          const uint32_t *__restrict__ seg_hi,
+                                                          uint64_t *__restrict__ part, int64_t npx,
+                                                          int n_min) {
+  __shared__ uint64_t ws[33];
+  const int64_t t0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x;
+  uint64_t v = 0;
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i)
+    v += seg_word(seg_lo, seg_hi, t0 + i * kScanThreads, npx, n_min);
+  uint64_t total;
+  block_exclusive_scan<uint64_t>(v, ws, total);
+  if (threadIdx.x == 0) part[blockIdx.x] = total;
+}
+
+// The CSR offsets, the active list, the heavy list and the counters: each tile's
+// words again (they are cheaper to form twice than to store and load: 36 -> 18 us
+// with their own pack, scan and finish passes on 921,600 pixels), scanned from
+// the sum of the tiles before it.
+__global__ void __launch_bounds__(kScanThreads) k_seg_finish(
+    const uint32_t *__restrict__ seg_lo, const uint32_t *__restrict__ seg_hi,
+    const uint64_t *__restrict__ part, uint32_t *__restrict__ offsets,
+    uint32_t *__restrict__ active, uint64_t *__restrict__ counters, int64_t npx, int n_min,
+    int heavy_min, int big_min, int64_t n_in, int64_t n_bins, uint64_t *__restrict__ heavy_list,
+    uint32_t *heavy_count, uint32_t slot, int64_t heavy_cap, uint32_t *flags) {
+  __shared__ uint64_t ws[33];
+  uint64_t pre = 0;
+  for (int64_t j = threadIdx.x; j < (int64_t)blockIdx.x; j += kScanThreads) pre += part[j];
+  uint64_t pre_total;
+  block_exclusive_scan<uint64_t>(pre, ws, pre_total);
+  __syncthreads();  // ws is reused below
+  const int64_t t0 = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
+  uint64_t v[kScanItems], sum = 0;
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    v[i] = seg_word(seg_lo, seg_hi, t0 + i, npx, n_min);
+    sum += v[i];
+  }
+  uint64_t tile_total;
+  uint64_t ex = block_exclusive_scan<uint64_t>(sum, ws, tile_total) + pre_total;
+  uint64_t events = 0;
+  uint32_t heavy = 0;
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    const int64_t k = t0 + i;
+    if (k <= npx) offsets[k] = (uint32_t)(ex >> 32);
+    if (k == npx) {
+      counters[0] = ex >> 32;                     // n_valid
+      counters[1] = (uint64_t)n_in - (ex >> 32);  // n_dropped
+      counters[2] = (uint32_t)ex;                 // n_active
+      counters[3] = (uint64_t)n_in;
+    }
+    if (v[i] & 1u) {
+      const uint32_t cnt = (uint32_t)(v[i] >> 32);
+      active[(uint32_t)ex] = (uint32_t)k;
+      events += cnt;
+      if (cnt >= (uint32_t)heavy_min) {
+        heavy += 1u;
+        // heavy pixels from the list's front, big ones from its back (the list
+        // holds every pixel of at least heavy_min events)
+        const bool big = cnt >= (uint32_t)big_min;
+        const uint32_t pos = atomicAdd(heavy_count + (big ? 1 : 0), 1u);
+        if ((int64_t)pos < heavy_cap)
+          heavy_list[big ? heavy_cap - 1 - pos : pos] = ((uint64_t)slot << 32) | (uint32_t)ex;
+        else
+          atomicOr(flags, DDHF_FLAG_CAPACITY);
+      }
+    }
+    ex += v[i];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    events += __shfl_xor_sync(0xffffffffu, events, o);
+    heavy += __shfl_xor_sync(0xffffffffu, heavy, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (events)
+      atomicAdd((unsigned long long *)&counters[5], (unsigned long long)events * n_bins);  // terms
+    if (heavy) atomicAdd((unsigned long long *)&counters[4], (unsigned long long)heavy);
+  }
+}
+
 // Exclusive scan; up to kScanDirectTiles tiles by a tile-sum pass and one
 // prefixed scan pass, beyond that recursively (scratch holds the per-level
 // partials). When total is not null, the grand total is written there.
@@ -636,25 +669,26 @@ ddhf_status launch_scan_u64(Ctx *c, const uint64_t *in, uint64_t *out, int64_t n
 }
 
 // k_scatter for a digit width of `bits` (1..kMaxDigitBits).
-template <bool DROP, int BITS = 1>
+template <bool DROP, int ITEMS, int BITS = 1>
 void launch_scatter(int bits, int64_t nch, cudaStream_t s, const uint32_t *kin,
                     const uint32_t *vin, int64_t n_in, const uint32_t *n_total, uint32_t *kout,
                     uint32_t *vout, const uint32_t *hscan, int shift, uint32_t *flags) {
   if constexpr (BITS <= kMaxDigitBits) {
     if (bits != BITS)
-      return launch_scatter<DROP, BITS + 1>(bits, nch, s, kin, vin, n_in, n_total, kout, vout,
-                                            hscan, shift, flags);
-    k_scatter<DROP, BITS><<<(unsigned)nch, kScatThreads, scatter_smem_bytes(1 << BITS), s>>>(
-        kin, vin, n_in, n_total, kout, vout, hscan, nch, shift, flags);
+      return launch_scatter<DROP, ITEMS, BITS + 1>(bits, nch, s, kin, vin, n_in, n_total, kout,
+                                                   vout, hscan, shift, flags);
+    k_scatter<DROP, BITS, ITEMS>
+        <<<(unsigned)nch, kScatThreads, scatter_smem_bytes(1 << BITS, kScatThreads * ITEMS), s>>>(
+            kin, vin, n_in, n_total, kout, vout, hscan, nch, shift, flags);
   }
 }
 
-template <bool DROP, int BITS = 1>
+template <bool DROP, int ITEMS, int BITS = 1>
 void scatter_attributes() {
   if constexpr (BITS <= kMaxDigitBits) {
-    cudaFuncSetAttribute(k_scatter<DROP, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         scatter_smem_bytes(1 << BITS));
-    scatter_attributes<DROP, BITS + 1>();
+    cudaFuncSetAttribute(k_scatter<DROP, BITS, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         scatter_smem_bytes(1 << BITS, kScatThreads * ITEMS));
+    scatter_attributes<DROP, ITEMS, BITS + 1>();
   }
 }
 
@@ -666,7 +700,13 @@ ddhf_status bin_core(Ctx *c, Slot &sl, const RawIn &raw, int n_min, int heavy_mi
   uint32_t *ntot = reinterpret_cast<uint32_t *>(c->qctl + 8);  // n_valid of this binning
   DDHF_CUDA_TRY(c, cudaMemsetAsync(ntot, 0, sizeof(uint32_t), s));
   DDHF_CUDA_TRY(c, cudaMemsetAsync(sl.counters, 0, 7 * sizeof(uint64_t), s));
-  const int64_t nch = ceil_div(n, kBinChunk);
+  // chunks of 8192 events, of 2048 up to half a large chunk per SM (a chunk is a
+  // block's serial work; beyond, the larger tables cost what the spread gains).
+  // The two passes' histograms and scatters: 19k events 26 -> 15 us, 0.57M 42 ->
+  // 27 us, 1.06M 50 -> 51 us
+  const bool few = ceil_div(n, kBinChunk) <= c->num_sms / 2;
+  const int chunk_n = few ? kSmallChunk : kBinChunk;
+  const int64_t nch = ceil_div(n, chunk_n);
   uint32_t *kbuf[2] = {c->keysA, c->keysB};
   uint32_t *vbuf[2] = {c->valsA, c->valsB};
   int shift = 0;
@@ -689,48 +729,52 @@ ddhf_status bin_core(Ctx *c, Slot &sl, const RawIn &raw, int n_min, int heavy_mi
                          (reinterpret_cast<uintptr_t>(raw.p) % 4 == 0);
         if (vec)
           k_hist_pack<true><<<(unsigned)nch, kBinThreads, 0, s>>>(raw, c->keysB, c->valsB,
-                                                                  c->hist, nch, nb);
+                                                                  c->hist, nch, chunk_n, nb);
         else
           k_hist_pack<false><<<(unsigned)nch, kBinThreads, 0, s>>>(raw, c->keysB, c->valsB,
-                                                                   c->hist, nch, nb);
+                                                                   c->hist, nch, chunk_n, nb);
         in.pk = c->keysB;
         in.pv = c->valsB;
       } else if (pass == 0) {
         k_hist<true><<<(unsigned)nch, kBinThreads, 0, s>>>(raw, nullptr, nullptr, c->hist, nch,
-                                                           shift, nb);
+                                                           chunk_n, shift, nb);
       } else {
-        k_hist<false><<<(unsigned)nch, kBinThreads, 0, s>>>(raw, ki, ntot, c->hist, nch, shift,
-                                                            nb);
+        k_hist<false><<<(unsigned)nch, kBinThreads, 0, s>>>(raw, ki, ntot, c->hist, nch, chunk_n,
+                                                            shift, nb);
       }
       DDHF_CUDA_TRY(c, cudaGetLastError());
       // pass 0: the grand total of the table is the number of kept events
       DDHF_CUDA_TRY(c, scan_rec<uint32_t>(c->hist, c->hist, (int64_t)nb * nch, c->scan_part,
                                           pass == 0 ? ntot : nullptr, s));
-      if (pass == 0)
-        launch_scatter<true>(bits, nch, s, in.pk, in.pv, n, ntot, ko, vo, c->hist, shift,
-                             c->flags);
-      else
-        launch_scatter<false>(bits, nch, s, ki, vi, n, ntot, ko, vo, c->hist, shift, c->flags);
+      auto scatter = [&](auto drop, auto items, const uint32_t *k, const uint32_t *v, int64_t nn) {
+        launch_scatter<decltype(drop)::value, decltype(items)::value>(
+            bits, nch, s, k, v, nn, ntot, ko, vo, c->hist, shift, c->flags);
+      };
+      constexpr std::integral_constant<int, kScatItems> large;
+      constexpr std::integral_constant<int, kSmallChunk / kScatThreads> small;
+      if (pass == 0 && few) scatter(std::true_type(), small, in.pk, in.pv, n);
+      else if (pass == 0) scatter(std::true_type(), large, in.pk, in.pv, n);
+      else if (few) scatter(std::false_type(), small, ki, vi, n);
+      else scatter(std::false_type(), large, ki, vi, n);
       DDHF_CUDA_TRY(c, cudaGetLastError());
       shift += bits;
     }
   }
   const uint32_t *kfinal = kbuf[(c->npass - 1) & 1];
-  DDHF_CUDA_TRY(c, cudaMemsetAsync(c->seg_lo, 0, npx * sizeof(uint32_t), s));
-  DDHF_CUDA_TRY(c, cudaMemsetAsync(c->seg_hi, 0, npx * sizeof(uint32_t), s));
+  // both bounds' arrays are one allocation
+  DDHF_CUDA_TRY(c, cudaMemsetAsync(c->seg_lo, 0, 2 * npx * sizeof(uint32_t), s));
   const int sm_blocks = c->num_sms * 8;
   if (nch > 0) {
     k_seg<<<sm_blocks, 256, 0, s>>>(kfinal, ntot, c->seg_lo, c->seg_hi, npx, c->flags);
     DDHF_CUDA_TRY(c, cudaGetLastError());
   }
-  unsigned pb = (unsigned)std::min<int64_t>(ceil_div(npx + 1, 256), sm_blocks);
-  k_pack<<<pb, 256, 0, s>>>(c->seg_lo, c->seg_hi, c->packed, npx, n_min);
-  DDHF_CUDA_TRY(c, cudaGetLastError());
-  DDHF_CUDA_TRY(c, scan_rec<uint64_t>(c->packed, c->packed, npx + 1,
-                                      reinterpret_cast<uint64_t *>(c->scan_part), nullptr, s));
-  k_finish<<<pb, 256, 0, s>>>(c->packed, c->seg_lo, c->seg_hi, sl.offsets, sl.active,
-                              sl.counters, npx, n_min, heavy_min, big_min, n, c->grid.n_bins,
-                              heavy_list, heavy_count, slot_tag, heavy_cap, c->flags);
+  const unsigned tiles = (unsigned)ceil_div(npx + 1, kScanTile);
+  uint64_t *part = reinterpret_cast<uint64_t *>(c->scan_part);
+  k_seg_sum<<<tiles, kScanThreads, 0, s>>>(c->seg_lo, c->seg_hi, part, npx, n_min);
+  k_seg_finish<<<tiles, kScanThreads, 0, s>>>(c->seg_lo, c->seg_hi, part, sl.offsets, sl.active,
+                                              sl.counters, npx, n_min, heavy_min, big_min, n,
+                                              c->grid.n_bins, heavy_list, heavy_count, slot_tag,
+                                              heavy_cap, c->flags);
   DDHF_CUDA_TRY(c, cudaGetLastError());
   return DDHF_OK;
 }
@@ -757,8 +801,10 @@ ddhf_status bin_packed(Ctx *c, Slot &sl, const uint32_t *keys, const uint32_t *v
 }
 
 void set_bin_attributes() {
-  scatter_attributes<true>();
-  scatter_attributes<false>();
+  scatter_attributes<true, kScatItems>();
+  scatter_attributes<false, kScatItems>();
+  scatter_attributes<true, kSmallChunk / kScatThreads>();
+  scatter_attributes<false, kSmallChunk / kScatThreads>();
 }
 
 }  // namespace ddhf

@@ -19,6 +19,7 @@ constexpr int kBinThreads = 256;   // threads of a histogram block (one chunk)
 constexpr int kScatThreads = 512;  // threads of a scatter block (one chunk, 16 warps)
 constexpr int kScatItems = 16;     // consecutive 32-event rows per scatter warp
 constexpr int kBinChunk = kScatThreads * kScatItems;  // 8192 events
+constexpr int kSmallChunk = 2048;  // the chunk of a binning of few events
 constexpr int kMaxBandWords = 8;   // comb rank band up to 256 positions
 constexpr uint32_t kSignBit = 0x80000000u;
 constexpr size_t kCanaryBytes = 256;        // guard region on each side of a buffer
@@ -151,9 +152,9 @@ struct Ctx {
   int64_t nchunks = 0;
   // sort scratch
   uint32_t *keysA = nullptr, *valsA = nullptr, *keysB = nullptr, *valsB = nullptr;
-  uint32_t *hist = nullptr;      // [2048 * nchunks]
+  uint32_t *hist = nullptr;      // [2048 * chunks]
   uint32_t *scan_part = nullptr; // block partials of the scans
-  uint32_t *seg_lo = nullptr, *seg_hi = nullptr;  // [npx]
+  uint32_t *seg_lo = nullptr, *seg_hi = nullptr;  // [npx] each, one allocation
   uint64_t *packed = nullptr;    // [npx + 1]
   // per-window slots
   std::vector<Slot> slots;
