@@ -70,7 +70,11 @@ struct SoftArgs {
 };
 
 constexpr uint64_t kD9 = 1000000000ull;
-constexpr int kGroupMax = 96;  // events of a pixel up to which lane groups take a harmonic each
+// Events of a pixel up to which lane groups take a harmonic each. Forward and
+// adjoint, 640x480 pixels of a textured scene / of Pareto noise, 6 harmonics,
+// Q = 3: limit 32 1.11 / 2.48 ms, 96 0.97 / 2.39, 256 0.96 / 2.38, none 0.98 /
+// up to a third more on the noise, whose longest pixels then run alone.
+constexpr int kGroupMax = 96;
 
 // Harmonic h's first frequency (q = -Q) of a pixel: integer mHz mod 1e9, the
 // rest in Hz, and the phase f tau_c in cycles.
@@ -127,17 +131,16 @@ __device__ __forceinline__ void soft_event(const SoftArgs &A, const SoftFreq &f,
 }
 
 // Events l, l + 32, ... of a pixel (one lane of the warp-wide order) into x.
-template <int NJ, bool BWD>
+template <int KQ, bool BWD>
 __device__ __forceinline__ void soft_lane(const SoftArgs &A, const SoftFreq &f, const uint32_t *ev,
-                                          int l, int cnt, int nq,
-                                          float (&x)[BWD ? 4 : 2][8 * NJ]) {
+                                          int l, int cnt, int nq, float (&x)[BWD ? 4 : 2][KQ]) {
 #pragma unroll 1
   for (int k = l; k < cnt; k += 32) {
     float2 z, u;
     float wtt;
     soft_event(A, f, ev[k], z, u, wtt);
 #pragma unroll
-    for (int q = 0; q < 8 * NJ; ++q) {
+    for (int q = 0; q < KQ; ++q) {
       if (q < nq) {
         x[0][q] += z.x;
         x[1][q] += z.y;
@@ -151,14 +154,16 @@ __device__ __forceinline__ void soft_lane(const SoftArgs &A, const SoftFreq &f, 
   }
 }
 
-// NJ: blocks of eight frequencies, 8 NJ >= 2Q+1. Bound by
-// instruction issue (76 %). Measured on 153,600 pixels of a 640x480 window (6
-// harmonics, Q = 3): forward 0.870 -> 0.378 ms, forward and backward with the
+// NJ blocks of eight frequencies and EX = 1 more, 8 NJ + EX >= 2Q+1: 9 and 17
+// frequencies with a whole block for the last one padded a third of the work
+// away (Q = 8, 6 harmonics: 1.12 ms, 0.97 so; one butterfly per frequency 0.98).
+// Bound by instruction issue (76 %). Measured on 153,600 pixels of a 640x480
+// window (6 harmonics, Q = 3): forward 0.870 -> 0.378 ms, both ways with the
 // gradient sums 2.29 -> 0.96 ms, the same bits.
-template <int NJ, bool BWD>
+template <int NJ, int EX, bool BWD>
 __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
   constexpr int kC = BWD ? 4 : 2;  // components: F re, im, and D re, im for the backward pass
-  constexpr int kQ = 8 * NJ;
+  constexpr int kQ = 8 * NJ + EX;
   // two sets of sums fit the registers
   constexpr bool kGroups = kC * kQ <= 32;
   __shared__ float sG[kSoftMaxH][kQ];             // G_hq, 0 for q >= 2Q+1
@@ -225,7 +230,7 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
               for (int c = 0; c < kC; ++c)
 #pragma unroll
                 for (int q = 0; q < kQ; ++q) y[c][q] = 0.f;
-              soft_lane<NJ, BWD>(A, f, A.ev + o0, (lane & 7) + 8 * half + 16 * p, cnt, nq, y);
+              soft_lane<kQ, BWD>(A, f, A.ev + o0, (lane & 7) + 8 * half + 16 * p, cnt, nq, y);
 #pragma unroll
               for (int c = 0; c < kC; ++c)
 #pragma unroll
@@ -238,7 +243,7 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
           }
         }
       } else {
-        soft_lane<NJ, BWD>(A, f, A.ev + o0, lane, cnt, nq, x);
+        soft_lane<kQ, BWD>(A, f, A.ev + o0, lane, cnt, nq, x);
 #pragma unroll 1
         for (int o = 16; o >= 8; o >>= 1)
 #pragma unroll
@@ -266,11 +271,21 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
             }
           y[c][j] = v[0];
         }
-      float P[NJ], Pd[NJ];
+      // the frequency beyond the blocks: whole, in every lane
+      if constexpr (EX != 0)
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        P[j] = y[0][j] * y[0][j] + y[1][j] * y[1][j];
-        if constexpr (BWD) Pd[j] = 2.f * (y[0][j] * y[2][j] + y[1][j] * y[3][j]);
+        for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+          for (int c = 0; c < kC; ++c)
+            x[c][8 * NJ] += __shfl_xor_sync(0xffffffffu, x[c][8 * NJ], o);
+      float P[NJ + EX], Pd[NJ + EX];
+#pragma unroll
+      for (int j = 0; j < NJ + EX; ++j) {
+        float v[kC];
+#pragma unroll
+        for (int c = 0; c < kC; ++c) v[c] = j < NJ ? y[c][j < NJ ? j : 0] : x[c][kQ - 1];
+        P[j] = v[0] * v[0] + v[1] * v[1];
+        if constexpr (BWD) Pd[j] = 2.f * (v[0] * v[2] + v[1] * v[3]);
       }
       // sums over q, in order, by every lane of the group
       const float wh = A.w[h], Z = sZ[h];
@@ -278,9 +293,11 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
 #pragma unroll
       for (int q = 0; q < kQ; ++q) {
         const int src = (lane & 24) + (q & 7);
-        const float Pq = __shfl_sync(0xffffffffu, P[q / 8], src);
-        float Pdq = 0.f;
-        if constexpr (BWD) Pdq = __shfl_sync(0xffffffffu, Pd[q / 8], src);
+        float Pq = P[q / 8], Pdq = BWD ? Pd[q / 8] : 0.f;
+        if (q < 8 * NJ) {
+          Pq = __shfl_sync(0xffffffffu, Pq, src);
+          if constexpr (BWD) Pdq = __shfl_sync(0xffffffffu, Pdq, src);
+        }
         if (q < nq) {
           const float G = sG[h][q];
           Ac += G * Pq;
@@ -297,9 +314,9 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
         if (A.g_f && h_ok && (grouped || lane < 8)) {
           // per evaluation frequency: g dS/df_hq = g w_h G_hq P'(f_hq) / (Z_h B)
 #pragma unroll
-          for (int j = 0; j < NJ; ++j) {
+          for (int j = 0; j < NJ + EX; ++j) {
             const int q = 8 * j + (lane & 7);
-            if (q < nq)
+            if (q < nq)  // of the frequency beyond the blocks, lane 0 alone
               A.g_f[(a * A.n_h + h) * (int64_t)nq + q] = gs * (wh * sG[h][q] * Pd[j] / (Z * Bv));
           }
         }
@@ -354,10 +371,10 @@ __global__ void __launch_bounds__(256) k_col_sum(const float *part, int64_t n_ro
   }
 }
 
-template <int NJ>
+template <int NJ, int EX>
 cudaError_t launch_soft(const SoftArgs &A, bool bwd, int blocks, cudaStream_t s) {
-  if (bwd) k_softcomb<NJ, true><<<blocks, 256, 0, s>>>(A);
-  else k_softcomb<NJ, false><<<blocks, 256, 0, s>>>(A);
+  if (bwd) k_softcomb<NJ, EX, true><<<blocks, 256, 0, s>>>(A);
+  else k_softcomb<NJ, EX, false><<<blocks, 256, 0, s>>>(A);
   return cudaGetLastError();
 }
 
@@ -493,11 +510,11 @@ extern "C" ddhf_status ddhf_softcomb(ddhf_ctx *h, int64_t n_px, const uint32_t *
   A.cursor = c->qctl + 4;
   DDHF_CUDA_TRY(c, cudaMemsetAsync(A.cursor, 0, sizeof(uint32_t), s));
   const int blocks = (int)std::min<int64_t>(ceil_div(n_px, 8), (int64_t)c->num_sms * 16);
-  switch ((2 * Q + 1 + 7) / 8) {
-    case 1: DDHF_CUDA_TRY(c, launch_soft<1>(A, bwd, blocks, s)); break;
-    case 2: DDHF_CUDA_TRY(c, launch_soft<2>(A, bwd, blocks, s)); break;
-    default: DDHF_CUDA_TRY(c, launch_soft<3>(A, bwd, blocks, s)); break;
-  }
+  const int nq = 2 * Q + 1;
+  if (nq <= 8) DDHF_CUDA_TRY(c, (launch_soft<1, 0>(A, bwd, blocks, s)));
+  else if (nq == 9) DDHF_CUDA_TRY(c, (launch_soft<1, 1>(A, bwd, blocks, s)));
+  else if (nq <= 16) DDHF_CUDA_TRY(c, (launch_soft<2, 0>(A, bwd, blocks, s)));
+  else DDHF_CUDA_TRY(c, (launch_soft<2, 1>(A, bwd, blocks, s)));
   if (bwd) k_col_sum<<<2 * n_h, 256, 0, s>>>(A.part, n_px, grad_w, grad_sigma, n_h);
   DDHF_CUDA_TRY(c, cudaGetLastError());
   return DDHF_OK;
