@@ -361,15 +361,26 @@ __device__ __forceinline__ void exact_bins(const BlockedArgs &A, int sum_p, int 
     if (j >= j_begin && (threadIdx.x & 31) == 0) row[j] = p2;
 }
 
-// Power of the lane's tile into Pw (row-major bins from row_base on).
+// Rows of 32 bins that a fused warp's spectrum takes: whole tiles, but single
+// tiles only up to four rows (the scratch of 640 bins in 4-row steps fits eight
+// warps of a block, 24 rows of it do not).
 template <int MT>
-__device__ __forceinline__ void finalize_tile(const Acc<MT> &acc, float *Pw, int row_base) {
+__host__ __device__ inline int spectrum_rows(int nbr) {
+  const int unit = MT == 1 ? 4 : 8 * MT;
+  return (nbr + unit - 1) / unit * unit;
+}
+
+// Power of the lane's tile into Pw (row-major bins from row_base on, nbr rows).
+template <int MT>
+__device__ __forceinline__ void finalize_tile(const Acc<MT> &acc, float *Pw, int row_base,
+                                              int nbr) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
   for (int i = 0; i < MT; ++i) {
     float pp[4], pm[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc.powers(i, q, pp[q], pm[q]);
+    if (MT == 1 && row_base + g >= nbr) return;  // beyond spectrum_rows
     float *row = Pw + (row_base + 8 * i + g) * 32;
     *reinterpret_cast<float4 *>(row + 16 + 4 * t) = make_float4(pp[0], pp[1], pp[2], pp[3]);
     *reinterpret_cast<float4 *>(row + 12 - 4 * t) = make_float4(pm[3], pm[2], pm[1], pm[0]);
@@ -437,7 +448,7 @@ __device__ __forceinline__ void pixel_spectrum_warp(const BlockedArgs &A, const 
     Acc<MT> acc;
     acc.zero();
     const int neg = accumulate<MT>(evp, cnt, 0, 1, A.nd, A.nd.f_row[pass], stage, acc);
-    finalize_tile<MT>(acc, Pw, b0);
+    finalize_tile<MT>(acc, Pw, b0, A.nbr);
     exact_bins(A, cnt - 2 * neg, 32 * b0, min(A.N, 32 * (b0 + 8 * MT)), Pw);
     __syncwarp();
   }
@@ -620,7 +631,7 @@ __device__ __forceinline__ void heavy_store(const BlockedArgs &A, const Acc<MT> 
                                             int ps, int sum_p, float *Pw) {
   const int b0 = ps * 8 * MT;
   if (FUSED) {
-    finalize_tile<MT>(acc, Pw, b0);
+    finalize_tile<MT>(acc, Pw, b0, A.nbr);
     exact_bins(A, sum_p, 32 * b0, min(A.N, 32 * (b0 + 8 * MT)), Pw);
   } else {
     store_tile<MT>(A, acc, a, b0, sum_p);
@@ -880,7 +891,7 @@ int blocked_warp_bytes(const Ctx *c, bool fused, int NW, int *pw_offset) {
   scratch = std::max(scratch, comb_scratch_bytes(c->comb, NW));
   scratch = (scratch + 15) & ~15;
   *pw_offset = scratch;
-  return scratch + (((int)c->gconst.nbr + 8 * MT - 1) / (8 * MT)) * 8 * MT * 32 * 4;
+  return scratch + spectrum_rows<MT>((int)c->gconst.nbr) * 32 * 4;
 }
 
 // A grid of `blocks` blocks (rounded down to whole clusters) in clusters of four:

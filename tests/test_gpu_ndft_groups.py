@@ -78,3 +78,26 @@ def test_blocked_spectra_at_every_edge(nb, a0, da, denom):
     A, _ = _spectra(s, ev, heavy_min=1 << 30)
     B, _ = _spectra(s, ev, heavy_min=1 << 30, warps_per_block=2, blocks_per_sm=1)
     assert torch.equal(A, B) and torch.equal(A[small], P[small])
+
+
+@pytest.mark.parametrize("nb,rows,wpb", [(630, 1, 8), (640, 1, 8), (640, 2, 4), (96, 1, 2),
+                                         (300, 0, 8)])
+def test_fused_spectra_fill_their_shared_rows(nb, rows, wpb):
+    # a comb of 35 bins takes the generic scoring, whose scratch leaves eight
+    # warps of a block just the 20 rows of 640 bins
+    build.build()
+    s = _scene(nb)
+    ev = ddhf.events_to_device(s)
+    out = []
+    for fuse in (1, 0):
+        c = ddhf.Context(s.W, s.H, s.grid, ddhf.default_params(n_min=1, M=5, d=3, tau_sf=1.0),
+                         max_events=s.n)
+        c.set_tuning(fuse=fuse, rows_per_lane=rows, warps_per_block=wpb)
+        mask = c.detect(*ev, s.t0, s.window_us, want_mask=True)[2].clone()
+        sc = {k: c.scores()[k].clone() for k in ("f0_bin", "snr", "log_sf")}
+        c.stats()
+        c.close()
+        out.append((mask, sc))
+    assert torch.equal(out[0][0], out[1][0])
+    for k in out[0][1]:
+        assert torch.equal(out[0][1][k].view(torch.int32), out[1][1][k].view(torch.int32)), k
