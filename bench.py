@@ -11,7 +11,7 @@ region starts (8.3 GB per step, far above L2, so no flush is needed).
 
 Metric: NDFT event-bin terms per second (terms = sum over active pixels of
 event count x bins, the work of Eq. 6), whole job over all ranks; also
-ms per window. Extra keys: roofline of the NDFT kernel (FP32 FMA-pipe bound),
+ms per window. Extra keys: roofline of the NDFT kernel (tensor cores),
 e2e through the C ABI from pinned host buffers, the plain one-warp-per-pixel
 pipeline on the same windows, and the FP64 oracle timed on a sample.
 
@@ -52,12 +52,12 @@ UNIT = "terms/s"
 WORKLOAD = ("C3: {W}x{H}, 8 consecutive 30 ms windows x 4 streams per step, Pareto(1.5) "
             "per-pixel counts capped at 20k, 3 drones; grid 0-1498 Hz step 2 Hz (750 bins); "
             "Table 2 parameters")
-OPS_PER_TERM = 3  # FP32 FMA-pipe lane-ops per term of the blocked three-multiplication form
+OPS_PER_TERM = 4  # FLOP per term of the blocked form (two real multiply-adds)
 # DRAM bytes (read + write) per active pixel of one launch, from one ncu capture
-# of the kernel on a 640x360 window of the same recipe (profiles/), scaled to a
+# of the kernel on one window of the same recipe (profiles/), scaled to a
 # launch by its active pixels (the traffic is per-pixel rows). A figure is
 # listed only while the kernel is the one that was captured.
-TRAFFIC_PER_PIXEL = {"k_comb<2>": 3044.0, "k_blocked<6,1,0>": 2894.0}
+TRAFFIC_PER_PIXEL = {"k_comb<2>": 3026.0, "k_blocked<3,1,0>": 3108.0}
 TRAFFIC_NOTE = ("null: the ncu DRAM capture of this kernel predates its current code "
                 "(profiles/ keeps the earlier figure)")
 
@@ -308,9 +308,10 @@ def measured_peaks():
     try:
         with open(path) as f:
             d = json.load(f)
-        return dict(hbm_gbs=float(d["hbm_gbs"]), source="measured")
+        return dict(hbm_gbs=float(d["hbm_gbs"]), bf16_tflops=float(d["bf16_tflops"]),
+                    source="measured")
     except (OSError, ValueError, KeyError):
-        return dict(hbm_gbs=6800.0, source="fallback")
+        return dict(hbm_gbs=6800.0, bf16_tflops=1900.0, source="fallback")
 
 
 class Clocks:
@@ -701,7 +702,7 @@ def main():
         del lab
     # ------------------------------------------------------------ spectrum forms, one window
     # window 0 alone through ddhf_power_spectrum: the blocked kernel on every
-    # active pixel (the FMA-pipe roofline of that kernel, without the hybrid
+    # active pixel (the roofline of that kernel, without the hybrid
     # split) and the hybrid form, whose heavy pixels take the uniform-grid
     # route (spread + dense product with the shared table)
     forms = None
@@ -716,7 +717,7 @@ def main():
         forms = dict(window="stream 0, window 0", active_pixels=na0,
                      terms=terms_of(w0, W, H, nb))
         # the blocked kernel alone takes every pixel, so its own heavy threshold
-        # (block-per-pixel from heavy_min events) is chosen here among a few
+        # (its pixels are listed and taken first) is chosen here among a few
         # values; the step's tuning picks heavy_min for the pixels that the
         # hybrid route leaves to it
         runs = [("blocked", ddhf.FORM["blocked"], dict(base, hybrid_min=0, heavy_min=h))
@@ -874,40 +875,41 @@ def main():
                                        f"alone, single precision), {secs2:.1f} s wall")
     f_avg = statistics.mean(fused_ms)
     fused_mode = statistics.mean(spec_ms) == 0.0
-    peak = peaks["ffma2_lane_per_s"] / 1e12
+    peak = measured_peaks()["bf16_tflops"]
     hybrid_on = not fused_mode and int(tuning.get("hybrid_min", 0)) > 0
     if fused_mode:
-        ndft_ms, kern = f_avg, "fused blocked NDFT + SF + comb kernel (k_blocked<TB,NW,1>)"
+        ndft_ms, kern = f_avg, "fused blocked NDFT + SF + comb kernel (k_blocked<MT,NW,1>)"
     else:
-        ndft_ms, kern = statistics.mean(spec_ms), "blocked NDFT spectrum kernel (k_blocked<TB,1,0>)"
+        ndft_ms, kern = statistics.mean(spec_ms), "blocked NDFT spectrum kernel (k_blocked<MT,1,0>)"
     achieved = OPS_PER_TERM * terms_step / (ndft_ms * 1e-3) / 1e12
     ndft_launches, ndft_launch_ms = nwin, ndft_ms / nwin
     if hybrid_on and forms:
         # the step's spectrum stage runs the blocked and the hybrid kernels; the
         # blocked kernel's own rate comes from the one-window FORM_BLOCKED run
-        kern = ("blocked NDFT spectrum kernel (k_blocked<TB,1,0>) on every active pixel of "
+        kern = ("blocked NDFT spectrum kernel (k_blocked<MT,1,0>) on every active pixel of "
                 "one window (ddhf_power_spectrum, FORM_BLOCKED)")
         achieved = forms["blocked_tops"]
         ndft_launches, ndft_launch_ms = 1, forms["blocked_ms"]
     elif hybrid_on:
         kern += " with the hybrid grid kernels (spectrum stage time)"
     n_act = sum(active_of(w, W, H) for w in wins)
-    tb = 6 if nb <= 768 and nb > 512 else None  # rows per lane the launcher picks for 750 bins
+    mt = 3 if nb <= 768 and nb > 512 else None  # m-tiles the launcher picks for 750 bins
     # the captured traffic is that of the blocked kernel on every active pixel
     blocked_alone = not fused_mode and (not hybrid_on or bool(forms))
-    tr_ndft = (TRAFFIC_PER_PIXEL["k_blocked<6,1,0>"] * n_act / nwin
-               if ("k_blocked<6,1,0>" in TRAFFIC_PER_PIXEL and blocked_alone and tb == 6
+    tr_ndft = (TRAFFIC_PER_PIXEL["k_blocked<3,1,0>"] * n_act / nwin
+               if ("k_blocked<3,1,0>" in TRAFFIC_PER_PIXEL and blocked_alone and mt == 3
                    and int(tuning.get("rows_per_lane", 0)) in (0, 6))
                else None)
-    roof_ndft = dict(bound="alu", achieved=achieved, peak=peak, unit="Tops/s",
+    roof_ndft = dict(bound="tensor", achieved=achieved, peak=peak, unit="TFLOP/s",
                      frac=achieved / peak, traffic=tr_ndft, traffic_unit="B per launch (window)",
                      traffic_note=None if tr_ndft is not None else TRAFFIC_NOTE,
                      kernel=kern, launches_per_step=ndft_launches, launch_ms=ndft_launch_ms,
                      kernel_ms_per_step=ndft_ms, share_of_step=ndft_ms / ms_step,
-                     peak_source=("measured: ddhf_measure_pipes, paired FP32 FMA (f32x2) "
-                                  f"chains on {peaks['sm_count']} SMs"),
-                     ops="3 FP32 FMA-pipe lane-ops per term (three-multiplication complex "
-                         "product)")
+                     peak_source=measured_peaks()["source"] + " bf16 GEMM rate",
+                     ops="4 FLOP per term (two real multiply-adds; each runs as four FP16 "
+                         "partial products)",
+                     note="bound by the latency of dependent steps at 16 warps per SM, neither "
+                          "by the tensor cores nor by HBM")
     roof_comb = None
     comb_reg = 512 < nb <= 768  # Table 2's M = 4, d = 3 on this grid: the register form
     if not fused_mode:

@@ -134,10 +134,13 @@ typedef struct {
  *           advanced by an exact modular step, then FP32 sin/cos per term.
  *  RECUR    one warp per pixel; each lane rotates its bins by an exact
  *           per-event step phasor, re-seeded exactly every 32 bins.
- *  BLOCKED  persistent kernel: F[32b + r] = sum_k A[b][k] B[k][r] with exact
- *           seeds A = p e^{-2 pi i a_{32b} tau} and rotations B = u^r, as a
- *           three-multiplication complex product per term; heavy pixels are
- *           split over a thread block. The form used by ddhf_detect.
+ *  BLOCKED  persistent kernel: rows of 32 bins around their centre, F[+-s] of
+ *           a row from four real sums over the events, as one real matrix
+ *           product per pixel on the tensor cores; each operand is a pair of
+ *           FP16 words (FP32 accuracy) and its phase an exact 64-bit fraction
+ *           of a turn. Pixels of 256 events or more are split over a team of
+ *           warps, of 2048 or more over several blocks. The form used by
+ *           ddhf_detect.
  *  NAIVE32  precision study only: FP32 phase 2 pi f t from the absolute time.
  *  KAHAN    SINCOS with compensated (Kahan) accumulation.
  *  F64      check path: FP64 phase and accumulation on the GPU.
@@ -167,15 +170,18 @@ typedef struct {
 #define DDHF_FORM_HYBRID 6
 
 /* Launch tuning of the persistent BLOCKED kernel (chosen by the autotuner).
- *  heavy_min   pixels with at least this many events (>= 32) are processed by
- *              a whole thread block (events split over its warps), the others
- *              by one warp each;
+ *  heavy_min   pixels with at least this many events (>= 32) are listed, to be
+ *              taken before the others, by a team of four warps each (events
+ *              split over them; two with 2 warps per block) or, from 2048
+ *              events, by a cluster of four thread blocks. Pixels of 256
+ *              events or more that are not listed go to such a team all the
+ *              same; the others to one warp each;
  *  warps_per_block  warps per thread block (2, 4 or 8);
  *  blocks_per_sm    resident blocks per SM used to size the persistent grid
  *                   (0 = as many as fit);
- *  rows_per_lane    32-bin rows held per lane (1, 2, 4, 6 or 8; 0 = chosen
- *                   from n_bins): a pass covers 4 * rows_per_lane rows, and
- *                   every pass re-seeds the phasor rows exactly;
+ *  rows_per_lane    1, 2, 4, 6 or 8 (0 = chosen from n_bins): a pass over the
+ *                   events covers 8 max(1, rows_per_lane / 2) rows of 32 bins,
+ *                   and every pass takes its phasor rows from exact phases;
  *  fuse             1: ddhf_detect / ddhf_detect_batch score each spectrum in
  *                   the kernel that computes it (spectra stay on chip); 0:
  *                   per window, a spectrum kernel writes a context-owned
