@@ -785,9 +785,8 @@ ddhf_status bin_window(Ctx *c, int slot_i, const int16_t *x, const int16_t *y, c
   sl.t0 = t0;
   sl.window_us = win;
   RawIn raw{x, y, t, p, n, t0, (uint64_t)win, c->W, c->H, c->params.polarity_01, c->row0};
-  return bin_core(c, sl, raw, c->params.n_min, std::min(c->tuning.heavy_min, kTeamPixel),
-                  std::max(c->tuning.heavy_min, kBigPixel), c->work, c->qctl, (uint32_t)slot_i,
-                  c->heavy_cap, s);
+  return bin_core(c, sl, raw, c->params.n_min, list_min(c->tuning), big_min(c->tuning), c->work,
+                  c->qctl, (uint32_t)slot_i, c->heavy_cap, s);
 }
 
 // Stable sort of pre-packed (key, value) pairs into a slot's per-pixel list;

@@ -327,6 +327,13 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
                      __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
 }
 
+// The work list of the spectrum kernel (heavy items from its front, big ones from
+// its back) holds the pixels of at least list_min events; those of at least
+// big_min are the big ones. Whoever fills the list and whoever runs it must take
+// both from the same tuning.
+inline int list_min(const ddhf_tuning &t) { return t.heavy_min < kTeamPixel ? t.heavy_min : kTeamPixel; }
+inline int big_min(const ddhf_tuning &t) { return t.heavy_min > kBigPixel ? t.heavy_min : kBigPixel; }
+
 // ---------------------------------------------------------- launch entry points
 // bin.cu
 ddhf_status bin_window(Ctx *c, int slot, const int16_t *x, const int16_t *y, const int64_t *t,

@@ -915,6 +915,8 @@ cudaError_t launch_clusters(K kern, int blocks, int threads, size_t smem, cudaSt
   return cudaLaunchKernelEx(&cfg, kern, A);
 }
 
+// The caller zeroes the cursors (words 5 to 7 of qctl) and, when the list is not
+// the one of a binning under this tuning, fills it (list_slot0).
 template <int MT, int NW, bool FUSED>
 ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cudaStream_t s,
                              int slot0 = 0, int64_t ld = 0, int skip_min = 0) {
@@ -935,7 +937,7 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
   A.ld = ld > 0 ? ld : c->gconst.N;
   A.vec_store = (A.ld % 4 == 0) && (reinterpret_cast<uintptr_t>(P) % 16 == 0);
   A.cap_px = cap_px;
-  A.heavy_min = A.light_max = std::min(c->tuning.heavy_min, kTeamPixel);  // as binning lists them
+  A.heavy_min = A.light_max = list_min(c->tuning);  // as the list was filled
   A.skip_min = skip_min;
   A.warp_bytes = blocked_warp_bytes<MT>(c, FUSED, NW, &A.pw_offset);
   A.flags = c->flags;
@@ -952,7 +954,6 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
     return DDHF_ERR_UNSUPPORTED;
   }
   int bps = c->tuning.blocks_per_sm > 0 ? std::min(occ, c->tuning.blocks_per_sm) : occ;
-  DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl + 5, 0, 3 * sizeof(uint32_t), s));
   DDHF_CUDA_TRY(c, launch_clusters(kern, c->num_sms * bps, wpb * 32, smem, s, A));
   return DDHF_OK;
 }
