@@ -470,8 +470,9 @@ ddhf_status ddhf_spectrum_median(ddhf_ctx *ctx, const float *P, int64_t rows, fl
  * + j] for a < n_active (cap_px >= n_active required). grid is a host pointer.
  * flags_dev (device uint32, nullable) receives, in stream order after the
  * spectra, the DDHF_FLAG_* bits this call raised: DDHF_FLAG_CAPACITY when its
- * list of heavy pixels overflowed (only possible with offsets beyond
- * n_events; those pixels' rows are NaN).
+ * list of heavy pixels (32,768 entries of at least 1024 events) overflowed,
+ * which takes a key listed many times or offsets beyond n_events; the rows of
+ * the entries that did not fit are NaN, the others are right.
  * Limits: n_events <= 2^25 events in ev, n_active <= 2^26. Larger sizes
  * return DDHF_ERR_INVALID_ARG. Its scratch is one fixed 256 KiB __device__
  * array (kept by every device that loads the library until exit). The first

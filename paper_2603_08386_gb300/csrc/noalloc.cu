@@ -42,7 +42,8 @@ constexpr int kMaxContexts = 64;
 struct NoAllocScratch {
   SlotView view;
   uint64_t counters[8];  // [2] = number of active pixels
-  uint32_t qctl[8];      // [0] heavy count, [1] big count, [2-4] cursors (heavy, light, big)
+  uint32_t qctl[8];      // [0] heavy count, [1] big count, [2-4] cursors (heavy, light, big),
+                         // [5] places of the list asked for
   uint32_t flags;
   uint32_t pad[3];
   uint64_t heavy[kNoAllocMaxHeavy];  // heavy work items (slot 0 << 32 | active index)
@@ -62,10 +63,13 @@ __global__ void k_noalloc_prepare(NoAllocScratch *s, const uint32_t *ev, const u
   }
 }
 
-// Heavy pixels (at least kNoAllocHeavyMin events) into the work list. With
-// offsets that stay within the n_events <= kNoAllocMaxEvents events of the
-// call the list cannot overflow; a pixel that does not fit (offsets beyond
-// n_events) gets a row of NaN and raises DDHF_FLAG_CAPACITY.
+// Heavy pixels (at least kNoAllocHeavyMin events) into the work list, from its
+// front, the big ones from its back. With distinct keys and offsets that stay
+// within the n_events <= kNoAllocMaxEvents events of the call the list cannot
+// overflow. A pixel that does not fit (more than kNoAllocMaxHeavy entries of both
+// classes together: keys listed many times, or offsets beyond n_events) gets a
+// row of NaN and raises DDHF_FLAG_CAPACITY. A place is asked for before an end is
+// chosen, so that the two ends never meet.
 __global__ void k_noalloc_heavy(NoAllocScratch *s, const uint32_t *offsets, const uint32_t *active,
                                 int64_t n_active, float *P, int n_bins) {
   for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n_active;
@@ -73,11 +77,9 @@ __global__ void k_noalloc_heavy(NoAllocScratch *s, const uint32_t *offsets, cons
     const uint32_t k = active[a];
     const uint32_t cnt = offsets[k + 1] - offsets[k];
     if (cnt >= (uint32_t)kNoAllocHeavyMin) {
-      // from the list's front, or (big pixels) from its back: it holds all of
-      // a call whose offsets stay within its events
-      const bool big = cnt >= (uint32_t)kBigPixel;
-      const uint32_t pos = atomicAdd(&s->qctl[big ? 1 : 0], 1u);
-      if ((int64_t)pos < kNoAllocMaxHeavy) {
+      if (atomicAdd(&s->qctl[5], 1u) < (uint32_t)kNoAllocMaxHeavy) {
+        const bool big = cnt >= (uint32_t)kBigPixel;
+        const uint32_t pos = atomicAdd(&s->qctl[big ? 1 : 0], 1u);
         s->heavy[big ? kNoAllocMaxHeavy - 1 - pos : pos] = (uint32_t)a;
       } else {
         atomicOr(&s->flags, DDHF_FLAG_CAPACITY);
