@@ -731,19 +731,22 @@ __device__ __noinline__ static void comb_records_any_d(const float *Pw, int N, i
 // scale = 64 BPL / (3 mean)): bucket g = floor(v scale) clamped to the last one,
 // as the float 2^23 + g, from one multiply-add to 2^23 rounded down, so no
 // float-to-integer conversion runs on the special-function pipe. Monotone in v
-// >= 0, so the bins of a bucket range are a range of full ranks. Any input (a
-// negative value, NaN) still gives an index below 1024 (BPL 24) or 4096 (96) to
-// hist_add: inside the scratch (the window maxima follow).
+// >= 0, so the bins of a bucket range are a range of full ranks. NaN (0 times an
+// infinite scale) gives the last bucket; a negative value, which no power is,
+// gives less than 2^23.
 template <int BPL>
 __device__ __forceinline__ float bucket_y(float v, float scale) {
   return fminf(__fmaf_rd(v, scale, 0x1p23f), 0x1p23f + (float)(32 * BPL - 1));
 }
 
 // Add one to bucket y in the histogram at shared address hist_sa (one counter
-// per bucket).
+// per bucket). A y below 2^23 counts in the word behind the histogram (the window
+// maximum of bin 0, which no candidate reads): the counts then fall short of N,
+// which comb_locate reports.
 template <int BPL>
 __device__ __forceinline__ void hist_add(uint32_t hist_sa, float y) {
-  const uint32_t a = hist_sa + ((__float_as_uint(y) & (BPL == 24 ? 1023u : 4095u)) << 2);
+  const uint32_t g = min(__float_as_uint(y) - 0x4B000000u, 32u * BPL);
+  const uint32_t a = hist_sa + (g << 2);
   asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(a) : "memory");
 }
 
