@@ -940,7 +940,8 @@ __device__ __forceinline__ void comb_nw_all(const float *rec, float *nws, const 
       }
     }
   }
-  // N(w) >= 0 (or -1): its bits order as a signed integer
+  // N(w) >= 0 (or -1): its bits order as a signed integer, once -0 is +0
+  maxnw = __fadd_rn(maxnw, 0.f);
   const int top = __reduce_max_sync(0xffffffffu, __float_as_int(maxnw));
   maxi = __reduce_min_sync(0xffffffffu, __float_as_int(maxnw) == top ? maxi : 0x7fffffff);
   maxnw = __int_as_float(top);

@@ -53,3 +53,15 @@ def test_negative_values_touch_no_other_row(N, M, d, h_min):
     c.close()
     for w, g, r in zip(want, got, again):
         assert torch.equal(w, g) and torch.equal(w, r)
+
+
+@pytest.mark.parametrize("N", [100, 750, 2000])
+def test_rows_of_negative_zero_score_as_zero(N):
+    c = _context(N, 4, 3, 4, tau_comb=0.0)
+    Z = torch.zeros((N_PX, N), device="cuda")
+    zero, neg = c.comb_score(Z), c.comb_score(-Z)
+    c.stats()
+    c.close()
+    assert (zero["f0_bin"] == 3).all() and (zero["mask"][:N_PX] == 1).all()
+    for k in ("log_sf", "snr", "f0_bin", "mask"):
+        assert torch.equal(zero[k], neg[k]), k
