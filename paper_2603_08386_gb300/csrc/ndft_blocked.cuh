@@ -69,52 +69,13 @@
 
 #include "comb.cuh"
 #include "ddhf_internal.cuh"
+#include "ndft_const.cuh"
 
 namespace ddhf {
 namespace blocked {
 
 constexpr int kGenChunk = 32;  // events staged per warp, one lane each
 constexpr int kGroup = 8;      // events per tensor-core step
-constexpr int kMaxPasses = 64; // 512 rows of 32 bins, at least 8 per pass
-
-// Phases as fractions of a turn in units of 2^-64.
-struct NdftConst {
-  uint64_t f_u;                // da / D (one bin)
-  uint64_t f_k8;               // 8.5 da / D (column k = 8)
-  uint64_t f_v;                // 32 da / D (one row)
-  uint64_t f_row[kMaxPasses];  // a_c(b0 + 4 MT) / D: the middle row of each pass
-  int32_t dc_first, dc_step;   // bins with a_j = 0 mod D: dc_first + i dc_step (-1: none)
-};
-
-inline uint64_t turn_fraction(unsigned __int128 num, uint64_t den) {
-  const uint64_t r = (uint64_t)(num % den);
-  return (uint64_t)((((unsigned __int128)r << 64) + den / 2) / den);
-}
-
-inline NdftConst make_ndft_const(const GridConst &g, int mt) {
-  NdftConst n{};
-  const unsigned __int128 a0 = g.a0, da = g.da;
-  n.f_u = turn_fraction(da, g.denom);
-  n.f_k8 = turn_fraction(17 * da, 2 * g.denom);
-  n.f_v = turn_fraction(32 * da, g.denom);
-  for (int i = 0; i < kMaxPasses; ++i)
-    n.f_row[i] = turn_fraction(2 * a0 + (64 * (unsigned)(8 * mt * i + 4 * mt) + 31) * da,
-                               2 * g.denom);
-  n.dc_first = -1;
-  uint64_t x = g.da, y = g.denom;
-  while (y) {
-    const uint64_t r = x % y;
-    x = y;
-    y = r;
-  }
-  n.dc_step = (int32_t)std::min<uint64_t>(g.denom / x, (uint64_t)1 << 30);
-  for (int j = 0; j < g.N && j < n.dc_step; ++j)
-    if ((g.a0 + (uint64_t)j * g.da) % g.denom == 0) {
-      n.dc_first = j;
-      break;
-    }
-  return n;
-}
 
 __device__ __forceinline__ void raise_flag(uint32_t *flags, uint32_t f) { atomicOr(flags, f); }
 
@@ -931,7 +892,7 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
   A.cursors = c->qctl + 5;
   A.N = c->gconst.N;
   A.nbr = c->gconst.nbr;
-  A.nd = make_ndft_const(c->gconst, MT);
+  A.nd = make_ndft_const(c->gconst.a0, c->gconst.da, c->gconst.denom, A.N, A.nbr, MT);
   A.cc = c->comb;
   A.P = P;
   A.ld = ld > 0 ? ld : c->gconst.N;

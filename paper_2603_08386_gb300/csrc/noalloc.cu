@@ -169,7 +169,7 @@ ddhf_status launch_noalloc(NoAllocScratch *sp, const GridConst &g, float *P, int
   A.cursors = &sp->qctl[2];
   A.N = g.N;
   A.nbr = g.nbr;
-  A.nd = blocked::make_ndft_const(g, MT);
+  A.nd = blocked::make_ndft_const(g.a0, g.da, g.denom, g.N, g.nbr, MT);
   A.cc = CombConst{};
   A.P = P;
   A.ld = g.N;
