@@ -175,7 +175,9 @@ typedef struct {
  *              split over them; two with 2 warps per block) or, from 2048
  *              events, by a cluster of four thread blocks. Pixels of 256
  *              events or more that are not listed go to such a team all the
- *              same; the others to one warp each;
+ *              same; the others to one warp each. So 256 to 2048 are one
+ *              setting; below 256 more pixels go to teams, above 2048 the
+ *              clusters start at heavy_min;
  *  warps_per_block  warps per thread block (2, 4 or 8);
  *  blocks_per_sm    resident blocks per SM used to size the persistent grid
  *                   (0 = as many as fit);

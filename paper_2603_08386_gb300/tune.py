@@ -20,15 +20,17 @@ import torch
 
 from . import ddhf
 
+# Every heavy_min from 256 to 2048 is the same launch (pixels of 256 events are
+# listed, of 2048 go to a cluster), so 1024 stands for them all.
 DEFAULT_CANDIDATES = [
     dict(heavy_min=hm, warps_per_block=wpb, blocks_per_sm=0, rows_per_lane=r, fuse=1, overlap=0)
-    for hm in (512, 1024, 4096)
+    for hm in (1024, 4096)
     for wpb in (4, 8)
     for r in (0, 4)
 ] + [
     dict(heavy_min=hm, warps_per_block=wpb, blocks_per_sm=0, rows_per_lane=r, fuse=0, overlap=ov,
          hybrid_min=hy)
-    for hm in (128, 256, 1024, 4096)
+    for hm in (128, 1024, 4096)
     for wpb in (4, 8)
     for r in (0, 4)
     for ov in (0, 1)
