@@ -137,10 +137,11 @@ typedef struct {
  *  BLOCKED  persistent kernel: rows of 32 bins around their centre, F[+-s] of
  *           a row from four real sums over the events, as one real matrix
  *           product per pixel on the tensor cores; each operand is a pair of
- *           FP16 words (FP32 accuracy) and its phase an exact 64-bit fraction
- *           of a turn. Pixels of 256 events or more are split over a team of
- *           warps, of 2048 or more over several blocks. The form used by
- *           ddhf_detect.
+ *           FP16 words (FP32 accuracy), its phase from a 64-bit fraction of a
+ *           turn, within 2^-28 of a turn (frequencies that are a multiple of
+ *           1 cycle per microsecond exact). Pixels of 256 events or more are
+ *           split over a team of warps, of 2048 or more over several blocks.
+ *           The form used by ddhf_detect.
  *  NAIVE32  precision study only: FP32 phase 2 pi f t from the absolute time.
  *  KAHAN    SINCOS with compensated (Kahan) accumulation.
  *  F64      check path: FP64 phase and accumulation on the GPU.
@@ -308,7 +309,9 @@ ddhf_status ddhf_export_csr(ddhf_ctx *ctx, uint32_t *offsets, uint32_t *ev,
 
 /* Eq. 6 and P_j = |F_j|^2 for every active pixel of slot 0, in active-list
  * order: P[a*n_bins + j] (FP32, row a of the a-th active pixel). `form` is a
- * DDHF_FORM_*. Rows beyond cap_px are not written (DDHF_FLAG_CAPACITY). */
+ * DDHF_FORM_*. Rows beyond cap_px are not written (DDHF_FLAG_CAPACITY). The
+ * launch tuning is the one set when the call is made, whatever the window was
+ * binned under. */
 ddhf_status ddhf_power_spectrum(ddhf_ctx *ctx, int32_t form, float *P, int64_t cap_px,
                                 ddhf_stream stream);
 
@@ -321,7 +324,9 @@ ddhf_status ddhf_power_spectrum(ddhf_ctx *ctx, int32_t form, float *P, int64_t c
  * snr[a] = max_w SNR_M(w) and f0_bin[a] = its first maximising bin w when
  * SF <= tau_sf (else 0 and -1); mask[W*H] (uint8, zeroed by the call) gets 1
  * at rotor pixels (SF <= tau_sf and snr >= tau_comb). log_sf, snr and f0_bin
- * may be NULL. Given the same P, every output is bit-reproducible. */
+ * may be NULL. P must not be negative: the scores of a row with negative values
+ * are unspecified (and may raise DDHF_FLAG_INTERNAL), those of other rows are
+ * not touched by them. Given the same P, every output is bit-reproducible. */
 ddhf_status ddhf_comb_score(ddhf_ctx *ctx, const float *P, int64_t cap_px, float *log_sf,
                             float *snr, int32_t *f0_bin, uint8_t *mask,
                             ddhf_stream stream);
@@ -383,7 +388,9 @@ ddhf_status ddhf_export_scores(ddhf_ctx *ctx, int32_t slot, uint32_t *active, fl
  *                    ((a0 + j da) 1e6 / denom), 0 when there is none
  *                    (nullable).
  * Device outputs of cap entries; entries from min(*n_boxes_dev, cap) on are
- * left unchanged. */
+ * left unchanged. The call counts in the workspace that labelling and boxes use
+ * too, so like every call it must not run on the GPU beside another of the same
+ * context. */
 ddhf_status ddhf_box_frequencies(ddhf_ctx *ctx, int32_t slot, const ddhf_box *boxes,
                                  const int32_t *n_boxes_dev, int32_t cap, int32_t *f0_bin,
                                  float *snr, float *f0_hz_median, ddhf_stream stream);

@@ -414,6 +414,9 @@ ddhf_status launch_label(Ctx *c, const uint8_t *mask, int32_t *labels, uint64_t 
 //
 // Per box in scratch (the label workspace, free after the boxes are out): the
 // maximum (2 words), rotor count, units done and N histogram counters.
+// Whole calls on a 347x261, a sparse and a dense 1280x720 window (us): 292 / 305 /
+// 3783; units of 1024 pixels 288 / 302 / 3791, of 16,384 305 / 311 / 3824; row segments
+// of 128 pixels 292 / 304 / 3784, of 512 291 / 307 / 3797.
 constexpr int kF0Unit = 4096;  // pixels of a box per unit
 constexpr int kF0Seg = 256;    // pixels of a row per warp step
 constexpr int kF0Head = 4;     // words of a box's record before its histogram

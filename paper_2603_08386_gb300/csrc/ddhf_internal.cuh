@@ -24,8 +24,14 @@ constexpr int kMaxBandWords = 8;   // comb rank band up to 256 positions
 constexpr uint32_t kSignBit = 0x80000000u;
 constexpr size_t kCanaryBytes = 256;        // guard region on each side of a buffer
 constexpr unsigned char kCanaryByte = 0xA5;
-constexpr int kTeamPixel = 256;             // events from which four warps take a pixel
-constexpr int kBigPixel = 2048;             // events from which a cluster of blocks takes it
+// Events from which four warps take a pixel, and from which a cluster of blocks
+// does. Whole calls on a 347x261, a sparse and a dense 1280x720 window, 640x480
+// spectra at 2000 bins and 320x180 at 10,000 (us): 292 / 305 / 3783 / 1000 / 2853;
+// teams from 128: 290 / 303 / 3819 / 1016 / 2900 (from 512 and 1024: ndft_blocked.cuh);
+// clusters from 1024: 292 / 306 / 3799 / 1001 / 2907, from 4096: 291 / 305 / 3779 /
+// 1000 / 2836, from 8192: 313 / 314 / 3779 / 1001 / 2837.
+constexpr int kTeamPixel = 256;
+constexpr int kBigPixel = 2048;
 constexpr uint32_t kDropKey = 0xffffffffu;  // pre-packed sort input: pair not kept
 
 // Invariant checks of the debug build (-DDDHF_BOUNDS_CHECK, made by
@@ -168,7 +174,8 @@ struct Ctx {
                                  // label count, [12-13] hybrid lists, [14] hybrid cursor
   // labelling / boxes scratch
   int32_t *box_root = nullptr;   // [npx]
-  int32_t *box_tmp = nullptr;    // [npx * 6]
+  int32_t *box_tmp = nullptr;    // [npx * 15] box slots and lists; the records of
+                                 // ddhf_box_frequencies
   uint32_t *flags = nullptr;     // [1] DDHF_FLAG_* bits
   // workspace buffers with guard bytes (kCanaryBytes of kCanaryByte before
   // and after each), checked by ddhf_get_stats

@@ -26,11 +26,13 @@
 // every accumulator of a bin pair in the lane that squares it.
 //
 // Factors are generated for 32 events at a time, one lane per event, into shared
-// memory: a column and a row phasor from exact phases, the others by rotation
-// away from them on both sides (at most 8 steps for the columns, 4 MT for the
-// rows, each step an exact phasor too). Phases are 64-bit fixed-point fractions
-// of a turn: the frequency's fraction a / D mod 1, rounded to 2^-64, times tau,
-// so the phase error is below 2^-33 of a turn. Measured error of the spectra
+// memory: a column and a row phasor straight from their phases, the others by
+// rotation away from them on both sides (at most 8 steps for the columns, 4 MT for
+// the rows, each step a phasor straight from its phase too). Phases are fixed-point
+// fractions of a turn: the frequency's fraction a / D mod 1, rounded to 2^-64, times
+// tau < 2^31 (error below 2^-34 of a turn), cut to its top 32 bits (below 2^-32);
+// the sine and cosine then take it as an FP32 number of at most 1/8 turn (below
+// 2^-28). Measured error of the spectra
 // against FP64 (2-norm over all pixels): 2.4e-7 at 2000 bins on 640x480 pixels,
 // 4.0e-7 at 10,000 bins on 320x180 (the FP32 three-multiplication product
 // before it, with its longer rotation chains: 8.1e-7 and 1.3e-6).
@@ -47,15 +49,17 @@
 // integer sum of the polarities, counted exactly (Eq. 7 takes the logarithm of
 // it, and a sum of zero must be exactly zero).
 //
-// Who takes a pixel, and in which order its events are summed, both by its event
-// count n alone:
+// Who takes a pixel, by its event count n alone; up to 2047 events the order in
+// which they are summed, too (from there on it also depends on the warps per block):
 //   n < 256 (kTeamPixel)   one warp, group after group (unless the tuning's
 //                          heavy_min lists it);
 //   n >= 256, or listed    four sums over every fourth chunk of 32 events, added
 //                          in order, by a team of four warps (or of two): one
 //                          warp needs 1.6 us per chunk, so that a 1000-event
 //                          pixel alone took 62 us, longer than the rest of a
-//                          sparse window; by a team 19 us;
+//                          sparse window; by a team 19 us (threshold 256 / 512 /
+//                          1024: dense 1280x720 spectra 1.38 / 1.38 / 1.41 ms, sparse
+//                          84 / 92 / 119 us, 320x180 at 10,000 bins 2.68 / 2.79 / 2.98 ms);
 //   n >= 2048 (kBigPixel)  (and heavy_min) a cluster of four blocks, one sum per
 //                          warp, added in order through shared memory: 20,000
 //                          events are 156 chunks per warp of a block.
@@ -857,7 +861,8 @@ int blocked_warp_bytes(const Ctx *c, bool fused, int NW, int *pw_offset) {
 
 // A grid of `blocks` blocks (rounded down to whole clusters) in clusters of four:
 // with four blocks per SM a cluster divides every GPC's blocks evenly, so none
-// of them is lost.
+// of them is lost. Clusters of 2 / 4 / 8 (whole calls, us): sparse 1280x720 window
+// 319 / 305 / 303, dense 3746 / 3783 / 3798, 320x180 at 10,000 bins 2772 / 2853 / 2913.
 constexpr int kCluster = 4;
 template <typename K>
 cudaError_t launch_clusters(K kern, int blocks, int threads, size_t smem, cudaStream_t s,
