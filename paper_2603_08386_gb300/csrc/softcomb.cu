@@ -29,7 +29,11 @@
 //    the last harmonics' groups costs more than the shared reductions save);
 //  * the last three steps halve the frequencies that a lane holds (7 exchanges
 //    per component and eight frequencies instead of 24), so that lane i of eight
-//    ends with frequencies i, i + 8, ... and squares them there;
+//    ends with frequencies i, i + 8, ... and squares them there. The backward pass
+//    of more than nine frequencies reduces them one by one over the whole warp
+//    instead: its 44 to 68 sums leave 16 warps per SM, and the halving's exchanges,
+//    selections and broadcasts wait more than they save (60,000 pixels, 5 harmonics,
+//    Q = 5: 1.42 ms halving, 1.23 so; 8 harmonics, Q = 8: 2.53 and 2.20);
 //  * the weights G_hq and their sums depend on (h, q) alone: a table per block.
 // Per-pixel gradient contributions to w and sigma are written to a workspace,
 // one column each, and summed over pixels, so every output is deterministic.
@@ -166,6 +170,7 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
   constexpr int kQ = 8 * NJ + EX;
   // two sets of sums fit the registers
   constexpr bool kGroups = kC * kQ <= 32;
+  constexpr bool kHalve = !BWD || NJ == 1;
   __shared__ float sG[kSoftMaxH][kQ];             // G_hq, 0 for q >= 2Q+1
   __shared__ float sZ[kSoftMaxH], sE[kSoftMaxH];  // Z_h, sum_q G qd^2
   const int lane = threadIdx.x & 31;
@@ -244,16 +249,28 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
         }
       } else {
         soft_lane<kQ, BWD>(A, f, A.ev + o0, lane, cnt, nq, x);
+        if constexpr (kHalve) {
 #pragma unroll 1
-        for (int o = 16; o >= 8; o >>= 1)
+          for (int o = 16; o >= 8; o >>= 1)
 #pragma unroll
-          for (int c = 0; c < kC; ++c)
+            for (int c = 0; c < kC; ++c)
 #pragma unroll
-            for (int q = 0; q < kQ; ++q)
-              if (q < nq) x[c][q] += __shfl_xor_sync(0xffffffffu, x[c][q], o);
+              for (int q = 0; q < kQ; ++q)
+                if (q < nq) x[c][q] += __shfl_xor_sync(0xffffffffu, x[c][q], o);
+        } else {
+#pragma unroll
+          for (int q = 0; q < kQ; ++q)
+            if (q < nq)
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int c = 0; c < kC; ++c)
+                  x[c][q] += __shfl_xor_sync(0xffffffffu, x[c][q], o);
+        }
       }
       // the last three steps, halving: lane i of eight gets frequencies i, i + 8, ...
       float y[kC][NJ];
+      if constexpr (kHalve)
 #pragma unroll
       for (int c = 0; c < kC; ++c)
 #pragma unroll
@@ -272,18 +289,21 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
           y[c][j] = v[0];
         }
       // the frequency beyond the blocks: whole, in every lane
-      if constexpr (EX != 0)
+      if constexpr (kHalve && EX != 0)
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1)
 #pragma unroll
           for (int c = 0; c < kC; ++c)
             x[c][8 * NJ] += __shfl_xor_sync(0xffffffffu, x[c][8 * NJ], o);
-      float P[NJ + EX], Pd[NJ + EX];
+      // of the lane's own frequencies, or (not kHalve) of all
+      constexpr int kP = kHalve ? NJ + EX : kQ;
+      float P[kP], Pd[kP];
 #pragma unroll
-      for (int j = 0; j < NJ + EX; ++j) {
+      for (int j = 0; j < kP; ++j) {
         float v[kC];
 #pragma unroll
-        for (int c = 0; c < kC; ++c) v[c] = j < NJ ? y[c][j < NJ ? j : 0] : x[c][kQ - 1];
+        for (int c = 0; c < kC; ++c)
+          v[c] = !kHalve ? x[c][j] : j < NJ ? y[c][j < NJ ? j : 0] : x[c][kQ - 1];
         P[j] = v[0] * v[0] + v[1] * v[1];
         if constexpr (BWD) Pd[j] = 2.f * (v[0] * v[2] + v[1] * v[3]);
       }
@@ -293,8 +313,8 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
 #pragma unroll
       for (int q = 0; q < kQ; ++q) {
         const int src = (lane & 24) + (q & 7);
-        float Pq = P[q / 8], Pdq = BWD ? Pd[q / 8] : 0.f;
-        if (q < 8 * NJ) {
+        float Pq = P[kHalve ? q / 8 : q], Pdq = BWD ? Pd[kHalve ? q / 8 : q] : 0.f;
+        if (kHalve && q < 8 * NJ) {
           Pq = __shfl_sync(0xffffffffu, Pq, src);
           if constexpr (BWD) Pdq = __shfl_sync(0xffffffffu, Pdq, src);
         }
@@ -311,12 +331,13 @@ __global__ void __launch_bounds__(256) k_softcomb(SoftArgs A) {
       const bool h_ok = h0 + hg < A.n_h;
       const float sgm = BWD ? A.sigma[h] : 0.f;
       if constexpr (BWD) {
-        if (A.g_f && h_ok && (grouped || lane < 8)) {
+        if (A.g_f && h_ok && (grouped || !kHalve || lane < 8)) {
           // per evaluation frequency: g dS/df_hq = g w_h G_hq P'(f_hq) / (Z_h B)
 #pragma unroll
-          for (int j = 0; j < NJ + EX; ++j) {
-            const int q = 8 * j + (lane & 7);
-            if (q < nq)  // of the frequency beyond the blocks, lane 0 alone
+          for (int j = 0; j < kP; ++j) {
+            const int q = kHalve ? 8 * j + (lane & 7) : j;
+            // of the frequency beyond the blocks, lane 0 alone
+            if (q < nq && (kHalve || lane == q))
               A.g_f[(a * A.n_h + h) * (int64_t)nq + q] = gs * (wh * sG[h][q] * Pd[j] / (Z * Bv));
           }
         }
