@@ -285,6 +285,7 @@ ddhf_status run_detect(Ctx *c, const ddhf_window *wins, int nw, ddhf_box *boxes,
                        int32_t *n_boxes_dev, uint8_t *masks_out, cudaStream_t s,
                        const cudaEvent_t *ready = nullptr) {
   if (c->timing) DDHF_CUDA_TRY(c, record_stage(c, 0, s));
+  DDHF_CUDA_TRY(c, note_list(c, false, s));
   const bool fused = c->tuning.fuse != 0 || !c->pbuf;
   if (fused) {
     DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, 2 * sizeof(uint32_t), s));  // heavy and big counts
@@ -368,6 +369,7 @@ ddhf_status run_detect(Ctx *c, const ddhf_window *wins, int nw, ddhf_box *boxes,
       if (we) DDHF_CUDA_TRY(c, record_event(we[4], s));
     }
   }
+  DDHF_CUDA_TRY(c, note_list(c, nw == 1, s));
   c->timing_fused = fused;
   c->timing_windows = nw;
   if (c->timing) DDHF_CUDA_TRY(c, record_stage(c, 2, s));
@@ -671,8 +673,10 @@ ddhf_status ddhf_bin_events(ddhf_ctx *h, const int16_t *x, const int16_t *y, con
   DDHF_TRY(check_window(c, x, y, t_us, p, n, window_us));
   cudaStream_t s = (cudaStream_t)stream;
   c->last_stream = s;
+  DDHF_CUDA_TRY(c, note_list(c, false, s));
   DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, 2 * sizeof(uint32_t), s));
   DDHF_TRY(bin_into(c, 0, x, y, t_us, p, n, t0_us, window_us, s));
+  DDHF_CUDA_TRY(c, note_list(c, true, s));
   c->binned = true;
   return DDHF_OK;
 }
@@ -822,12 +826,14 @@ ddhf_status ddhf_detect_batch(ddhf_ctx *h, const ddhf_window *wins, int32_t n_wi
     }
     cudaStream_t cap_s = nullptr;
     DDHF_CUDA_TRY(c, cudaStreamCreateWithFlags(&cap_s, cudaStreamNonBlocking));
+    const bool in_graph = c->list_in_graph;  // this graph is replayed by this call alone
     // kernels read tuning-dependent attributes at launch; set them before capture
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cap_s, cudaStreamCaptureModeThreadLocal);
     ddhf_status st = DDHF_OK;
     if (e == cudaSuccess) st = run_detect(c, wins, n_windows, boxes, cap, n_boxes_dev, masks_out, cap_s);
     cudaError_t e2 = cudaStreamEndCapture(cap_s, &graph);
+    c->list_in_graph = in_graph;
     cudaStreamDestroy(cap_s);
     if (e != cudaSuccess || e2 != cudaSuccess || st != DDHF_OK) {
       if (graph) cudaGraphDestroy(graph);
@@ -859,6 +865,7 @@ ddhf_status ddhf_detect_batch(ddhf_ctx *h, const ddhf_window *wins, int32_t n_wi
     }
     c->graph_key = key;
   }
+  DDHF_CUDA_TRY(c, note_list(c, n_windows == 1, s));
   DDHF_CUDA_TRY(c, cudaGraphLaunch(c->graph_exec, s));
   c->binned = true;
   return DDHF_OK;

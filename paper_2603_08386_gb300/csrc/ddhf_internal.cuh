@@ -195,6 +195,10 @@ struct Ctx {
   GridConst gconst{};
   cudaStream_t last_stream = nullptr;
   bool binned = false;
+  // the work list: slot 0's pixels alone under these thresholds (0: something else)
+  int listed_min = 0, listed_big = 0;
+  bool list_in_graph = false;    // calls that fill it were captured by the caller: any
+                                 // replay may change it without the host knowing
   std::string last_error;
   // stage timing (tracing)
   bool timing = false;
@@ -340,6 +344,18 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 // both from the same tuning.
 inline int list_min(const ddhf_tuning &t) { return t.heavy_min < kTeamPixel ? t.heavy_min : kTeamPixel; }
 inline int big_min(const ddhf_tuning &t) { return t.heavy_min > kBigPixel ? t.heavy_min : kBigPixel; }
+
+// Records that work enqueued on `s` fills the work list, with slot 0's pixels alone
+// under the current tuning when slot0 is set, else with something else.
+inline cudaError_t note_list(Ctx *c, bool slot0, cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(s, &cs);
+  if (e != cudaSuccess) return e;
+  if (cs != cudaStreamCaptureStatusNone) c->list_in_graph = true;
+  c->listed_min = slot0 ? list_min(c->tuning) : 0;
+  c->listed_big = slot0 ? big_min(c->tuning) : 0;
+  return cudaSuccess;
+}
 
 // ---------------------------------------------------------- launch entry points
 // bin.cu

@@ -23,18 +23,29 @@ __global__ void k_list_pixels(const SlotView *view, int list_min, int big_min, u
 }
 
 // The work list of slot 0's pixels under the tuning of this call, and the kernel's
-// cursors zeroed (with them word 4, which every soft comb zeroes itself). The list
-// that the binning left may be of another tuning (ddhf_set_tuning came since), of
-// the last window of a batch, or of all its windows. A listed pixel has at least 32
-// events, so the list's capacity (a 32nd of the events) holds both ends. 5 us on
-// 307,200 pixels (latency: three dependent loads), beside the 0.99 ms of the whole
-// call at 2000 bins.
+// cursors zeroed. The list that the last binning or detection left may be of another
+// tuning (ddhf_set_tuning came since), of the last window of a batch, or of all its
+// windows: it is filled again unless the host knows that it is the right one. A
+// captured call always fills it (what precedes its replays is not known here). A
+// listed pixel has at least 32 events, so the list's capacity (a 32nd of the events)
+// holds both ends. Filling costs 5 us on 307,200 pixels, 11 in calls so small that
+// their launches bound them.
 ddhf_status list_slot0(Ctx *c, cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  DDHF_CUDA_TRY(c, cudaStreamIsCapturing(s, &cs));
+  if (cs == cudaStreamCaptureStatusNone && !c->list_in_graph &&
+      c->listed_min == list_min(c->tuning) && c->listed_big == big_min(c->tuning)) {
+    DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl + 5, 0, 3 * sizeof(uint32_t), s));
+    return DDHF_OK;
+  }
+  c->listed_min = c->listed_big = 0;
+  // with word 4, which every soft comb zeroes itself
   DDHF_CUDA_TRY(c, cudaMemsetAsync(c->qctl, 0, 8 * sizeof(uint32_t), s));
   const int blocks = (int)std::min<int64_t>(ceil_div(c->npx, 256), (int64_t)c->num_sms * 8);
   k_list_pixels<<<blocks, 256, 0, s>>>(c->d_views, list_min(c->tuning), big_min(c->tuning),
                                        c->work, c->heavy_cap, c->qctl, c->flags);
   DDHF_CUDA_TRY(c, cudaGetLastError());
+  DDHF_CUDA_TRY(c, note_list(c, true, s));
   return DDHF_OK;
 }
 
