@@ -816,26 +816,40 @@ __global__ void __launch_bounds__(256, 2) k_blocked(const __grid_constant__ Bloc
 }
 
 // Pixels of kTeamPixel events and fewer than A.heavy_min, which no list holds
-// (the no-allocation entry point, whose fixed scratch lists the larger ones), by
-// teams of four warps, one team per block: each takes 32 active pixels at a time.
+// (the no-allocation entry point with many active pixels, whose fixed scratch lists
+// the larger ones), by teams of four warps, one team per block. A block takes runs of
+// up to 32 active pixels, short enough that every block gets sixteen of them, and
+// looks at four runs at once. n_heavy[6] says whether there is any such pixel.
 template <int MT>
 __global__ void __launch_bounds__(128, 4) k_team_scan(const __grid_constant__ BlockedArgs A) {
   extern __shared__ float4 smem4[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned char *stage = reinterpret_cast<unsigned char *>(smem4) + warp * A.warp_bytes;
   __shared__ int s_neg[4];
+  if (A.n_heavy[6] == 0) return;
   const SlotView &v = A.views[0];
-  const int64_t n_act = (int64_t)v.counters[2];
-  for (int64_t a0 = 32 * (int64_t)blockIdx.x; a0 < n_act; a0 += 32 * (int64_t)gridDim.x) {
-    int cnt = 0;
-    if (a0 + lane < n_act) {
-      const uint32_t key = v.active[a0 + lane];
-      cnt = (int)(v.offsets[key + 1] - v.offsets[key]);
+  const int64_t n_act = (int64_t)v.counters[2], blocks = gridDim.x;
+  const int64_t run = max((int64_t)1, min((int64_t)32, n_act / (16 * blocks)));
+  for (int64_t r0 = blockIdx.x; r0 * run < n_act; r0 += 4 * blocks) {
+    uint32_t m[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t a = (r0 + u * blocks) * run + lane;
+      int cnt = 0;
+      if (lane < run && a < n_act) {
+        const uint32_t key = v.active[a];
+        cnt = (int)(v.offsets[key + 1] - v.offsets[key]);
+      }
+      m[u] = __ballot_sync(0xffffffffu, cnt >= kTeamPixel && cnt < A.heavy_min);
     }
-    for (uint32_t m = __ballot_sync(0xffffffffu, cnt >= kTeamPixel && cnt < A.heavy_min); m;
-         m &= m - 1)  // the same pixels in every warp of the block
-      for (int ps = 0; ps < (A.nbr + 8 * MT - 1) / (8 * MT); ++ps)
-        team_item<MT, 1, false, 4>(A, (uint64_t)(a0 + __ffs(m) - 1), ps, stage, warp, 0, s_neg);
+#pragma unroll 1
+    for (int u = 0; u < 4; ++u)
+      for (uint32_t k = u == 0 ? m[0] : u == 1 ? m[1] : u == 2 ? m[2] : m[3]; k; k &= k - 1) {
+        // the same pixels in every warp of the block
+        const int64_t px = (r0 + u * blocks) * run + __ffs(k) - 1;
+        for (int ps = 0; ps < (A.nbr + 8 * MT - 1) / (8 * MT); ++ps)
+          team_item<MT, 1, false, 4>(A, (uint64_t)px, ps, stage, warp, 0, s_neg);
+      }
   }
 }
 
