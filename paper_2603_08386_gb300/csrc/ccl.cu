@@ -410,9 +410,13 @@ ddhf_status launch_label(Ctx *c, const uint8_t *mask, int32_t *labels, uint64_t 
 // (SNR bits, -active index) to the box's maximum and adds its rotor pixels'
 // dominant bins to the box's histogram, one counter per bin, and the box's
 // last unit reads the lower median off the histogram. The order of these
-// integer atomics does not matter.
+// integer atomics does not matter. A box of one unit, as most are, needs no
+// record: its block counts in shared memory and reads the median off there, or
+// (grids of more than kF0SharedBins bins) selects it by two passes over 7 bits of
+// the bin (3,000 boxes of 5x5 pixels at 750 bins: 103 us with a record each, 40 so;
+// at 5000 bins 137 and 53).
 //
-// Per box in scratch (the label workspace, free after the boxes are out): the
+// A record in scratch (the label workspace, free after the boxes are out): the
 // maximum (2 words), rotor count, units done and N histogram counters.
 // Whole calls on a 347x261, a sparse and a dense 1280x720 window (us): 292 / 305 /
 // 3783; units of 1024 pixels 288 / 302 / 3791, of 16,384 305 / 311 / 3824; row segments
@@ -431,10 +435,12 @@ struct BoxF0Args {
   const ddhf_box *boxes;
   const int32_t *n_boxes;
   int32_t cap, W, H, N;
-  int32_t room;          // boxes whose records fit the scratch
-  uint32_t *first_unit;  // [min(cap, room) + 1] first unit of each box
+  int32_t room;          // boxes that the scratch has entries for
+  uint32_t *first_unit;  // [room + 1] first unit of each box
+  uint32_t *rec_of;      // [room] the record of a box of several units
   int32_t rec_words;     // words of a record: kF0Head + N, rounded up to even
-  uint32_t *rec;         // [room] records
+  int32_t rec_room;      // records
+  uint32_t *rec;         // [rec_room][rec_words]
   int32_t *f0_out;
   float *snr_out, *med_hz;
   int64_t g_a0, g_da, g_denom;
@@ -539,116 +545,196 @@ __device__ __forceinline__ void box_f0_reduce(unsigned long long &best, uint32_t
   }
 }
 
-// First units of the boxes and cleared records (block 0 the former); boxes
-// beyond the scratch's room (many boxes on a small sensor with a large grid)
-// are done here, one block each: strongest pixel, then the lower median by a
-// two-digit radix selection (bins below 2^14, 7 bits per pass).
-__global__ void __launch_bounds__(256) k_box_f0_plan(BoxF0Args A) {
-  __shared__ unsigned long long red[8];
-  __shared__ uint32_t cnt[8];
-  __shared__ uint32_t hist[128];
-  __shared__ uint32_t sel[2];
-  const int nb = min(*A.n_boxes, A.cap), nr = min(nb, A.room);
+// The lower median (the bin of rank (total - 1) / 2) of a histogram, get(k) being
+// counter k, by the whole block; cnt: eight words.
+template <typename G>
+__device__ __forceinline__ void box_f0_median(const BoxF0Args &A, int b, uint32_t total,
+                                              uint32_t *cnt, G get) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t words = (int64_t)max(nr, 0) * A.rec_words;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < words;
-       i += (int64_t)gridDim.x * blockDim.x)
-    A.rec[i] = 0;
-  if (blockIdx.x == 0) {
-    uint32_t base = 0;
-    for (int b0 = 0; b0 < nr; b0 += 256) {
-      const int b = b0 + threadIdx.x;
-      uint32_t inc = b < nr ? box_units(box_rows(A, A.boxes[b])) : 0u;
-      const uint32_t own = inc;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t u = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += u;
-      }
-      if (lane == 31) cnt[warp] = inc;
-      __syncthreads();
-      uint32_t pre = base;
-      for (int w = 0; w < 8; ++w) {
-        if (w < warp) pre += cnt[w];
-        base += cnt[w];
-      }
-      if (b < nr) A.first_unit[b] = pre + inc - own;
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) A.first_unit[max(nr, 0)] = base;
+  const uint32_t rank = total > 0 ? (total - 1) / 2 : 0;
+  const int per = (A.N + 255) / 256, k0 = (int)threadIdx.x * per, k1 = min(A.N, k0 + per);
+  uint32_t own = 0;
+  for (int k = k0; k < k1; ++k) own += get(k);
+  uint32_t inc = own;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
   }
-  const int64_t n_act = (int64_t)A.counters[2];
-  for (int b = A.room + (int)blockIdx.x; b < nb; b += (int)gridDim.x) {
-    const BoxRows r = box_rows(A, A.boxes[b]);
-    unsigned long long best = 0ull;
-    uint32_t n = 0;
-    box_visit(A, r, n_act, warp, 8, r.items, [&](int64_t i) {
-      const unsigned long long v =
-          ((unsigned long long)__float_as_uint(A.snr[i]) << 32) | (0xffffffffu - (uint32_t)i);
-      best = v > best ? v : best;
-      ++n;
-    });
-    box_f0_reduce(best, n, red, cnt);
-    if (threadIdx.x == 0) box_f0_best(A, b, best);
-    if (!A.med_hz) continue;
-    uint32_t rank = n > 0 ? (n - 1) / 2 : 0, prefix = 0;
-    for (int pass = 0; pass < 2 && n > 0; ++pass) {
-      const int shift = pass == 0 ? 7 : 0;
-      for (int k = threadIdx.x; k < 128; k += blockDim.x) hist[k] = 0;
-      __syncthreads();
-      box_visit(A, r, n_act, warp, 8, r.items, [&](int64_t i) {
-        const uint32_t v = (uint32_t)A.f0[i];
-        if (!ddhf_check(v < (1u << 14), A.flags)) return;
-        if (pass == 1 && (v >> 7) != prefix) return;
-        atomicAdd(&hist[(v >> shift) & 127u], 1u);
-      });
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        int dsel = 127;
-        for (int k = 0; k < 128; ++k) {
-          if (rank < run + hist[k]) {
-            dsel = k;
-            break;
-          }
-          run += hist[k];
-        }
-        sel[0] = (uint32_t)dsel;
-        sel[1] = rank - run;
+  __syncthreads();  // cnt has been read
+  if (lane == 31) cnt[warp] = inc;
+  __syncthreads();
+  uint32_t pre = inc - own;
+  for (int w = 0; w < warp; ++w) pre += cnt[w];
+  if (total == 0) {
+    if (threadIdx.x == 0) A.med_hz[b] = 0.f;
+  } else if (rank >= pre && rank < pre + own) {
+    uint32_t run = pre;
+    for (int k = k0; k < k1; ++k) {
+      const uint32_t h = get(k);
+      if (rank < run + h) {
+        A.med_hz[b] = box_f0_hz(A, (uint32_t)k);
+        break;
       }
-      __syncthreads();
-      prefix = pass == 0 ? sel[0] : (prefix << 7) | sel[0];
-      rank = sel[1];
-      __syncthreads();
+      run += h;
     }
-    if (threadIdx.x == 0) A.med_hz[b] = n > 0 ? box_f0_hz(A, prefix) : 0.f;
   }
 }
 
-// The units of the boxes that have a record, and each box's results by its
-// last unit. SHARED: a unit counts its bins in shared memory first.
+struct BoxF0Shared {
+  unsigned long long red[8];
+  uint32_t cnt[8];
+  uint32_t hist[128];
+  uint32_t sel[2];
+};
+
+// A whole box by one block. SHARED: sh_hist holds a counter per bin; else the
+// lower median by a two-digit radix selection (bins below 2^14, 7 bits per pass).
+template <bool SHARED>
+__device__ __forceinline__ void box_f0_one(const BoxF0Args &A, int b, int64_t n_act,
+                                           BoxF0Shared &sh, uint32_t *sh_hist) {
+  const int warp = threadIdx.x >> 5;
+  const BoxRows r = box_rows(A, A.boxes[b]);
+  const bool want_med = A.med_hz != nullptr;
+  if (SHARED && want_med) {
+    for (int k = threadIdx.x; k < A.N; k += blockDim.x) sh_hist[k] = 0;
+    __syncthreads();
+  }
+  unsigned long long best = 0ull;
+  uint32_t n = 0;
+  box_visit(A, r, n_act, warp, 8, r.items, [&](int64_t i) {
+    const unsigned long long v =
+        ((unsigned long long)__float_as_uint(A.snr[i]) << 32) | (0xffffffffu - (uint32_t)i);
+    best = v > best ? v : best;
+    ++n;
+    if (SHARED && want_med)
+      atomicAdd(&sh_hist[min((uint32_t)A.f0[i], (uint32_t)A.N - 1)], 1u);  // always below N
+  });
+  box_f0_reduce(best, n, sh.red, sh.cnt);  // its barriers also end the shared counting
+  if (threadIdx.x == 0) box_f0_best(A, b, best);
+  if (!want_med) return;
+  if (SHARED) {
+    box_f0_median(A, b, n, sh.cnt, [&](int k) { return sh_hist[k]; });
+    __syncthreads();
+    return;
+  }
+  uint32_t rank = n > 0 ? (n - 1) / 2 : 0, prefix = 0;
+  for (int pass = 0; pass < 2 && n > 0; ++pass) {
+    const int shift = pass == 0 ? 7 : 0;
+    for (int k = threadIdx.x; k < 128; k += blockDim.x) sh.hist[k] = 0;
+    __syncthreads();
+    box_visit(A, r, n_act, warp, 8, r.items, [&](int64_t i) {
+      const uint32_t v = (uint32_t)A.f0[i];
+      if (!ddhf_check(v < (1u << 14), A.flags)) return;
+      if (pass == 1 && (v >> 7) != prefix) return;
+      atomicAdd(&sh.hist[(v >> shift) & 127u], 1u);
+    });
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t run = 0;
+      int dsel = 127;
+      for (int k = 0; k < 128; ++k) {
+        if (rank < run + sh.hist[k]) {
+          dsel = k;
+          break;
+        }
+        run += sh.hist[k];
+      }
+      sh.sel[0] = (uint32_t)dsel;
+      sh.sel[1] = rank - run;
+    }
+    __syncthreads();
+    prefix = pass == 0 ? sh.sel[0] : (prefix << 7) | sh.sel[0];
+    rank = sh.sel[1];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) A.med_hz[b] = n > 0 ? box_f0_hz(A, prefix) : 0.f;
+}
+
+// Exclusive sum of v over the block's 256 threads, plus base, which then takes the
+// total too.
+__device__ __forceinline__ uint32_t box_scan(uint32_t v, uint32_t &base, uint32_t *cnt) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t inc = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t u = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += u;
+  }
+  __syncthreads();  // cnt has been read
+  if (lane == 31) cnt[warp] = inc;
+  __syncthreads();
+  uint32_t pre = base;
+  for (int w = 0; w < 8; ++w) {
+    if (w < warp) pre += cnt[w];
+    base += cnt[w];
+  }
+  return pre + inc - v;
+}
+
+// Units and records of the boxes, and the records cleared. A box of several units
+// takes the next record; without one (boxes of more than kF0Unit pixels beyond
+// rec_room) it is one unit. Every block does the sums, to know how many records to
+// clear, and block 0 writes them. Boxes beyond the room (a caller's capacity of
+// more than 15 npx / 4 boxes) are done here, one block each.
+__global__ void __launch_bounds__(256) k_box_f0_plan(BoxF0Args A) {
+  __shared__ BoxF0Shared sh;
+  const int nb = min(*A.n_boxes, A.cap), nr = min(nb, A.room);
+  uint32_t recs = 0, units = 0;
+  for (int b0 = 0; b0 < nr; b0 += 256) {
+    const int b = b0 + (int)threadIdx.x;
+    const uint32_t own = b < nr ? box_units(box_rows(A, A.boxes[b])) : 0u;
+    const uint32_t r = box_scan(own > 1 ? 1u : 0u, recs, sh.cnt);
+    const bool has_rec = own > 1 && r < (uint32_t)A.rec_room;
+    const uint32_t u = box_scan(has_rec ? own : min(own, 1u), units, sh.cnt);
+    if (blockIdx.x == 0 && b < nr) {
+      A.first_unit[b] = u;
+      A.rec_of[b] = r;
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) A.first_unit[max(nr, 0)] = units;
+  const int64_t words = (int64_t)min(recs, (uint32_t)A.rec_room) * A.rec_words;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < words;
+       i += (int64_t)gridDim.x * blockDim.x)
+    A.rec[i] = 0;
+  const int64_t n_act = (int64_t)A.counters[2];
+  for (int b = A.room + (int)blockIdx.x; b < nb; b += (int)gridDim.x)
+    box_f0_one<false>(A, b, n_act, sh, nullptr);
+}
+
+// The box of unit u: the last b with first[b] <= u (first ascends, first[nb] > u),
+// by the whole warp.
+__device__ __forceinline__ int unit_box(const uint32_t *first, int nb, uint32_t u) {
+  int lo = 0, hi = nb;
+  while (hi - lo > 1) {
+    const int step = (hi - lo + 31) / 32, i = lo + ((int)(threadIdx.x & 31) + 1) * step;
+    const int below = __popc(__ballot_sync(0xffffffffu, i < hi && first[i] <= u));
+    lo += below * step;
+    hi = min(hi, lo + step);
+  }
+  return lo;
+}
+
+// The units of the boxes, and the results of a box of several by its last unit.
+// SHARED: a unit counts its bins in shared memory first.
 template <bool SHARED>
 __global__ void __launch_bounds__(256) k_box_f0_units(BoxF0Args A) {
   extern __shared__ uint32_t sh_hist[];
-  __shared__ unsigned long long red[8];
-  __shared__ uint32_t cnt[8];
+  __shared__ BoxF0Shared sh;
   __shared__ uint32_t s_last;
   const int nr = min(min(*A.n_boxes, A.cap), A.room);
   if (nr <= 0) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int warp = threadIdx.x >> 5;
   const int64_t n_act = (int64_t)A.counters[2];
   const uint32_t n_units = A.first_unit[nr];
   const bool want_med = A.med_hz != nullptr;
   for (uint32_t u = blockIdx.x; u < n_units; u += gridDim.x) {
-    int lo = 0, hi = nr - 1;  // the box of unit u
-    while (lo < hi) {
-      const int m = (lo + hi + 1) >> 1;
-      if (A.first_unit[m] <= u) lo = m;
-      else hi = m - 1;
-    }
-    const int b = lo;
+    const int b = n_units == (uint32_t)nr ? (int)u : unit_box(A.first_unit, nr, u);
     const uint32_t part = u - A.first_unit[b], parts = A.first_unit[b + 1] - A.first_unit[b];
+    if (parts == 1) {
+      box_f0_one<SHARED>(A, b, n_act, sh, sh_hist);
+      continue;
+    }
     const BoxRows r = box_rows(A, A.boxes[b]);
-    uint32_t *rec = A.rec + (int64_t)b * A.rec_words, *hist = rec + kF0Head;
+    uint32_t *rec = A.rec + (int64_t)A.rec_of[b] * A.rec_words, *hist = rec + kF0Head;
     if (SHARED && want_med) {
       for (int k = threadIdx.x; k < A.N; k += blockDim.x) sh_hist[k] = 0;
       __syncthreads();
@@ -666,7 +752,7 @@ __global__ void __launch_bounds__(256) k_box_f0_units(BoxF0Args A) {
       const uint32_t f = min((uint32_t)A.f0[i], (uint32_t)A.N - 1);  // always below N
       atomicAdd(SHARED ? &sh_hist[f] : &hist[f], 1u);
     });
-    box_f0_reduce(best, n, red, cnt);  // its barriers also end the shared counting
+    box_f0_reduce(best, n, sh.red, sh.cnt);  // its barriers also end the shared counting
     if (SHARED && want_med)
       for (int k = threadIdx.x; k < A.N; k += blockDim.x)
         if (sh_hist[k]) atomicAdd(&hist[k], sh_hist[k]);
@@ -683,34 +769,7 @@ __global__ void __launch_bounds__(256) k_box_f0_units(BoxF0Args A) {
     if (threadIdx.x == 0)
       box_f0_best(A, b, __ldcg(reinterpret_cast<const unsigned long long *>(rec)));
     if (!want_med) continue;
-    const uint32_t total = __ldcg(&rec[2]);
-    // lower median: the bin that holds rank (total - 1) / 2
-    const uint32_t rank = total > 0 ? (total - 1) / 2 : 0;
-    const int per = (A.N + 255) / 256, k0 = (int)threadIdx.x * per, k1 = min(A.N, k0 + per);
-    uint32_t own = 0;
-    for (int k = k0; k < k1; ++k) own += __ldcg(&hist[k]);
-    uint32_t inc = own;
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += v;
-    }
-    if (lane == 31) cnt[warp] = inc;
-    __syncthreads();
-    uint32_t pre = inc - own;
-    for (int w = 0; w < warp; ++w) pre += cnt[w];
-    if (total == 0) {
-      if (threadIdx.x == 0) A.med_hz[b] = 0.f;
-    } else if (rank >= pre && rank < pre + own) {
-      uint32_t run = pre;
-      for (int k = k0; k < k1; ++k) {
-        const uint32_t h = __ldcg(&hist[k]);
-        if (rank < run + h) {
-          A.med_hz[b] = box_f0_hz(A, (uint32_t)k);
-          break;
-        }
-        run += h;
-      }
-    }
+    box_f0_median(A, b, __ldcg(&rec[2]), sh.cnt, [&](int k) { return __ldcg(&hist[k]); });
     __syncthreads();
   }
 }
@@ -732,13 +791,16 @@ ddhf_status launch_box_f0(Ctx *c, int slot, const ddhf_box *boxes, const int32_t
   A.W = c->W;
   A.H = c->H;
   A.N = c->grid.n_bins;
-  // records (8-byte aligned, of an even number of words) in the box workspace
-  // of 15 npx words, after a word of first_unit each and one more
+  // in the box workspace of 15 npx words: two words of a box each and one more, in
+  // up to half of it, then the records (8-byte aligned, of an even number of words)
   A.rec_words = (kF0Head + A.N + 1) & ~1;
   const int64_t words = 15 * c->npx;
-  A.room = (int32_t)std::min<int64_t>(cap, std::max<int64_t>(0, (words - 4) / (A.rec_words + 1)));
+  A.room = (int32_t)std::min<int64_t>(cap, words / 4);
   A.first_unit = reinterpret_cast<uint32_t *>(c->box_tmp);
-  A.rec = A.first_unit + ((A.room + 1 + 1) & ~1);
+  A.rec_of = A.first_unit + A.room + 1;
+  const int64_t head = (2 * (int64_t)A.room + 2) & ~(int64_t)1;
+  A.rec = A.first_unit + head;
+  A.rec_room = (int32_t)std::max<int64_t>(0, (words - head) / A.rec_words);
   A.f0_out = f0_out;
   A.snr_out = snr_out;
   A.med_hz = med_hz;
@@ -749,7 +811,7 @@ ddhf_status launch_box_f0(Ctx *c, int slot, const ddhf_box *boxes, const int32_t
   A.flags = c->flags;
   k_box_f0_plan<<<c->num_sms, 256, 0, s>>>(A);
   if (A.room > 0) {
-    const unsigned units = (unsigned)c->num_sms * 4;
+    const unsigned units = (unsigned)c->num_sms * 6;
     if (A.N <= kF0SharedBins)
       k_box_f0_units<true><<<units, 256, A.N * sizeof(uint32_t), s>>>(A);
     else
