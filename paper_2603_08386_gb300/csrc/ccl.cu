@@ -69,7 +69,7 @@ __global__ void k_label_init(const uint8_t *__restrict__ mask, int32_t *__restri
     const int64_t i = i0 + lane;
     const bool fg = i < npx && mask[i] != 0;
     const uint32_t b = __ballot_sync(0xffffffffu, fg);
-    const uint32_t row = __ballot_sync(0xffffffffu, i % W == 0);
+    const uint32_t row = __ballot_sync(0xffffffffu, (uint32_t)i % (uint32_t)W == 0);
     const uint32_t start = b & (~(b << 1) | row);  // lane 0 of a run that came in starts too
     const uint32_t mine = start & (0xffffffffu >> (31 - lane));
     if (i < npx) lab[i] = fg ? (int32_t)(i - lane + (31 - __clz(mine))) : -1;
@@ -85,7 +85,7 @@ __global__ void k_label_union(const uint8_t *__restrict__ mask, int32_t *lab, in
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < npx;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (!mask[i]) continue;
-    const int x = (int)(i % W), y = (int)(i / W);
+    const int y = (int)((uint32_t)i / (uint32_t)W), x = (int)i - y * W;
     // Only the unions that no other pixel's own unions imply. A run that crosses
     // a segment is joined at the segment's first pixel. Two rows' overlapping
     // runs are joined where their overlap begins: a pixel whose left neighbour
