@@ -60,9 +60,10 @@
 //                          sparse window; by a team 19 us (threshold 256 / 512 /
 //                          1024: dense 1280x720 spectra 1.38 / 1.38 / 1.41 ms, sparse
 //                          84 / 92 / 119 us, 320x180 at 10,000 bins 2.68 / 2.79 / 2.98 ms);
-//   n >= 2048 (kBigPixel)  (and heavy_min) a cluster of four blocks, one sum per
-//                          warp, added in order through shared memory: 20,000
-//                          events are 156 chunks per warp of a block.
+//   n >= 2048 (kBigPixel)  (and heavy_min) a cluster of four blocks (fused, of two or
+//                          one in more rounds too), one sum per warp, added in
+//                          order through shared memory: 20,000 events are 156
+//                          chunks per warp of a block.
 // Big pixels first, then the listed ones, then the light. When several passes
 // cover the bins, each (pixel, pass) of the first two is an item of its own.
 #pragma once
@@ -80,6 +81,7 @@ namespace blocked {
 
 constexpr int kGenChunk = 32;  // events staged per warp, one lane each
 constexpr int kGroup = 8;      // events per tensor-core step
+constexpr int kShares = 4;     // shares of a big pixel: the blocks of its cluster
 
 __device__ __forceinline__ void raise_flag(uint32_t *flags, uint32_t f) { atomicOr(flags, f); }
 
@@ -651,10 +653,10 @@ __device__ __noinline__ void team_item(const BlockedArgs &A, uint64_t it, int pa
   }
 }
 
-// A big pixel by the blocks of a cluster: warp w of block r takes chunks r nw +
-// w, + blocks nw, ...; warp 0 of each block adds its warps' sums, that of the
+// A pass of a big pixel by the four blocks of a cluster: warp w of block r takes
+// chunks r nw + w, + 4 nw, ...; warp 0 of each block adds its warps' sums, that of the
 // first block the other blocks'.
-template <int MT, int NW, bool FUSED>
+template <int MT>
 __device__ __noinline__ void cluster_item(const BlockedArgs &A, uint64_t it, int pass,
                                           unsigned char *stage, int *s_neg) {
   namespace cg = cooperative_groups;
@@ -662,8 +664,7 @@ __device__ __noinline__ void cluster_item(const BlockedArgs &A, uint64_t it, int
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int blocks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   HeavyPixel h;
-  if (!heavy_pixel<FUSED>(A, it, h)) return;  // the same answer in every block
-  float *Pw = reinterpret_cast<float *>(stage + A.pw_offset);
+  if (!heavy_pixel<false>(A, it, h)) return;  // the same answer in every block
   float *part = reinterpret_cast<float *>(stage);
   const int p0 = pass >= 0 ? pass : 0;
   const int p1 = pass >= 0 ? pass + 1 : (A.nbr + 8 * MT - 1) / (8 * MT);
@@ -703,11 +704,86 @@ __device__ __noinline__ void cluster_item(const BlockedArgs &A, uint64_t it, int
         }
         neg += *cluster.map_shared_rank(s_neg, r);
       }
-      heavy_store<MT, FUSED>(A, acc, h.a, ps, h.cnt - 2 * neg, Pw);
+      heavy_store<MT, false>(A, acc, h.a, ps, h.cnt - 2 * neg, nullptr);
     }
     cluster.sync();  // the other blocks' sums have been read
   }
-  if (FUSED && warp == 0 && rank == 0) {
+}
+
+// All passes of a big pixel and its scores (FUSED), by a cluster of four blocks, or of
+// two or one in rounds: four shares, added in the order of cluster_item. A form of
+// its own: the sum kept between rounds spills (in cluster_item 320x180 pixels of
+// 10,000 bins 2.84 -> 2.93 ms).
+template <int MT, int NW>
+__device__ __noinline__ void cluster_rounds(const BlockedArgs &A, uint64_t it,
+                                            unsigned char *stage, int *s_neg) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int blocks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  HeavyPixel h;
+  if (!heavy_pixel<true>(A, it, h)) return;  // the same answer in every block
+  float *Pw = reinterpret_cast<float *>(stage + A.pw_offset);
+  float *part = reinterpret_cast<float *>(stage);
+  for (int ps = 0; ps < (A.nbr + 8 * MT - 1) / (8 * MT); ++ps) {
+    float tot[16 * MT];  // the sum so far
+    int neg_tot = 0;
+#pragma unroll 1
+    for (int r0 = 0; r0 < kShares; r0 += blocks) {
+      Acc<MT> acc;
+      acc.zero();
+      int neg = accumulate<MT>(h.v->ev + h.o0, h.cnt, (r0 + rank) * nw + warp, kShares * nw, A.nd,
+                               A.nd.f_row[ps], stage, acc);
+#pragma unroll
+      for (int i = 0; i < 16 * MT; ++i) part[i * 32 + lane] = acc.x[i / 16][(i / 4) % 4][i % 4];
+      if (lane == 0) s_neg[warp] = neg;
+      __syncthreads();
+      if (warp == 0) {
+        for (int w2 = 1; w2 < nw; ++w2) {
+          const float *op = reinterpret_cast<const float *>(stage + w2 * A.warp_bytes);
+#pragma unroll
+          for (int i = 0; i < 16 * MT; ++i) {
+            float &x = acc.x[i / 16][(i / 4) % 4][i % 4];
+            x = __fadd_rn(x, op[i * 32 + lane]);
+          }
+          neg += s_neg[w2];
+        }
+        if (rank != 0) {
+#pragma unroll
+          for (int i = 0; i < 16 * MT; ++i)
+            part[i * 32 + lane] = acc.x[i / 16][(i / 4) % 4][i % 4];
+          if (lane == 0) s_neg[0] = neg;
+        }
+      }
+      cluster.sync();
+      if (warp == 0 && rank == 0) {
+        neg_tot += neg;
+        if (r0 > 0)
+#pragma unroll
+          for (int i = 0; i < 16 * MT; ++i) {
+            float &x = acc.x[i / 16][(i / 4) % 4][i % 4];
+            x = __fadd_rn(tot[i], x);
+          }
+        for (int r = 1; r < blocks; ++r) {
+          const float *op = cluster.map_shared_rank(part, r);
+#pragma unroll
+          for (int i = 0; i < 16 * MT; ++i) {
+            float &x = acc.x[i / 16][(i / 4) % 4][i % 4];
+            x = __fadd_rn(x, op[i * 32 + lane]);
+          }
+          neg_tot += *cluster.map_shared_rank(s_neg, r);
+        }
+        if (r0 + blocks < kShares) {
+#pragma unroll
+          for (int i = 0; i < 16 * MT; ++i) tot[i] = acc.x[i / 16][(i / 4) % 4][i % 4];
+        } else {
+          heavy_store<MT, true>(A, acc, h.a, ps, h.cnt - 2 * neg_tot, Pw);
+        }
+      }
+      cluster.sync();  // the other blocks' sums have been read
+    }
+  }
+  if (warp == 0 && rank == 0) {
     CombOut o = comb_warp<NW>(Pw, A.cc, stage);
     store_scores<NW>(A, *h.v, h.a, h.key, o);
   }
@@ -747,8 +823,9 @@ __device__ __noinline__ void listed_pixels(const BlockedArgs &A, unsigned char *
       const uint32_t item = *cluster.map_shared_rank(&s_item[0], 0);
       cluster.sync();
       if (item / per_px >= n_big) break;
-      cluster_item<MT, NW, FUSED>(A, A.heavy[A.heavy_cap - 1 - item / per_px],
-                                  FUSED ? -1 : (int)(item % per_px), stage, s_neg);
+      const uint64_t it = A.heavy[A.heavy_cap - 1 - item / per_px];
+      if constexpr (FUSED) cluster_rounds<MT, NW>(A, it, stage, s_neg);
+      else cluster_item<MT>(A, it, (int)(item % per_px), stage, s_neg);
     }
   }
   if (blockDim.x >= 128) team_loop<MT, NW, FUSED, 4>(A, per_px, stage, s_item, s_neg);
@@ -873,22 +950,28 @@ int blocked_warp_bytes(const Ctx *c, bool fused, int NW, int *pw_offset) {
   return scratch + spectrum_rows<MT>((int)c->gconst.nbr) * 32 * 4;
 }
 
-// A grid of `blocks` blocks (rounded down to whole clusters) in clusters of four:
-// with four blocks per SM a cluster divides every GPC's blocks evenly, so none
-// of them is lost. Clusters of 2 / 4 / 8 (whole calls, us): sparse 1280x720 window
-// 319 / 305 / 303, dense 3746 / 3783 / 3798, 320x180 at 10,000 bins 2772 / 2853 / 2913.
-constexpr int kCluster = 4;
+// Blocks per cluster of a fused grid with `bps` blocks per SM (an unfused one has
+// clusters of four). A GPC that its clusters do not fill leaves slots idle for the
+// whole launch: with four blocks per SM clusters of four divide every GPC's blocks
+// evenly, with the two that the fused kernel's scratch often leaves those of two, where
+// four cost 3 to 5 % (640 bins, comb of 35 bins, 76,800 pixels: whole detection 4.80 ms,
+// by two 4.55). Clusters of 2 / 4 / 8 of the unfused kernel (whole calls, us): sparse
+// 1280x720 window 319 / 305 / 303, dense 3746 / 3783 / 3798, 320x180 at 10,000 bins
+// 2772 / 2853 / 2913.
+inline int fused_cluster(int bps) { return bps % 4 == 0 ? 4 : bps > 1 ? 2 : 1; }
+
+// A grid of `blocks` blocks (rounded down to whole clusters).
 template <typename K>
-cudaError_t launch_clusters(K kern, int blocks, int threads, size_t smem, cudaStream_t s,
-                            const BlockedArgs &A) {
+cudaError_t launch_clusters(K kern, int blocks, int cluster, int threads, size_t smem,
+                            cudaStream_t s, const BlockedArgs &A) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)std::max(kCluster, blocks / kCluster * kCluster));
+  cfg.gridDim = dim3((unsigned)std::max(cluster, blocks / cluster * cluster));
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = kCluster;
+  at.val.clusterDim.x = (unsigned)cluster;
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
@@ -934,7 +1017,8 @@ ddhf_status launch_blocked_t(Ctx *c, int n_slots, float *P, int64_t cap_px, cuda
     return DDHF_ERR_UNSUPPORTED;
   }
   int bps = c->tuning.blocks_per_sm > 0 ? std::min(occ, c->tuning.blocks_per_sm) : occ;
-  DDHF_CUDA_TRY(c, launch_clusters(kern, c->num_sms * bps, wpb * 32, smem, s, A));
+  DDHF_CUDA_TRY(c, launch_clusters(kern, c->num_sms * bps, FUSED ? fused_cluster(bps) : kShares,
+                                   wpb * 32, smem, s, A));
   return DDHF_OK;
 }
 

@@ -196,7 +196,8 @@ ddhf_status launch_noalloc(NoAllocScratch *sp, const GridConst &g, float *P, int
           cudaSuccess ||
       occ < 1)
     return DDHF_ERR_CUDA;
-  if (blocked::launch_clusters(kern, num_sms * occ, kNoAllocWarps * 32, smem, s, A) != cudaSuccess)
+  if (blocked::launch_clusters(kern, num_sms * occ, blocked::kShares, kNoAllocWarps * 32, smem, s,
+                               A) != cudaSuccess)
     return DDHF_ERR_CUDA;
   if (list_min <= kTeamPixel) return DDHF_OK;
   auto scan = blocked::k_team_scan<MT>;
